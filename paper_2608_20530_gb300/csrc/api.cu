@@ -201,25 +201,47 @@ GemmArgs gemm(const void* A, lilicorr_dtype_t a_dt, int lda, const void* W, lili
   return g;
 }
 
-// Few rows: split-N CUDA-core kernel. bf16 operands: tensor cores. Otherwise the
-// tiled fp32 CUDA-core kernel (the fp32 head keeps fp32 arithmetic throughout).
-// The persistent tensor-core kernel is the one run_gemm picks for g.
-bool takes_gemm_tc(const GemmArgs& g) {
-  return !(g.M <= 64 || (g.a_dt == LILICORR_F32 && g.M <= 1024)) && !gemm_small_supported(g) &&
-         gemm_tc_supported(g);
+// The kernel that a product of the network takes.
+enum class GemmPath { SKINNY, ROWS, SMALL, SPLIT, TC, SIMT };
+
+// bf16 operands: tensor cores (one tile of rows and short Kd: whole-K copies; few output
+// tiles: Kd split over a cluster; else the persistent kernel), but for the fewest rows, where
+// the split-N CUDA-core kernel spreads the weights over many CTAs. fp32 operands stay on
+// the CUDA cores (the fp32 head keeps fp32 arithmetic throughout).
+GemmPath gemm_path(const GemmArgs& g) {
+  const bool fold = g.c2 || g.ss_in;          // only these two kernels fold an RMSNorm
+  if (fold) return gemm_split_supported(g) ? GemmPath::SPLIT : GemmPath::TC;
+  // fp32 activations (the tensor-core kernels take bf16) at per-sequence row counts above
+  // 16: 16 x 32 output blocks with the rows staged (256 x 512 x 512: 54 -> ~5 us); few rows
+  // otherwise: the split-N kernel
+  if (g.a_dt == LILICORR_F32 && g.M > 16 && g.M <= 1024 && gemm_rows_supported(g))
+    return GemmPath::ROWS;
+  if (g.M > 4 && gemm_split_supported(g)) return GemmPath::SPLIT;
+  if (g.M <= 64 || (g.a_dt == LILICORR_F32 && g.M <= 1024)) return GemmPath::SKINNY;
+  if (gemm_small_supported(g)) return GemmPath::SMALL;
+  if (gemm_tc_supported(g)) return GemmPath::TC;
+  return GemmPath::SIMT;
+}
+
+// Whether g, with its folded RMSNorm, runs on a kernel that folds it.
+bool folds(const GemmArgs& g) {
+  return gemm_path(g) == GemmPath::SPLIT || (g.M > 64 && gemm_tc_supported(g));
+}
+
+// Sums of squares per row that a folded producer writes.
+int gemm_ss_slots(const GemmArgs& g) {
+  return gemm_path(g) == GemmPath::SPLIT ? gemm_split_ss_slots(g.N) : gemm_tc_ss_slots(g.M, g.N);
 }
 
 lilicorr_status_t run_gemm(const GemmArgs& g, cudaStream_t st) {
-  // a folded RMSNorm only exists in the persistent tensor-core kernel
-  if (g.c2 || g.ss_in) return takes_gemm_tc(g) ? launch_gemm_tc(g, st) : LILICORR_ERR_SHAPE;
-  // fp32 activations (the tensor-core kernels take bf16) at per-sequence row counts above
-  // 16: 16 x 32 output blocks with the rows staged (256 x 512 x 512: 54 -> ~5 us); few rows
-  // otherwise: the split-N kernel spreads the weights over many CTAs
-  if (g.a_dt == LILICORR_F32 && g.M > 16 && g.M <= 1024 && gemm_rows_supported(g))
-    return launch_gemm_rows(g, st);
-  if (g.M <= 64 || (g.a_dt == LILICORR_F32 && g.M <= 1024)) return launch_gemm_skinny(g, st);
-  if (gemm_small_supported(g)) return launch_gemm_small(g, st);
-  if (gemm_tc_supported(g)) return launch_gemm_tc(g, st);
+  switch (gemm_path(g)) {
+    case GemmPath::SKINNY: return launch_gemm_skinny(g, st);
+    case GemmPath::ROWS: return launch_gemm_rows(g, st);
+    case GemmPath::SMALL: return launch_gemm_small(g, st);
+    case GemmPath::SPLIT: return launch_gemm_split(g, st);
+    case GemmPath::TC: return gemm_tc_supported(g) ? launch_gemm_tc(g, st) : LILICORR_ERR_SHAPE;
+    case GemmPath::SIMT: break;
+  }
   return launch_gemm_simt(g, st);
 }
 
@@ -270,6 +292,7 @@ struct HeadCall {
              lilicorr_dtype_t c_dt, int ldc, int M, int Nn, int Kd) const {
     GemmArgs g = gemm(A, a_dt, lda, W, wdt, ldw, C, c_dt, ldc, M, Nn, Kd);
     g.status = status;
+    g.w_const = 1;
     return g;
   }
   // RMSNorm folded around a product (App. A's pre-norm x / rms(x) * gain): the product
@@ -278,8 +301,9 @@ struct HeadCall {
   void norm_out(GemmArgs& g, const float* gain) const {
     g.c2 = xn; g.ldc2 = D; g.c2_gain = gain; g.ss_out = ss;
   }
-  void norm_in(GemmArgs& g) const {
-    g.ss_in = ss; g.ss_slots = gemm_tc_ss_slots(N, D); g.ss_dim = D;
+  // `from`: the producer whose sums of squares the product reads
+  void norm_in(GemmArgs& g, const GemmArgs& from) const {
+    g.ss_in = ss; g.ss_slots = gemm_ss_slots(from); g.ss_dim = D;
   }
   // the final norm into the fusion layer's input [x; x*t] (App. A), both blocks at once:
   // xn [N, 2D] receives bf16(state * gain) and bf16(state * gain * t of the sequence)
@@ -327,31 +351,52 @@ lilicorr_status_t run_fusion_t(const HeadCall& c, cudaStream_t st) {
   g.bias = c.h->fuse_b;
   return run_gemm(g, st);
 }
-// Fork both chains from `st` onto the head's side streams; join_prologue makes `st` wait
-// for them. The joins are recorded even when a launch fails, so a capture stays balanced.
-lilicorr_status_t fork_prologue(const HeadCall& c, const void* hidden, const void* target,
-                                cudaStream_t st) {
-  lilicorr_head* hm = const_cast<lilicorr_head*>(c.h);
-  LL_CUDA_TRY(cudaEventRecord(hm->ev_fork, st));
-  LL_CUDA_TRY(cudaStreamWaitEvent(hm->side, hm->ev_fork, 0));
-  LL_CUDA_TRY(cudaStreamWaitEvent(hm->side2, hm->ev_fork, 0));
-  // side: drafter-state projection, then (once t exists) the fusion layer's t block;
-  // side2: the target state, then the anchor vector
-  lilicorr_status_t s1 = run_drafter_proj(c, hidden, hm->side);
-  lilicorr_status_t s2 = run_target(c, target, hm->side2);
-  LL_CUDA_TRY(cudaEventRecord(hm->ev_t, hm->side2));
-  LL_CUDA_TRY(cudaStreamWaitEvent(hm->side, hm->ev_t, 0));
-  if (s1 == LILICORR_OK) s1 = run_fusion_t(c, hm->side);
-  if (s2 == LILICORR_OK) s2 = run_anchor(c, hm->side2);
-  LL_CUDA_TRY(cudaEventRecord(hm->ev_join, hm->side));
-  LL_CUDA_TRY(cudaEventRecord(hm->ev_join2, hm->side2));
-  return s1 != LILICORR_OK ? s1 : s2;
-}
-lilicorr_status_t join_prologue(const lilicorr_head* h, cudaStream_t st) {
-  LL_CUDA_TRY(cudaStreamWaitEvent(st, h->ev_join, 0));
-  LL_CUDA_TRY(cudaStreamWaitEvent(st, h->ev_join2, 0));
-  return LILICORR_OK;
-}
+// Both chains, forked from the caller's stream onto the head's side streams: the
+// drafter-state projection, then (once t exists) the fusion layer's t block on one; the target
+// state, then the anchor vector, on the other. join_hidden / join_target make the caller's
+// stream wait for the projected drafter state / for everything. Both joins are recorded at
+// the latest by the destructor, also when a launch fails, so a capture stays balanced.
+struct Prologue {
+  lilicorr_head* h;
+  cudaStream_t st;
+  bool forked = false, hidden_joined = false, target_joined = false;
+  Prologue(const lilicorr_head* head, cudaStream_t stream)
+      : h(const_cast<lilicorr_head*>(head)), st(stream) {}
+  // hidden_here: nothing runs on `st` before the drafter state is needed, so its projection
+  // takes `st` itself instead of a side stream
+  lilicorr_status_t fork(const HeadCall& c, const void* hidden, const void* target,
+                         bool hidden_here) {
+    LL_CUDA_TRY(cudaEventRecord(h->ev_fork, st));
+    LL_CUDA_TRY(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
+    LL_CUDA_TRY(cudaStreamWaitEvent(h->side2, h->ev_fork, 0));
+    forked = true;
+    hidden_joined = hidden_here;
+    lilicorr_status_t s1 = run_drafter_proj(c, hidden, hidden_here ? st : h->side);
+    if (!hidden_here) LL_CUDA_TRY(cudaEventRecord(h->ev_hid, h->side));
+    lilicorr_status_t s2 = run_target(c, target, h->side2);
+    LL_CUDA_TRY(cudaEventRecord(h->ev_t, h->side2));
+    LL_CUDA_TRY(cudaStreamWaitEvent(h->side, h->ev_t, 0));
+    if (s1 == LILICORR_OK) s1 = run_fusion_t(c, h->side);
+    if (s2 == LILICORR_OK) s2 = run_anchor(c, h->side2);
+    return s1 != LILICORR_OK ? s1 : s2;
+  }
+  lilicorr_status_t join_hidden() {
+    if (!forked || hidden_joined) return LILICORR_OK;
+    hidden_joined = true;
+    LL_CUDA_TRY(cudaStreamWaitEvent(st, h->ev_hid, 0));
+    return LILICORR_OK;
+  }
+  lilicorr_status_t join_target() {
+    if (!forked || target_joined) return LILICORR_OK;
+    target_joined = true;
+    LL_CUDA_TRY(cudaEventRecord(h->ev_join, h->side));
+    LL_CUDA_TRY(cudaEventRecord(h->ev_join2, h->side2));
+    LL_CUDA_TRY(cudaStreamWaitEvent(st, h->ev_join, 0));
+    LL_CUDA_TRY(cudaStreamWaitEvent(st, h->ev_join2, 0));
+    return LILICORR_OK;
+  }
+  ~Prologue() { (void)join_target(); }         // waits for all of both side streams
+};
 
 // Whether every product around the chain's RMSNorms takes the persistent tensor-core
 // kernel (the only one that folds a norm): bf16 heads with more node rows than one tile.
@@ -373,18 +418,22 @@ bool fold_norms(const HeadCall& c) {
   }
   c.final_norm_out(p[5], h->final_norm);
   p[6].bias_rows = c.cb; p[6].rows_per_bias = c.LK; p[6].act = ACT_SILU;
-  for (int i : {1, 3, 6}) c.norm_in(p[i]);
+  c.norm_in(p[1], p[0]);                      // also after W_2 of the layer before (p[4])
+  c.norm_in(p[3], p[2]);
+  c.norm_in(p[6], p[5]);
   for (const GemmArgs& g : p)
-    if (!takes_gemm_tc(g)) return false;
+    if (!folds(g)) return false;
   return true;
 }
 
-// Candidate-dependent part, after the prologue: nodes, the Transformer, fusion and the
-// out/in heads. Writes oi = [W_o u + b_o | W_i u + b_i] (not yet normalised).
+// Candidate-dependent part: nodes, the Transformer, fusion and the out/in heads. Writes
+// oi = [W_o u + b_o | W_i u + b_i] (not yet normalised). `pro` holds the candidate-independent
+// part still running on the side streams; the chain waits for each half where it first reads
+// it, the network kernels (one launch) for both at their start.
 // With `tail`, the cluster kernel also forms the pair scores and walks; *tail_done says
 // whether it did (otherwise the caller launches the pair kernel).
-lilicorr_status_t run_body(const HeadCall& c, const int32_t* ids, const float* logp,
-                           cudaStream_t st, const ClusterTail* tail = nullptr,
+lilicorr_status_t run_body(const HeadCall& c, Prologue& pro, const int32_t* ids,
+                           const float* logp, cudaStream_t st, const ClusterTail* tail = nullptr,
                            bool* tail_done = nullptr) {
   if (tail_done) *tail_done = false;
   const lilicorr_head* h = c.h;
@@ -397,24 +446,28 @@ lilicorr_status_t run_body(const HeadCall& c, const int32_t* ids, const float* l
   const bool cluster = h->cluster_maps &&
                        (g_fused_enabled == 3 ||
                         (g_fused_enabled == 1 && c.B <= net_cluster_capacity()));
+  const bool fused =
+      h->net_maps && (g_fused_enabled == 2 || (g_fused_enabled == 1 && c.B >= FUSED_MIN_B));
+  // 129-256 nodes per sequence: two CTAs per sequence, one 128-node tile each
+  const bool pair = h->pair_maps && g_fused_enabled != 0;
+  LL_TRY(pro.join_hidden());
+  if (cluster || fused || pair) LL_TRY(pro.join_target());
   if (cluster) {
     if (tail_done) *tail_done = tail != nullptr;
     return launch_net_cluster(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st, tail);
   }
-  if (h->net_maps && (g_fused_enabled == 2 || (g_fused_enabled == 1 && c.B >= FUSED_MIN_B)))
-    return launch_net_fused(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st);
-  // 129-256 nodes per sequence: two CTAs per sequence, one 128-node tile each
-  if (h->pair_maps && g_fused_enabled != 0)
-    return launch_net_pair(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st);
+  if (fused) return launch_net_fused(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st);
+  if (pair) return launch_net_pair(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st);
   // nodes: x = fold[id] + hproj + slot + rank, then x += W_c2 c1 + b_c2
   LL_TRY(launch_node_build(h, c.B, ids, logp, c.hproj, c.c1, adt, c.x, c.status, st));
-  GemmArgs g = c.G(c.c1, adt, D, h->conf2_w, D, c.x, F32, D, N, D, D);
+  GemmArgs g = c.G(c.c1, adt, D, h->conf2_w, D, c.x, F32, D, N, D, D), from;
   g.bias = h->conf2_b;
   g.residual = c.x; g.ldr = D;
-  // the RMSNorms fold into the products around them when every one of those runs on the
-  // persistent tensor-core kernel; otherwise each is a kernel of its own
+  // the RMSNorms fold into the products around them when every one of those runs on a
+  // tensor-core kernel that folds them; otherwise each is a kernel of its own
   const bool fold = fold_norms(c);
   if (fold) c.norm_out(g, h->layer[0].an);
+  from = g;
   LL_TRY(run_gemm(g, st));
   // Transformer layers
   for (int i = 0; i < d.n_layers; ++i) {
@@ -422,7 +475,7 @@ lilicorr_status_t run_body(const HeadCall& c, const int32_t* ids, const float* l
     if (!fold) LL_TRY(launch_rmsnorm(c.x, N, D, l.an, c.xn, adt, st));
     g = c.G(c.xn, adt, D, l.wqkv, D, c.qkv, c.qkv_dt, 3 * D, N, 3 * D, D);
     g.bias = l.bqkv;
-    if (fold) c.norm_in(g);
+    if (fold) c.norm_in(g, from);
     LL_TRY(run_gemm(g, st));
     if (c.tc_attn && attention_umma_supported(d.L, d.K, D, d.n_heads) &&
         (g_attn_umma == 1 || (g_attn_umma == 2 && d.L * d.K == 256 && d.K % 8 == 0)))
@@ -437,21 +490,24 @@ lilicorr_status_t run_body(const HeadCall& c, const int32_t* ids, const float* l
     g.bias = l.bo;
     g.residual = c.x; g.ldr = D;
     if (fold) c.norm_out(g, l.fn);
+    from = g;
     LL_TRY(run_gemm(g, st));
     if (!fold) LL_TRY(launch_rmsnorm(c.x, N, D, l.fn, c.xn, adt, st));
     g = c.G(c.xn, adt, D, l.w1, D, c.hf, adt, F, N, F, D);
     g.bias = l.b1;
     g.act = ACT_SILU;
-    if (fold) c.norm_in(g);
+    if (fold) c.norm_in(g, from);
     LL_TRY(run_gemm(g, st));
     g = c.G(c.hf, adt, F, l.w2, F, c.x, F32, D, N, D, F);
     g.bias = l.b2;
     g.residual = c.x; g.ldr = D;
     // the last layer's output feeds the final norm: both blocks of the fusion input
+    if (i + 1 == d.n_layers) LL_TRY(pro.join_target());
     if (fold) {
       if (i + 1 < d.n_layers) c.norm_out(g, h->layer[i + 1].an);
       else c.final_norm_out(g, h->final_norm);
     }
+    from = g;
     LL_TRY(run_gemm(g, st));
   }
   // fusion u = SiLU(W_f [x; t; x*t] + b_f) with x the final-normed state (the t block is
@@ -461,7 +517,7 @@ lilicorr_status_t run_body(const HeadCall& c, const int32_t* ids, const float* l
   g.bias_rows = c.cb;
   g.rows_per_bias = c.LK;
   g.act = ACT_SILU;
-  if (fold) c.norm_in(g);
+  if (fold) c.norm_in(g, from);
   LL_TRY(run_gemm(g, st));
   // out and in heads in one product: oi = [W_o u + b_o | W_i u + b_i]
   g = c.G(c.u, adt, D, h->woi, D, c.oi, F32, 2 * d.d, N, 2 * d.d, D);
@@ -474,10 +530,10 @@ lilicorr_status_t run_head(const lilicorr_head* h, int B, const int32_t* ids, co
                            const void* hidden, const void* target, void* ws, const WsLayout& w,
                            cudaStream_t st) {
   const HeadCall c(h, B, ws, w);
-  const lilicorr_status_t sp = fork_prologue(c, hidden, target, st);
-  LL_TRY(join_prologue(h, st));
-  LL_TRY(sp);
-  return run_body(c, ids, logp, st);
+  Prologue pro(h, st);
+  LL_TRY(pro.fork(c, hidden, target, true));
+  LL_TRY(run_body(c, pro, ids, logp, st));
+  return pro.join_target();
 }
 
 }  // namespace
@@ -587,6 +643,7 @@ lilicorr_status_t lilicorr_head_create(const lilicorr_head_desc* desc, const voi
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->ev_join2) cudaEventDestroy(h->ev_join2);
     if (h->ev_t) cudaEventDestroy(h->ev_t);
+    if (h->ev_hid) cudaEventDestroy(h->ev_hid);
     free(h);
     return s;
   };
@@ -595,7 +652,8 @@ lilicorr_status_t lilicorr_head_create(const lilicorr_head_desc* desc, const voi
       cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_join2, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&h->ev_t, cudaEventDisableTiming) != cudaSuccess)
+      cudaEventCreateWithFlags(&h->ev_t, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_hid, cudaEventDisableTiming) != cudaSuccess)
     return fail(LILICORR_ERR_CUDA);
   if (cudaMalloc(&h->pool, pool_bytes) != cudaSuccess) return fail(LILICORR_ERR_CUDA);
   h->pool_bytes = pool_bytes;
@@ -660,6 +718,7 @@ lilicorr_status_t lilicorr_head_destroy(lilicorr_head* h) {
   if (h->ev_join) cudaEventDestroy(h->ev_join);
   if (h->ev_join2) cudaEventDestroy(h->ev_join2);
   if (h->ev_t) cudaEventDestroy(h->ev_t);
+  if (h->ev_hid) cudaEventDestroy(h->ev_hid);
   if (cur != h->device) cudaSetDevice(cur);
   free(h);
   return e == cudaSuccess ? LILICORR_OK : LILICORR_ERR_CUDA;
@@ -869,13 +928,11 @@ lilicorr_status_t lilicorr_select_block_walk(const lilicorr_head* head, int B, c
   float* logp = at<float>(ws, w.logp);
   // the candidate-independent projections run beside the top-K pass
   const HeadCall call(head, B, ws, w);
-  const lilicorr_status_t sp = fork_prologue(call, drafter_hidden, target_hidden, stream);
-  const lilicorr_status_t st = sp != LILICORR_OK ? sp
-      : launch_topk_lse(logits, d.dtype, R, d.V, d.K, ids, logp, at<float>(ws, w.lse),
-                        at<uint32_t>(ws, w.status), at<uint32_t>(ws, w.counters),
-                        at<void>(ws, w.partials), stream);
-  LL_TRY(join_prologue(head, stream));                      // always rejoin, even on error
-  LL_TRY(st);
+  Prologue pro(head, stream);
+  LL_TRY(pro.fork(call, drafter_hidden, target_hidden, false));
+  LL_TRY(launch_topk_lse(logits, d.dtype, R, d.V, d.K, ids, logp, at<float>(ws, w.lse),
+                         at<uint32_t>(ws, w.status), at<uint32_t>(ws, w.counters),
+                         at<void>(ws, w.partials), stream));
   ClusterTail tail;
   tail.anchor = at<float>(ws, w.anc);
   tail.A = at<float>(ws, w.A);
@@ -883,7 +940,7 @@ lilicorr_status_t lilicorr_select_block_walk(const lilicorr_head* head, int B, c
   tail.choice = at<int32_t>(ws, w.choice);
   tail.tokens = tokens;
   bool tail_done = false;
-  LL_TRY(run_body(call, ids, logp, stream, walk == LILICORR_WALK_GREEDY ? &tail : nullptr,
+  LL_TRY(run_body(call, pro, ids, logp, stream, walk == LILICORR_WALK_GREEDY ? &tail : nullptr,
                   &tail_done));
   if (tail_done) return LILICORR_OK;
   PairWalkArgs a;
@@ -935,6 +992,7 @@ lilicorr_status_t lilicorr_test_linear(const void* A, lilicorr_dtype_t a_dt, int
     case 3: return gemm_tc_supported(g) ? launch_gemm_tc(g, stream) : LILICORR_ERR_DTYPE;
     case 4: return gemm_small_supported(g) ? launch_gemm_small(g, stream) : LILICORR_ERR_SHAPE;
     case 5: return launch_gemm_rows(g, stream);
+    case 6: return gemm_split_supported(g) ? launch_gemm_split(g, stream) : LILICORR_ERR_SHAPE;
   }
   return LILICORR_ERR_ARG;
 }

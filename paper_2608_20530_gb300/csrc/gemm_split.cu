@@ -1,0 +1,350 @@
+// Tensor-core linear layer for few output tiles: C[M, N] = epilogue(A W^T), bf16 A and W, with
+// Kd split over a thread-block cluster.
+//
+// A head of width 1024 with one request multiplies 120 node rows by [1024 .. 3072, 1024 .. 2048]
+// weights: 16 to 48 tiles of 128 x 64, so a kernel with one CTA per tile leaves two thirds of
+// the SMs idle while the others stream Kd / 64 chunks one after the other. Here S = 1, 2, 4 or 8 CTAs, one cluster, share a tile:
+// each multiplies its part of Kd into its own tensor memory, parks the 128 x BN partial sums
+// in its shared memory, and after a cluster barrier every CTA adds up the S partials of the
+// rows r, r + S, r + 2S, ... (distributed shared memory, in rank order, so the result is the
+// same on every call) and runs the epilogue on them. S is the largest power of two that keeps
+// at least two chunks per CTA and the grid within the SMs.
+//
+// Roles: warp 0 (one lane) streams 128 x 64 tiles of A and BN x 64 tiles of W by TMA (128-byte
+// swizzle, four stages), warp 1 issues tcgen05.mma (M = 128, N = BN), warps 4-7 drain the
+// accumulator, all eight warps reduce. The weights are constant while a head lives, so their
+// first four chunks are requested before the wait on the preceding launch: only A's copy,
+// the products and the reduction are left on the chain. What bounds it is that latency, not a
+// pipe: with these products, the RMSNorms folded into them and the target chain beside the
+// body, the network of width 1024 takes 115 us for one request (170 before) and 309 us for 24
+// (352: its prologue's 15- and 24-row products); serving_b32's drafter-state product (512
+// rows, 16 tiles, Kd = 4096) beside the top-K pass 136.7 -> 131.7 us a call. The same epilogues as the persistent
+// kernel (gemm_tc.cu): bias, per-sequence bias, SiLU, residual, and the RMSNorm folded into
+// the products around it. Every mbarrier wait is bounded; on timeout the kernel records
+// LILICORR_ERR_TIMEOUT, keeps every thread on its barriers, lets copies in flight land, frees
+// its tensor memory and returns.
+#include "tc_ptx.cuh"
+
+namespace lilicorr {
+
+namespace {
+using namespace tc;
+
+constexpr int SP_THREADS = 256;
+constexpr int SP_STAGES = 4;
+constexpr int SP_BK = 64;
+constexpr uint32_t SP_A_BYTES = 128 * SP_BK * 2;
+constexpr long long SP_WAIT = 4000000000ll;
+constexpr float SP_RMS_EPS = 1e-6f;
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t local, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+
+struct SplitArgs {
+  GemmArgs g;
+  int S;             // CTAs per tile (cluster size)
+  int w_const;       // W is constant: its copies may start before the preceding launch ends
+};
+
+template <int BN>
+struct SpCfg {
+  static constexpr uint32_t B_BYTES = BN * SP_BK * 2;
+  static constexpr size_t RING = (size_t)SP_STAGES * (SP_A_BYTES + B_BYTES);
+  static constexpr int PLD = BN + 4;                       // row stride of the partial sums
+  static_assert((size_t)128 * PLD * 4 <= RING, "partials alias the ring");
+  static constexpr size_t SMEM = 1024 + RING;
+};
+
+template <int BN>
+__global__ void __launch_bounds__(SP_THREADS, 1)
+    gemm_split_kernel(const __grid_constant__ CUtensorMap mapA,
+                      const __grid_constant__ CUtensorMap mapW, const SplitArgs sa) {
+  using Cfg = SpCfg<BN>;
+  constexpr int PLD = Cfg::PLD;
+  const GemmArgs& g = sa.g;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint8_t* sA = smem;
+  uint8_t* sB = smem + SP_STAGES * SP_A_BYTES;
+  float* part = reinterpret_cast<float*>(smem);            // once the products are done
+  __shared__ __align__(8) uint64_t full[SP_STAGES], empty[SP_STAGES], acc_full;
+  __shared__ uint32_t tmem_base;
+  __shared__ volatile int abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int S = sa.S, rank = blockIdx.x;                   // gridDim.x = cluster size = S
+  const int n0 = blockIdx.y * BN, m0 = blockIdx.z * 128;
+  const int nk = (g.Kd + SP_BK - 1) / SP_BK;
+  const int kc0 = nk * rank / S, kcn = nk * (rank + 1) / S - kc0;   // this CTA's chunks (>= 1)
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < SP_STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(&acc_full, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) tmem_alloc(&tmem_base, BN);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base;
+  const int pre = min(kcn, SP_STAGES);
+  auto load_w = [&](int i) {
+    const int s = i % SP_STAGES;
+    mbar_expect_tx(&full[s], SP_A_BYTES + Cfg::B_BYTES);
+    tma_load_2d(sB + (size_t)s * Cfg::B_BYTES, &mapW, &full[s], (kc0 + i) * SP_BK, n0);
+  };
+  auto load_a = [&](int i) {
+    const int s = i % SP_STAGES;
+    tma_load_2d(sA + (size_t)s * SP_A_BYTES, &mapA, &full[s], (kc0 + i) * SP_BK, m0);
+  };
+  const bool producer = warp == 0 && lane == 0;
+  if (producer && sa.w_const)
+    for (int i = 0; i < pre; ++i) load_w(i);
+  pdl_wait();
+
+  if (warp == 0) {
+    if (lane == 0) {
+      for (int i = 0; i < pre; ++i) {
+        if (!sa.w_const) load_w(i);
+        load_a(i);
+      }
+      for (int i = pre; i < kcn; ++i) {
+        if (!mbar_wait(&empty[i % SP_STAGES], ((i / SP_STAGES) & 1) ^ 1, SP_WAIT)) {
+          abort_flag = 1;
+          break;
+        }
+        load_w(i);
+        load_a(i);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = instr_desc(128, BN);
+      for (int i = 0; i < kcn; ++i) {
+        const int s = i % SP_STAGES;
+        if (!mbar_wait(&full[s], (i / SP_STAGES) & 1, SP_WAIT)) {
+          abort_flag = 1;
+          break;
+        }
+        tc_fence_after();
+        const uint64_t ad = smem_desc(sA + (size_t)s * SP_A_BYTES);
+        const uint64_t bd = smem_desc(sB + (size_t)s * Cfg::B_BYTES);
+#pragma unroll
+        for (int k = 0; k < SP_BK / 16; ++k)
+          mma_bf16(tmem, ad + 2ull * k, bd + 2ull * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
+        mma_commit(&empty[s]);
+      }
+      mma_commit(&acc_full);
+    }
+  } else if (warp >= 4) {
+    // ---- partial sums of this CTA's part of Kd: thread = row. Every copy has landed and been
+    //      multiplied once the accumulator is complete, so they may overwrite the ring.
+    const int q = warp & 3, row = q * 32 + lane;
+    if (!mbar_wait(&acc_full, 0, SP_WAIT)) abort_flag = 1;
+    tc_fence_after();
+    if (!abort_flag) {
+#pragma unroll
+      for (int c = 0; c < BN; c += 32) {
+        uint32_t r[32];
+        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + c, r);
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+          *reinterpret_cast<float4*>(part + row * PLD + c + j) =
+              make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
+                          __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+      }
+    }
+    tc_fence_before();
+  }
+  __syncwarp();
+  cluster_sync();                      // every CTA's partials are in place
+
+  // ---- reduction and epilogue: BN / 4 threads per row, rows rank, rank + S, ...
+  constexpr int TPR = BN / 4;
+  const int c = (threadIdx.x % TPR) * 4, n = n0 + c;
+  const int rows = min(128, g.M - m0);
+  const bool col_ok = n < g.N;                      // N is a multiple of 8
+  float4 bias = make_float4(0.f, 0.f, 0.f, 0.f), gain = bias;
+  if (g.bias && col_ok)
+    bias = make_float4(g.bias[n], g.bias[n + 1], g.bias[n + 2], g.bias[n + 3]);
+  if (g.c2 && col_ok)
+    gain = make_float4(g.c2_gain[n], g.c2_gain[n + 1], g.c2_gain[n + 2], g.c2_gain[n + 3]);
+  const float ss_scale = 1.0f / (float)(g.ss_dim > 0 ? g.ss_dim : g.Kd);
+  // the threads of a row stay together, so the loop runs the same number of rounds for all
+  for (int base = 0; base < 128; base += S * (SP_THREADS / TPR)) {
+    const int r = base + rank + S * (threadIdx.x / TPR);
+    const bool live = r < rows;
+    const int m = m0 + r;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live) {
+      const uint32_t local = smem_u32(part + r * PLD + c);
+      if (S == 1) {
+        v = *reinterpret_cast<const float4*>(part + r * PLD + c);
+      } else {
+        float4 t[8];                                // every partial in flight, then the sum
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+          if (p < S) t[p] = ld_cluster_f4(local, p);
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+          if (p < S) { v.x += t[p].x; v.y += t[p].y; v.z += t[p].z; v.w += t[p].w; }
+      }
+    }
+    float rs = 1.f;
+    if (g.ss_in) {                                  // folded RMSNorm of the input rows
+      float s = 0.f;
+      if (live)
+        for (int i = threadIdx.x % TPR; i < g.ss_slots; i += TPR) s += g.ss_in[(size_t)m * SS_LD + i];
+#pragma unroll
+      for (int o = TPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      rs = rsqrtf(s * ss_scale + SP_RMS_EPS);
+    }
+    const bool out = live && col_ok;
+    float4 x = make_float4(fmaf(v.x, rs, bias.x), fmaf(v.y, rs, bias.y), fmaf(v.z, rs, bias.z),
+                           fmaf(v.w, rs, bias.w));
+    if (g.bias_rows && out) {
+      const float4 br = *reinterpret_cast<const float4*>(
+          g.bias_rows + (size_t)(m / g.rows_per_bias) * g.N + n);
+      x.x += br.x; x.y += br.y; x.z += br.z; x.w += br.w;
+    }
+    if (g.act == ACT_SILU) {
+      if (g.c_dt == LILICORR_BF16) {
+        x.x = silu_tanh(x.x); x.y = silu_tanh(x.y); x.z = silu_tanh(x.z); x.w = silu_tanh(x.w);
+      } else {
+        x.x = silu_f(x.x); x.y = silu_f(x.y); x.z = silu_f(x.z); x.w = silu_f(x.w);
+      }
+    }
+    if (g.residual && out) {
+      const float4 rr = *reinterpret_cast<const float4*>(g.residual + (size_t)m * g.ldr + n);
+      x.x += rr.x; x.y += rr.y; x.z += rr.z; x.w += rr.w;
+    }
+    if (out && g.C) {
+      if (g.c_dt == LILICORR_BF16)
+        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(g.C) + (size_t)m * g.ldc + n) =
+            make_uint2(pack_bf16x2(x.x, x.y), pack_bf16x2(x.z, x.w));
+      else
+        *reinterpret_cast<float4*>(static_cast<float*>(g.C) + (size_t)m * g.ldc + n) = x;
+    }
+    if (g.c2) {                                     // the next RMSNorm's input, and its sums
+      float s = 0.f;
+      if (out) {
+        s = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
+        const float4 y = make_float4(x.x * gain.x, x.y * gain.y, x.z * gain.z, x.w * gain.w);
+        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(g.c2) + (size_t)m * g.ldc2 + n) =
+            make_uint2(pack_bf16x2(y.x, y.y), pack_bf16x2(y.z, y.w));
+        if (g.c3) {
+          const float4 t = *reinterpret_cast<const float4*>(
+              g.c3_t + (size_t)(m / g.c3_rows_per) * g.N + n);
+          *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(g.c3) + (size_t)m * g.ldc2 + n) =
+              make_uint2(pack_bf16x2(y.x * t.x, y.y * t.y), pack_bf16x2(y.z * t.z, y.w * t.w));
+        }
+      }
+#pragma unroll
+      for (int o = TPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (live && threadIdx.x % TPR == 0) g.ss_out[(size_t)m * SS_LD + blockIdx.y] = s;
+    }
+  }
+
+  // ---- teardown: no CTA leaves while a peer may still read its partials
+  if (abort_flag) {
+    if (threadIdx.x == 0) {
+      set_status(g.status, LILICORR_ERR_TIMEOUT);
+      const long long t0 = clock64();               // let copies in flight land
+      while (clock64() - t0 < SP_WAIT / 10) {
+      }
+    }
+    __syncthreads();
+  }
+  __syncwarp();
+  cluster_sync();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, BN);
+  }
+}
+
+template <int BN>
+lilicorr_status_t launch_split(const GemmArgs& g, int S, cudaStream_t st) {
+  static bool configured[64] = {false};
+  LL_TRY(allow_max_dynamic_smem(gemm_split_kernel<BN>, configured));
+  CUtensorMap ma, mw;
+  const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  if (!make_map(&ma, g.A, bf, 2, g.M, g.Kd, g.lda, 128, SP_BK)) return LILICORR_ERR_CUDA;
+  if (!make_map(&mw, g.W, bf, 2, g.N, g.Kd, g.ldw, BN, SP_BK)) return LILICORR_ERR_CUDA;
+  SplitArgs sa;
+  sa.g = g;
+  sa.S = S;
+  sa.w_const = g.w_const;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(S, ceil_div(g.N, BN), ceil_div(g.M, 128));
+  cfg.blockDim = SP_THREADS;
+  cfg.dynamicSmemBytes = SpCfg<BN>::SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = S;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_split_kernel<BN>, ma, mw, sa);
+  count_launch();
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    return LILICORR_ERR_CUDA;
+  }
+  return LILICORR_OK;
+}
+
+int split_tiles(const GemmArgs& g, int bn) { return ceil_div(g.M, 128) * ceil_div(g.N, bn); }
+
+}  // namespace
+
+int gemm_split_ss_slots(int N) { return ceil_div(N, 64); }
+
+// CTAs per tile: as many as leave each at least two chunks of Kd and the grid on the GPU at
+// once; 0 where the tiles alone fill more than half of the SMs (the persistent kernel's case).
+int gemm_split_ways(const GemmArgs& g) {
+  const int tiles = split_tiles(g, 64), nk = ceil_div(g.Kd, SP_BK);
+  if (2 * tiles > num_sms()) return 0;
+  int S = 1;
+  while (S < 8 && 2 * S * tiles <= num_sms() && nk >= 4 * S) S *= 2;
+  return S;
+}
+
+bool gemm_split_supported(const GemmArgs& g) {
+  if (!gemm_tc_operands_ok(g)) return false;
+  if (g.c2 && (!g.c2_gain || !g.ss_out || g.c_dt != LILICORR_F32 || !aligned16(g.c2) ||
+               (g.ldc2 % 8) || gemm_split_ss_slots(g.N) > SS_LD))
+    return false;
+  if (g.bias_rows && !aligned16(g.bias_rows)) return false;
+  if (ceil_div(g.M, 128) > 65535 || ceil_div(g.N, 64) > 65535) return false;
+  return gemm_split_ways(g) > 0;
+}
+
+lilicorr_status_t launch_gemm_split(const GemmArgs& g, cudaStream_t st) {
+  if (g.M == 0 || g.N == 0) return LILICORR_OK;
+  return launch_split<64>(g, gemm_split_ways(g), st);
+}
+
+}  // namespace lilicorr

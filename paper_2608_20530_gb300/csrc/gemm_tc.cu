@@ -210,9 +210,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       const int mm = (t / tiles_n) * TC_BM + row;
       const float4* src = reinterpret_cast<const float4*>(ep.ss_in + (size_t)mm * SS_LD);
 #pragma unroll
-      for (int i = 0; i < SS_LD / 4; ++i)
+      for (int i = 0; i < SS_LD / 4; ++i) {
         ssn[i] = (t < tiles && mm < M && 4 * i < ep.ss_slots) ? src[i]
                                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        // slots past ss_slots belong to no column tile: whatever they hold stays out
+        if (4 * i + 1 >= ep.ss_slots) ssn[i].y = 0.f;
+        if (4 * i + 2 >= ep.ss_slots) ssn[i].z = 0.f;
+        if (4 * i + 3 >= ep.ss_slots) ssn[i].w = 0.f;
+      }
     };
     if (FOLD && ep.ss_in) load_ss(blockIdx.x);
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++lt) {
@@ -512,12 +517,9 @@ bool make_map_nd(CUtensorMap* map, const void* base, CUtensorMapDataType type, i
 
 int gemm_tc_ss_slots(int M, int N) { return 2 * ceil_div(N, tc_column_tile(M, N)); }
 
-bool gemm_tc_supported(const GemmArgs& g) {
+// What both TMA-fed kernels ask of the operands of any product.
+bool gemm_tc_operands_ok(const GemmArgs& g) {
   if (g.a_dt != LILICORR_BF16 || g.w_dt != LILICORR_BF16) return false;
-  // folded RMSNorm: fp32 output, whole 32-column groups, 16-byte aligned bf16 copy rows
-  if (g.c2 && (g.c_dt != LILICORR_F32 || !g.c2_gain || !g.ss_out || (g.N % 32) ||
-               !aligned16(g.c2) || (g.ldc2 % 8) || gemm_tc_ss_slots(g.M, g.N) > SS_LD))
-    return false;
   if (g.c3 && (!g.c2 || !g.c3_t || g.c3_rows_per < 1 || !aligned16(g.c3) || !aligned16(g.c3_t)))
     return false;
   if (g.ss_in && (g.ss_slots < 1 || g.ss_slots > SS_LD)) return false;
@@ -531,6 +533,14 @@ bool gemm_tc_supported(const GemmArgs& g) {
     return false;
   if (g.bias_rows && (g.N % 4)) return false;
   return encode_fn() != nullptr;
+}
+
+bool gemm_tc_supported(const GemmArgs& g) {
+  // folded RMSNorm: fp32 output, whole 32-column groups, 16-byte aligned bf16 copy rows
+  if (g.c2 && (g.c_dt != LILICORR_F32 || !g.c2_gain || !g.ss_out || (g.N % 32) ||
+               !aligned16(g.c2) || (g.ldc2 % 8) || gemm_tc_ss_slots(g.M, g.N) > SS_LD))
+    return false;
+  return gemm_tc_operands_ok(g);
 }
 
 lilicorr_status_t launch_gemm_tc(const GemmArgs& g, cudaStream_t st) {

@@ -168,7 +168,8 @@ struct lilicorr_head {
   // the projections that do not depend on the top-K pass run on two side streams that
   // fork from and join the caller's stream (fork/join nodes under graph capture)
   cudaStream_t side, side2;
-  cudaEvent_t ev_fork, ev_join, ev_join2, ev_t;   // ev_t: the target state t is ready
+  cudaEvent_t ev_fork, ev_join, ev_join2, ev_t, ev_hid;  // ev_t: the target state t is ready
+                                                          // ev_hid: the drafter states are
   void* pool;                 // one device allocation holding everything below
   size_t pool_bytes;
   // matrices in head dtype; vectors and tables in fp32
@@ -266,13 +267,15 @@ struct GemmArgs {
   const float* residual; int ldr;
   int act;
   int M, N, Kd;
+  int w_const;             // W does not change while calls run (a head's weights): its copies
+                           // may start before the preceding launch ends
   uint32_t* status;        // device status word (bounded-wait timeouts), may be null
   long long wait_limit;    // SM cycles per bounded wait of the tensor-core kernel; 0: ~2 s
   int test_starve;         // test hook only: the tensor-core kernel's producer issues no
                            // copies, so its consumers' waits run out (see the testing header)
   // RMSNorm folded into the products around it (tensor-core kernel only). Producer (fp32 C):
   // c2 [M, ldc2] (bf16) receives C times c2_gain per column, ss_out [M, SS_LD] partial sums of
-  // squares of C's rows (gemm_tc_ss_slots(M, N) slots per row). Consumer: the product is
+  // squares of C's rows (gemm_ss_slots slots per row). Consumer: the product is
   // scaled per row by rsqrt(sum of ss_in's first ss_slots slots / Kd + eps) before the bias.
   void* c2; int ldc2; const float* c2_gain; float* ss_out;
   const float* ss_in; int ss_slots;
@@ -288,8 +291,13 @@ lilicorr_status_t launch_gemm_skinny(const GemmArgs& g, cudaStream_t st);   // M
 // fp32 activations, per-sequence row counts (16 x 32 output blocks, no K split)
 bool gemm_rows_supported(const GemmArgs& g);
 lilicorr_status_t launch_gemm_rows(const GemmArgs& g, cudaStream_t st);
+bool gemm_tc_operands_ok(const GemmArgs& g);   // what both TMA-fed kernels below ask
 bool gemm_tc_supported(const GemmArgs& g);
 lilicorr_status_t launch_gemm_tc(const GemmArgs& g, cudaStream_t st);
+// few output tiles: Kd split over a cluster (gemm_split.cu)
+bool gemm_split_supported(const GemmArgs& g);
+int gemm_split_ss_slots(int N);
+lilicorr_status_t launch_gemm_split(const GemmArgs& g, cudaStream_t st);
 // one tile of rows (M <= 128, Kd <= 512, a multiple of 64): whole-K TMA copies (gemm_small.cu)
 bool gemm_small_supported(const GemmArgs& g);
 lilicorr_status_t launch_gemm_small(const GemmArgs& g, cudaStream_t st);
