@@ -15,79 +15,193 @@ constexpr float RMS_EPS = 1e-6f;
 constexpr float UNIT_EPS = 1e-12f;
 
 // ----------------------------------------------------------------------------- linear
-constexpr int GB_M = 64, GB_N = 64, GB_K = 16, G_THREADS = 256;
+// fp32 CUDA-core linear layer. A CTA of 256 threads owns a 64 x 64 output tile; its four
+// groups of 64 threads (8 x 8 outputs each thread) take a quarter each of every 32-wide step of
+// Kd and add their sums up at the end. What bounds it: one wave of CTAs (2048 rows x 256
+// columns are 128 tiles), so the chain of Kd steps within a CTA, and shared-memory reads (a
+// 16-byte read takes four cycles of the SM: 8 x 8 outputs read 16 values for 64 products, 8 x 4
+// outputs 12 for 32). One group with all of Kd had one warp per scheduler, each read of shared
+// memory exposed: 31 us for 2048 x 256 x 256. Pairs of columns are one f32x2 multiply-add; the
+// next step's operands are loaded (16 bytes a thread where rows allow) while this one is
+// multiplied.
+// 2048 x 256 x 256: 31 -> 15.5 us; 2048 x 256 x 512: 55 -> 23.6 us (cold).
+constexpr int GB_M = 64, GB_N = 64, GB_K = 32, G_THREADS = 256, G_GROUPS = 4;
 
-template <typename TA, typename TW, typename TC>
-__global__ void __launch_bounds__(G_THREADS) gemm_simt_kernel(GemmArgs g) {
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+  return ((uint64_t)__float_as_uint(hi) << 32) | __float_as_uint(lo);
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// four consecutive elements of row r starting at column k (zeros outside [0, rows) x [0, cols))
+template <bool VEC>
+__device__ __forceinline__ float4 load4(const float* p, int r, int rows, int k, int cols, int ld) {
+  if (r >= rows) return make_float4(0.f, 0.f, 0.f, 0.f);
+  p += (size_t)r * ld + k;
+  if (VEC) return k < cols ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+  return make_float4(k < cols ? p[0] : 0.f, k + 1 < cols ? p[1] : 0.f, k + 2 < cols ? p[2] : 0.f,
+                     k + 3 < cols ? p[3] : 0.f);
+}
+template <bool VEC>
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p, int r, int rows, int k, int cols,
+                                        int ld) {
+  if (r >= rows) return make_float4(0.f, 0.f, 0.f, 0.f);
+  p += (size_t)r * ld + k;
+  if (VEC) {
+    if (k >= cols) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u),
+                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
+  }
+  return make_float4(k < cols ? __bfloat162float(p[0]) : 0.f,
+                     k + 1 < cols ? __bfloat162float(p[1]) : 0.f,
+                     k + 2 < cols ? __bfloat162float(p[2]) : 0.f,
+                     k + 3 < cols ? __bfloat162float(p[3]) : 0.f);
+}
+
+// VEC: rows of both operands in whole aligned groups of four elements
+template <typename TA, typename TW, typename TC, bool VEC>
+__global__ void __launch_bounds__(G_THREADS, 2) gemm_simt_kernel(GemmArgs g) {
   pdl_wait();
-  __shared__ float As[GB_K][GB_M + 4];
-  __shared__ __align__(16) float Ws[GB_K][GB_N + 4];
+  constexpr int LDT = GB_M + 4, KG = GB_K / G_GROUPS;
+  static_assert(GB_M == GB_N && GB_M * GB_K == 8 * G_THREADS, "two groups of four a thread");
+  // [buffer][A or W][k][row]; after the products two groups' sums at a time
+  __shared__ __align__(16) float sm[2][2][GB_K][LDT];
+  static_assert(sizeof(sm) >= 2 * GB_M * LDT * sizeof(float), "two groups' sums fit");
   const TA* A = static_cast<const TA*>(g.A);
   const TW* W = static_cast<const TW*>(g.W);
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, grp = tid >> 6;
   const int m0 = blockIdx.y * GB_M, n0 = blockIdx.x * GB_N;
-  const int tx = tid & 15, ty = tid >> 4;
-  float acc[4][4];
+  const int tx = tid & 7, ty = (tid >> 3) & 7;
+  const int lr = tid >> 3, lk = (tid & 7) * 4;        // rows lr and lr + 32, columns lk..lk + 3
+  uint64_t acc[8][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-  for (int k0 = 0; k0 < g.Kd; k0 += GB_K) {
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  float4 ra[2], rw[2];
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int i = tid; i < GB_M * GB_K; i += G_THREADS) {
-      const int r = i / GB_K, c = i % GB_K;
-      const int gm = m0 + r, gk = k0 + c;
-      As[c][r] = (gm < g.M && gk < g.Kd) ? ld_elem(A, (size_t)gm * g.lda + gk) : 0.f;
-      const int gn = n0 + r;
-      Ws[c][r] = (gn < g.N && gk < g.Kd) ? ld_elem(W, (size_t)gn * g.ldw + gk) : 0.f;
+    for (int h = 0; h < 2; ++h) {
+      ra[h] = load4<VEC>(A, m0 + lr + 32 * h, g.M, k0 + lk, g.Kd, g.lda);
+      rw[h] = load4<VEC>(W, n0 + lr + 32 * h, g.N, k0 + lk, g.Kd, g.ldw);
     }
-    __syncthreads();
+  };
+  auto stash = [&](int b) {
 #pragma unroll
-    for (int kk = 0; kk < GB_K; ++kk) {
-      float a[4];
+    for (int h = 0; h < 2; ++h) {
+      const int r = lr + 32 * h;
+      sm[b][0][lk][r] = ra[h].x; sm[b][0][lk + 1][r] = ra[h].y;
+      sm[b][0][lk + 2][r] = ra[h].z; sm[b][0][lk + 3][r] = ra[h].w;
+      sm[b][1][lk][r] = rw[h].x; sm[b][1][lk + 1][r] = rw[h].y;
+      sm[b][1][lk + 2][r] = rw[h].z; sm[b][1][lk + 3][r] = rw[h].w;
+    }
+  };
+  fetch(0);
+  stash(0);
+  __syncthreads();
+  int b = 0;
+  for (int k0 = 0; k0 < g.Kd; k0 += GB_K, b ^= 1) {
+    const bool more = k0 + GB_K < g.Kd;
+    if (more) fetch(k0 + GB_K);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-      const float4 b = *reinterpret_cast<const float4*>(&Ws[kk][tx * 4]);
+    for (int kk = 0; kk < KG; ++kk) {
+      // rows ty*4.. and 32 + ty*4.., columns tx*4.. and 32 + tx*4..
+      const float* as = sm[b][0][grp * KG + kk];
+      const float* ws = sm[b][1][grp * KG + kk];
+      const float4 a0 = *reinterpret_cast<const float4*>(as + ty * 4);
+      const float4 a1 = *reinterpret_cast<const float4*>(as + 32 + ty * 4);
+      const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(ws + tx * 4);
+      const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(ws + 32 + tx * 4);
+      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[i][0] = fmaf(a[i], b.x, acc[i][0]);
-        acc[i][1] = fmaf(a[i], b.y, acc[i][1]);
-        acc[i][2] = fmaf(a[i], b.z, acc[i][2]);
-        acc[i][3] = fmaf(a[i], b.w, acc[i][3]);
+      for (int i = 0; i < 8; ++i) {
+        const uint64_t aa = pack_f32x2(a[i], a[i]);
+        acc[i][0] = fma_f32x2(aa, w0.x, acc[i][0]);
+        acc[i][1] = fma_f32x2(aa, w0.y, acc[i][1]);
+        acc[i][2] = fma_f32x2(aa, w1.x, acc[i][2]);
+        acc[i][3] = fma_f32x2(aa, w1.y, acc[i][3]);
       }
     }
+    if (more) stash(b ^ 1);           // its last readers are behind the previous barrier
     __syncthreads();
   }
-  TC* C = static_cast<TC*>(g.C);
+  // ---- the groups' sums: 2 into 0 and 3 into 1, then both for the epilogue
+  float* red = &sm[0][0][0][0];
+  auto at = [&](int q, int i, int j) {              // thread's rows i, column quads j
+    return reinterpret_cast<ulonglong2*>(red + (size_t)q * GB_M * LDT +
+                                         ((i >> 2) * 32 + ty * 4 + (i & 3)) * LDT + j * 32 + tx * 4);
+  };
+  auto put = [&](int q) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= g.M) continue;
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) *at(q, i, j) = make_ulonglong2(acc[i][2 * j], acc[i][2 * j + 1]);
+  };
+  if (grp >= 2) put(grp - 2);
+  __syncthreads();
+  if (grp < 2) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const ulonglong2 o = *at(grp, i, j);
+        acc[i][2 * j] = add_f32x2(acc[i][2 * j], o.x);
+        acc[i][2 * j + 1] = add_f32x2(acc[i][2 * j + 1], o.y);
+      }
+    // each thread overwrites only what it has just read itself
+    put(grp);
+  }
+  __syncthreads();
+  // ---- epilogue: 16 threads a row, four columns each
+  TC* C = static_cast<TC*>(g.C);
+  const int c = (tid & 15) * 4, n = n0 + c;
+#pragma unroll
+  for (int r = tid >> 4; r < GB_M; r += G_THREADS / 16) {
+    const int m = m0 + r;
+    if (m >= g.M) break;
+    const float4 s0 = *reinterpret_cast<const float4*>(red + r * LDT + c);
+    const float4 s1 = *reinterpret_cast<const float4*>(red + (GB_M + r) * LDT + c);
+    const float s[4] = {s0.x + s1.x, s0.y + s1.y, s0.z + s1.z, s0.w + s1.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= g.N) continue;
-      float v = acc[i][j];
-      if (g.bias) v += g.bias[n];
-      if (g.bias_rows) v += g.bias_rows[(size_t)(m / g.rows_per_bias) * g.N + n];
+      if (n + j >= g.N) break;
+      float v = s[j];
+      if (g.bias) v += g.bias[n + j];
+      if (g.bias_rows) v += g.bias_rows[(size_t)(m / g.rows_per_bias) * g.N + n + j];
       if (g.act == ACT_SILU) v = silu_f(v);
-      if (g.residual) v += g.residual[(size_t)m * g.ldr + n];
-      st_elem(C, (size_t)m * g.ldc + n, v);
+      if (g.residual) v += g.residual[(size_t)m * g.ldr + n + j];
+      st_elem(C, (size_t)m * g.ldc + n + j, v);
     }
   }
 }
 
-template <typename TA, typename TW>
+template <typename TA, typename TW, bool VEC>
 lilicorr_status_t gemm_dispatch_c(const GemmArgs& g, dim3 grid, cudaStream_t st) {
-  if (g.c_dt == LILICORR_F32) LL_TRY(launch_k(gemm_simt_kernel<TA, TW, float>, grid, G_THREADS, 0, st, g));
-  else LL_TRY(launch_k(gemm_simt_kernel<TA, TW, __nv_bfloat16>, grid, G_THREADS, 0, st, g));
-  return LILICORR_OK;
+  if (g.c_dt == LILICORR_F32)
+    return launch_k(gemm_simt_kernel<TA, TW, float, VEC>, grid, G_THREADS, 0, st, g);
+  return launch_k(gemm_simt_kernel<TA, TW, __nv_bfloat16, VEC>, grid, G_THREADS, 0, st, g);
 }
 template <typename TA>
 lilicorr_status_t gemm_dispatch_w(const GemmArgs& g, dim3 grid, cudaStream_t st) {
-  if (g.w_dt == LILICORR_F32) return gemm_dispatch_c<TA, float>(g, grid, st);
-  return gemm_dispatch_c<TA, __nv_bfloat16>(g, grid, st);
+  // groups of four elements: Kd and the row strides multiples of 4, bases on 16 (fp32) or 8
+  // (bf16) bytes; other operands are read element by element
+  const uintptr_t am = sizeof(TA) * 4 - 1, wm = g.w_dt == LILICORR_F32 ? 15 : 7;
+  const bool vec = g.Kd % 4 == 0 && g.lda % 4 == 0 && g.ldw % 4 == 0 &&
+                   !(reinterpret_cast<uintptr_t>(g.A) & am) &&
+                   !(reinterpret_cast<uintptr_t>(g.W) & wm);
+  if (g.w_dt == LILICORR_F32)
+    return vec ? gemm_dispatch_c<TA, float, true>(g, grid, st)
+               : gemm_dispatch_c<TA, float, false>(g, grid, st);
+  return vec ? gemm_dispatch_c<TA, __nv_bfloat16, true>(g, grid, st)
+             : gemm_dispatch_c<TA, __nv_bfloat16, false>(g, grid, st);
 }
 
 // ----------------------------------------------------------------------------- skinny linear
