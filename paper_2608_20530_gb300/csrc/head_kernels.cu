@@ -606,76 +606,173 @@ __global__ void unit_rows_kernel(const float* __restrict__ src, int rows, int n,
 }
 
 // ----------------------------------------------------------------------------- attention
-// One CTA per (sequence, head): all L*K nodes attend to all L*K nodes (no mask),
-// logits q.k / sqrt(hd) + dist[h, s_j - s_i + L - 1] + same[h] * 1{s_i == s_j}.
+// A CTA takes a block of queries of one (sequence, head): all L*K nodes attend to all L*K
+// nodes (no mask), logits q.k / sqrt(hd) + dist[h, s_j - s_i + L - 1] + same[h] * 1{s_i == s_j}.
 // qkv rows hold [q | k | v], each D wide, head h in columns [h*hd, (h+1)*hd).
+//
+// Bound by shared-memory reads, so a warp takes AQ = 4 queries at once and everything moves in
+// 16-byte pieces: scores with a lane per key, four keys and four queries a lane (8 reads per 64
+// products); P V with a lane per four columns (and, below 128-wide heads, per part of the
+// keys), the four queries' probabilities of a key one piece (2 reads per 16 products). One
+// query a warp and single words read twice per product: 128 nodes x 128 (sequence, head)
+// pairs of 32, 45 us -> 22 us (cold).
+constexpr int AQ = 4;
+
+__device__ __forceinline__ void fma4(float& acc, const float4& a, const float4& b) {
+  acc = fmaf(a.x, b.x, acc);
+  acc = fmaf(a.y, b.y, acc);
+  acc = fmaf(a.z, b.z, acc);
+  acc = fmaf(a.w, b.w, acc);
+}
+
 template <typename TO>
-__global__ void attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads,
-                                 int q_per_cta, const float* __restrict__ dist,
-                                 const float* __restrict__ same, TO* __restrict__ out) {
+__global__ void __launch_bounds__(256)
+attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads, int q_per_cta,
+                 const float* __restrict__ dist, const float* __restrict__ same,
+                 TO* __restrict__ out) {
   pdl_wait();
-  extern __shared__ float sm[];
+  extern __shared__ __align__(16) float sm[];
   const int LK = L * K, hd = D / n_heads;
   const int b = blockIdx.x / n_heads, h = blockIdx.x % n_heads;
   const int q0 = blockIdx.y * q_per_cta, q1 = min(LK, q0 + q_per_cta);
   const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* Ks = sm;                       // [LK][hd + 1]
-  float* Vs = Ks + (size_t)LK * (hd + 1);   // [LK][hd]
-  float* Qw = Vs + (size_t)LK * hd;     // [nw][hd]
-  float* Pw = Qw + (size_t)nw * hd;     // [nw][LK]
+  const int kld = hd + 4;                      // K rows a piece apart in banks
+  float* Ks = sm;                              // [LK][hd + 4]
+  float* Vs = Ks + (size_t)LK * kld;           // [LK][hd]
+  float* Qw = Vs + (size_t)LK * hd;            // [nw][AQ][hd]
+  float* Pw = Qw + (size_t)nw * AQ * hd;       // [nw][LK][AQ]
+  float* s_dist = Pw + (size_t)nw * LK * AQ;   // [2L - 1]
   const size_t ld = 3 * (size_t)D;
-  const float* base = qkv + (size_t)b * LK * ld;
-  const int hv = hd / 4;                       // 16-byte vectors per head row
+  const float* base = qkv + (size_t)b * LK * ld + h * hd;
+  const int hv = hd / 4;                       // 16-byte pieces per head row
 #pragma unroll 4
   for (int i = threadIdx.x; i < LK * hv; i += blockDim.x) {
     const int j = i / hv, c = (i % hv) * 4;
-    const float4 kv = *reinterpret_cast<const float4*>(base + j * ld + D + h * hd + c);
-    const float4 vv = *reinterpret_cast<const float4*>(base + j * ld + 2 * D + h * hd + c);
-    float* kd = Ks + j * (hd + 1) + c;
-    kd[0] = kv.x; kd[1] = kv.y; kd[2] = kv.z; kd[3] = kv.w;
-    *reinterpret_cast<float4*>(Vs + j * hd + c) = vv;
+    *reinterpret_cast<float4*>(Ks + j * kld + c) =
+        *reinterpret_cast<const float4*>(base + j * ld + D + c);
+    *reinterpret_cast<float4*>(Vs + j * hd + c) =
+        *reinterpret_cast<const float4*>(base + j * ld + 2 * D + c);
   }
+  for (int i = threadIdx.x; i < 2 * L - 1; i += blockDim.x)
+    s_dist[i] = dist[(size_t)h * (2 * L - 1) + i];
   __syncthreads();
   const float scale = rsqrtf((float)hd);
-  const float* dh = dist + (size_t)h * (2 * L - 1);
   const float sh = same[h];
-  float* q = Qw + warp * hd;
-  float* p = Pw + (size_t)warp * LK;
-  for (int i = q0 + warp; i < q1; i += nw) {
-    for (int c = lane; c < hd; c += 32) q[c] = base[(size_t)i * ld + h * hd + c];
+  float* q = Qw + (size_t)warp * AQ * hd;
+  float4* p = reinterpret_cast<float4*>(Pw + (size_t)warp * LK * AQ);
+  // P V: lane = columns 4 cg.., keys ks, ks + nks, ...
+  const int cg = lane % hv, ks = lane / hv, nks = 32 / hv;
+  for (int i0 = q0 + AQ * warp; i0 < q1; i0 += AQ * nw) {
+    const int nq = min(AQ, q1 - i0);           // a short last group repeats its last query
+    for (int i = lane; i < AQ * hv; i += 32)
+      *reinterpret_cast<float4*>(q + 4 * i) = *reinterpret_cast<const float4*>(
+          base + (size_t)(i0 + min(i / hv, nq - 1)) * ld + 4 * (i % hv));
     __syncwarp();
-    const int si = i / K;
-    float mx = -INFINITY;
-    for (int j = lane; j < LK; j += 32) {
-      const float* kj = Ks + j * (hd + 1);
-      float acc = 0.f;
-      for (int c = 0; c < hd; ++c) acc = fmaf(q[c], kj[c], acc);
-      const int sj = j / K;
-      const float v = acc * scale + dh[sj - si + L - 1] + (si == sj ? sh : 0.f);
-      p[j] = v;
-      mx = fmaxf(mx, v);
+    int si[AQ];
+    float mx[AQ];
+#pragma unroll
+    for (int a = 0; a < AQ; ++a) {
+      si[a] = (i0 + min(a, nq - 1)) / K;
+      mx[a] = -INFINITY;
     }
-    mx = warp_max(mx);
-    float sum = 0.f;
-    for (int j = lane; j < LK; j += 32) {
-      const float e = __expf(p[j] - mx);
+    for (int j0 = 0; j0 < LK; j0 += 128) {
+      float s[4][AQ];
+      const float* kr[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        kr[t] = Ks + min(j0 + lane + 32 * t, LK - 1) * kld;
+#pragma unroll
+        for (int a = 0; a < AQ; ++a) s[t][a] = 0.f;
+      }
+      for (int c = 0; c < hd; c += 4) {
+        float4 qv[AQ];
+#pragma unroll
+        for (int a = 0; a < AQ; ++a) qv[a] = *reinterpret_cast<const float4*>(q + a * hd + c);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const float4 kv = *reinterpret_cast<const float4*>(kr[t] + c);
+#pragma unroll
+          for (int a = 0; a < AQ; ++a) fma4(s[t][a], qv[a], kv);
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int j = j0 + lane + 32 * t;
+        if (j >= LK) continue;
+        const int sj = j / K;
+#pragma unroll
+        for (int a = 0; a < AQ; ++a) {
+          s[t][a] = s[t][a] * scale + s_dist[sj - si[a] + L - 1] + (si[a] == sj ? sh : 0.f);
+          mx[a] = fmaxf(mx[a], s[t][a]);
+        }
+        p[j] = make_float4(s[t][0], s[t][1], s[t][2], s[t][3]);
+      }
+    }
+    float sum[AQ];
+#pragma unroll
+    for (int a = 0; a < AQ; ++a) {
+      mx[a] = warp_max(mx[a]);
+      sum[a] = 0.f;
+    }
+    for (int j = lane; j < LK; j += 32) {      // each lane the keys it scored
+      float4 e = p[j];
+      e.x = __expf(e.x - mx[0]); e.y = __expf(e.y - mx[1]);
+      e.z = __expf(e.z - mx[2]); e.w = __expf(e.w - mx[3]);
       p[j] = e;
-      sum += e;
+      sum[0] += e.x; sum[1] += e.y; sum[2] += e.z; sum[3] += e.w;
     }
-    sum = warp_sum(sum);
     __syncwarp();
-    const float inv = 1.0f / sum;
-    for (int c = lane; c < hd; c += 32) {
-      float acc = 0.f;
-      for (int j = 0; j < LK; ++j) acc = fmaf(p[j], Vs[j * hd + c], acc);
-      st_elem(out, ((size_t)b * LK + i) * D + h * hd + c, acc * inv);
+    float4 o[AQ];
+#pragma unroll
+    for (int a = 0; a < AQ; ++a) {
+      sum[a] = 1.0f / warp_sum(sum[a]);
+      o[a] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (ks < nks)
+#pragma unroll 4
+      for (int j = ks; j < LK; j += nks) {
+        const float4 v = *reinterpret_cast<const float4*>(Vs + j * hd + 4 * cg);
+        const float4 pj = p[j];
+        const float w[AQ] = {pj.x, pj.y, pj.z, pj.w};
+#pragma unroll
+        for (int a = 0; a < AQ; ++a) {
+          o[a].x = fmaf(w[a], v.x, o[a].x);
+          o[a].y = fmaf(w[a], v.y, o[a].y);
+          o[a].z = fmaf(w[a], v.z, o[a].z);
+          o[a].w = fmaf(w[a], v.w, o[a].w);
+        }
+      }
+#pragma unroll
+    for (int a = 0; a < AQ; ++a) {
+      float4 r = o[a];
+      for (int k = 1; k < nks; ++k) {          // the parts of the keys, in order
+        const int src = cg + k * hv;
+        r.x += __shfl_sync(0xffffffffu, o[a].x, src);
+        r.y += __shfl_sync(0xffffffffu, o[a].y, src);
+        r.z += __shfl_sync(0xffffffffu, o[a].z, src);
+        r.w += __shfl_sync(0xffffffffu, o[a].w, src);
+      }
+      if (ks == 0 && a < nq) {
+        TO* dst = out + ((size_t)b * LK + i0 + a) * D + h * hd + 4 * cg;
+        st_elem(dst, 0, r.x * sum[a]);
+        st_elem(dst, 1, r.y * sum[a]);
+        st_elem(dst, 2, r.z * sum[a]);
+        st_elem(dst, 3, r.w * sum[a]);
+      }
     }
     __syncwarp();
   }
 }
 
+// floats of shared memory beside s_dist, for `warps` warps
+size_t attention_floats(int LK, int hd, int warps) {
+  return (size_t)LK * (2 * hd + 4) + (size_t)warps * AQ * (hd + LK);
+}
+
 }  // namespace
 
+// What the CUDA-core attention core may take of shared memory decides which heads exist (the
+// limit lies at 200 KB of this); launch_attention takes as many warps as then fit.
 size_t attention_smem_bytes(int LK, int hd, int warps) {
   return sizeof(float) * ((size_t)LK * (hd + 1) + (size_t)LK * hd + (size_t)warps * hd +
                           (size_t)warps * LK);
@@ -787,16 +884,21 @@ lilicorr_status_t launch_attention(const float* qkv, int B, int L, int K, int D,
                                    const float* dist, const float* same, void* out,
                                    lilicorr_dtype_t out_dt, cudaStream_t st) {
   if (B == 0) return LILICORR_OK;
-  const int warps = 8;
-  const int LK = L * K;
-  const size_t smem = attention_smem_bytes(LK, D / n_heads, warps);
+  const int LK = L * K, hd = D / n_heads;
+  // the most warps whose queries and probabilities fit beside K and V (every head that
+  // exists leaves room for two)
+  const size_t most = SMEM_PER_BLOCK_MAX - 2 * LILICORR_MAX_L * sizeof(float);
+  int warps = 8;
+  while (warps > 2 && attention_floats(LK, hd, warps) * sizeof(float) > most) warps /= 2;
+  const size_t smem = (attention_floats(LK, hd, warps) + 2 * L - 1) * sizeof(float);
   static bool cfg_f32[64] = {false}, cfg_bf16[64] = {false};
   LL_TRY(allow_max_dynamic_smem(attention_kernel<float>, cfg_f32));
   LL_TRY(allow_max_dynamic_smem(attention_kernel<__nv_bfloat16>, cfg_bf16));
-  // split the queries of a (sequence, head) over CTAs until the grid covers the GPU
-  int qblocks = ceil_div(2 * num_sms(), B * n_heads);
-  qblocks = max(1, min(qblocks, ceil_div(LK, 2 * warps)));
-  const int q_per_cta = ceil_div(LK, qblocks);
+  // split the queries of a (sequence, head) over CTAs until the grid covers the GPU; each warp
+  // takes whole groups of AQ
+  int qblocks = ceil_div(4 * num_sms(), B * n_heads);
+  qblocks = max(1, min(qblocks, ceil_div(LK, AQ * warps)));
+  const int q_per_cta = ceil_div(ceil_div(LK, qblocks), AQ) * AQ;
   qblocks = ceil_div(LK, q_per_cta);
   dim3 grid(B * n_heads, qblocks);
   if (out_dt == LILICORR_F32)
