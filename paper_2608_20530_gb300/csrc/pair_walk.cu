@@ -154,12 +154,12 @@ __device__ __forceinline__ float dot4(const float4& x, const float4& y, float ac
 }
 
 // Dot products of the 4 x 4 block of rows x (xr..xr+3, the earlier slot) and y (yr..yr+3,
-// slot j) over the 16-byte columns f = split, split + 16, ... within [f0, f1); the thread's
+// slot j) over the 16-byte columns f = split, split + step, ... within [f0, f1); the thread's
 // squared norms of those rows alongside when nx / ny are asked for.
 __device__ __forceinline__ void block_dots(const float* sm, int ds, int xr, int yr, int f0, int f1,
-                                           int split, bool want_nx, bool want_ny,
+                                           int split, int step, bool want_nx, bool want_ny,
                                            float (&acc)[4][4], float (&nx)[4], float (&ny)[4]) {
-  for (int f = f0 + split; f < f1; f += 16) {
+  for (int f = f0 + split; f < f1; f += step) {
     float4 xv[4], yv[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -191,16 +191,17 @@ __device__ __forceinline__ void sum16(float (&v)[N]) {
 // CTA (b, j): the slot pair (j - 1, j), or the anchor row (j = 0). The K in vectors of slot
 // j (rows 0 .. K-1) and the earlier slot's out vectors or the anchor (rows R ..) are staged
 // in shared memory by asynchronous copies in two column halves, so the products of the
-// first half run while the second lands. The nrows x K outputs go in 4 x 4 blocks: thread t
-// takes block t / 16 and the 16-byte columns t % 16, t % 16 + 16, ... of every row, so the
-// 16 lanes of a block read 256 consecutive bytes of a row (no bank conflicts) and each
-// loaded piece feeds four products; the 16 partial sums meet by shuffles. The row norms
+// first half run while the second lands. The nrows x K outputs go in 4 x 4 blocks: a group of
+// 16 lanes takes a block and 16 of its 16-byte columns at a time, so it reads 256 consecutive
+// bytes of a row (no bank conflicts) and each loaded piece feeds four products; the 16
+// partial sums meet by shuffles. The row norms
 // come out of the same pass (blocks of the first row / column group).
 __global__ void __launch_bounds__(PW_THREADS) pair_block_kernel(PairWalkArgs a) {
   pdl_wait();
   extern __shared__ float sm[];
   __shared__ int s_last;
   __shared__ float s_nx[LILICORR_MAX_K], s_ny[LILICORR_MAX_K];
+  __shared__ float s_part[PW_THREADS / 16][24];    // a group's 16 sums, 4 + 4 norms
   __shared__ uint8_t s_back[LILICORR_MAX_L * LILICORR_MAX_K];
   __shared__ uint8_t s_path[LILICORR_MAX_L];
   const int b = blockIdx.x, j = blockIdx.y;
@@ -247,38 +248,55 @@ __global__ void __launch_bounds__(PW_THREADS) pair_block_kernel(PairWalkArgs a) 
     const int r = 4 * bx + (split >> 2), k2 = 4 * by + (split & 3);
     if (r < nrows && k2 < K) outp[(size_t)r * K + k2] = v / (s_nx[r] * s_ny[k2]);
   };
-  auto put_norms = [&](int bx, int by, const float (&nx)[4], const float (&ny)[4]) {
-    if (split != 0) return;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      if (by == 0 && 4 * bx + r < nrows) s_nx[4 * bx + r] = fmaxf(sqrtf(nx[r]), UNIT_EPS);
-      if (bx == 0 && 4 * by + r < K) s_ny[4 * by + r] = fmaxf(sqrtf(ny[r]), UNIT_EPS);
-    }
-  };
 
   if (nblk <= PW_THREADS / 16) {
-    // one block per thread (K <= 16): the first half's products while the second lands
-    const int blk = threadIdx.x >> 4;
-    const bool active = blk < nblk;
-    const int bx = active ? blk / nby : 0, by = active ? blk % nby : 0;
+    // one block per thread (K <= 16): the first half's products while the second lands. With
+    // fewer blocks than groups of 16 lanes, `parts` groups share a block's columns (8
+    // candidates: four blocks, four parts each; left to one group each, 64 of the 256
+    // threads did all of the work: 200 x 15 slots of 8 x 1024-wide vectors, 51 -> 44 us cold,
+    // 196 MB) and their sums meet in shared memory, in order.
+    const int grp = threadIdx.x >> 4;
+    const int parts = PW_THREADS / 16 / nblk;
+    const int blk = grp % nblk, part = grp / nblk;
+    const bool active = part < parts;
+    const int bx = blk / nby, by = blk % nby;
+    const int f_first = split + 16 * part, f_step = 16 * parts;
     float acc[4][4] = {}, nx[4] = {}, ny[4] = {};
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
-    if (active) block_dots(sm, ds, R + 4 * bx, 4 * by, 0, h4, split, by == 0, bx == 0, acc, nx, ny);
+    if (active)
+      block_dots(sm, ds, R + 4 * bx, 4 * by, 0, h4, f_first, f_step, by == 0, bx == 0, acc, nx, ny);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    if (active) block_dots(sm, ds, R + 4 * bx, 4 * by, h4, d4, split, by == 0, bx == 0, acc, nx, ny);
-    sum16(nx);
-    sum16(ny);
-    if (active) put_norms(bx, by, nx, ny);
+    if (active)
+      block_dots(sm, ds, R + 4 * bx, 4 * by, h4, d4, f_first, f_step, by == 0, bx == 0, acc, nx, ny);
+    // a lane keeps output split of its block; the norms' sums follow in lanes 0-3 and 4-7
     float flat[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) flat[i] = acc[i >> 2][i & 3];
     sum16(flat);
+    sum16(nx);
+    sum16(ny);
+    float v = 0.f, n = 0.f;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i >> 2][i & 3] = flat[i];
+    for (int i = 0; i < 16; ++i) v = split == i ? flat[i] : v;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) n = split == i ? nx[i] : split == 4 + i ? ny[i] : n;
+    s_part[grp][split] = v;
+    if (split < 8) s_part[grp][16 + split] = n;
+    __syncthreads();
+    if (part == 0) {
+      for (int q = 1; q < parts; ++q) {
+        v += s_part[grp + q * nblk][split];
+        if (split < 8) n += s_part[grp + q * nblk][16 + split];
+      }
+      n = fmaxf(sqrtf(n), UNIT_EPS);
+      if (split < 4 && by == 0 && 4 * bx + split < nrows) s_nx[4 * bx + split] = n;
+      if (split >= 4 && split < 8 && bx == 0 && 4 * by + split - 4 < K) s_ny[4 * by + split - 4] = n;
+    }
     __syncthreads();                               // the norms
-    if (active) put(bx, by, acc);
+    const int r = 4 * bx + (split >> 2), k2 = 4 * by + (split & 3);
+    if (part == 0 && r < nrows && k2 < K) outp[(size_t)r * K + k2] = v / (s_nx[r] * s_ny[k2]);
   } else {
     // more blocks than the CTA holds at once (K > 16): norms first, then block after block
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -291,7 +309,7 @@ __global__ void __launch_bounds__(PW_THREADS) pair_block_kernel(PairWalkArgs a) 
       float acc[4][4] = {}, nx[4] = {}, ny[4] = {};
       const bool xs = blk < nbx;
       const int bx = xs ? blk : 0, by = xs ? 0 : (act ? blk - nbx : 0);
-      if (act) block_dots(sm, ds, R + 4 * bx, 4 * by, 0, d4, split, xs, !xs, acc, nx, ny);
+      if (act) block_dots(sm, ds, R + 4 * bx, 4 * by, 0, d4, split, 16, xs, !xs, acc, nx, ny);
       sum16(nx);
       sum16(ny);
       if (act && split == 0)
@@ -307,7 +325,7 @@ __global__ void __launch_bounds__(PW_THREADS) pair_block_kernel(PairWalkArgs a) 
       const bool active = blk < nblk;                // warp-uniform: 2 blocks per warp
       const int bx = active ? blk / nby : 0, by = active ? blk % nby : 0;
       float acc[4][4] = {}, nx[4], ny[4];
-      if (active) block_dots(sm, ds, R + 4 * bx, 4 * by, 0, d4, split, false, false, acc, nx, ny);
+      if (active) block_dots(sm, ds, R + 4 * bx, 4 * by, 0, d4, split, 16, false, false, acc, nx, ny);
       float flat[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) flat[i] = acc[i >> 2][i & 3];
