@@ -74,10 +74,18 @@ __device__ void viterbi_sequence(const float* A, const float* P, int b, int L, i
     const float* Ps = P + (size_t)(s - 1) * K * K;
     float bv = -INFINITY;
     int bk = 0;
-    for (int k = 0; k < K; ++k) {
-      const float pk = __shfl_sync(0xffffffffu, best, k);
-      const float c = pk + sigma * (lane < K ? Ps[k * K + lane] : 0.f);
-      if (c > bv) { bv = c; bk = k; }             // strict: the lower predecessor on ties
+    for (int k0 = 0; k0 < K; k0 += 8) {           // eight predecessors' scores in flight:
+      // 200 x 15 slots x 8, 9.8 -> 8.3 us cold against one at a time
+      float c[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = k0 + u;
+        const float pk = __shfl_sync(0xffffffffu, best, k & 31);
+        c[u] = pk + sigma * (lane < K && k < K ? Ps[k * K + lane] : 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u)                 // strict: the lower predecessor on ties
+        if (k0 + u < K && c[u] > bv) { bv = c[u]; bk = k0 + u; }
     }
     if (lane < K) back[s * K + lane] = (uint8_t)bk;
     best = lane < K ? bv : -INFINITY;
