@@ -790,7 +790,8 @@ lilicorr_status_t lilicorr_topk_lse_merge(const void* partials, int P, int rows,
   if (rows == 0) return LILICORR_OK;
   if (!partials || !ids || !logp || !lse) return LILICORR_ERR_ARG;
   if (reinterpret_cast<uintptr_t>(partials) & 7) return LILICORR_ERR_ARG;
-  return launch_topk_merge(partials, P, rows, K, ids, logp, lse, status, stream);
+  const size_t rb = topk_partial_bytes(K);
+  return launch_topk_merge(partials, rb * rows, rb, P, rows, K, ids, logp, lse, status, stream);
 }
 
 size_t lilicorr_lm_head_topk_workspace_bytes(int rows, int H, int V, int K) {

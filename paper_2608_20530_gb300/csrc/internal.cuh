@@ -246,15 +246,16 @@ __device__ __forceinline__ float key_value(uint64_t k) {
 __device__ __forceinline__ int32_t key_id(uint64_t k) {
   return (int32_t)(0xFFFFFFFFu - (uint32_t)k);
 }
-// LM-head projection fused with step (1) (lm_head.cu): records [P][rows] in ws, then merged
+// LM-head projection fused with step (1) (lm_head.cu): records [rows][P] in ws, then merged
 bool lm_head_supported(int rows, int H, int V, int K);
 size_t lm_head_records_bytes(int rows, int V, int K);
 lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, int rows, int H,
                                       int V, int K, void* recs, int32_t* ids, float* logp,
                                       float* lse, uint32_t* status, cudaStream_t st);
-// merge P shards' records [P][rows][topk_partial_bytes(K)] into the final outputs
-lilicorr_status_t launch_topk_merge(const void* partials, int P, int rows, int K, int32_t* ids,
-                                    float* logp, float* lse, uint32_t* status, cudaStream_t st);
+// merge P partial records per row, record p of row r at partials + p * ld_p + r * ld_row
+lilicorr_status_t launch_topk_merge(const void* partials, size_t ld_p, size_t ld_row, int P,
+                                    int rows, int K, int32_t* ids, float* logp, float* lse,
+                                    uint32_t* status, cudaStream_t st);
 
 // Generic linear layer C = act(A W^T + bias [+ bias_rows[m / rows_per_bias]]) [+ residual].
 enum { ACT_NONE = 0, ACT_SILU = 1 };

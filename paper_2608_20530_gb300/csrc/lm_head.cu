@@ -217,9 +217,9 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
       }
     }
     if (valid && !abort_flag) {
-      // this CTA's partial record of row grow: record index n_first (one per CTA of
-      // the row block), rows of the record set in order
-      unsigned char* rec = recs + ((size_t)n_first * sh.rows + grow) * topk_partial_bytes(K);
+      // this CTA's partial record of row grow: a row's records lie side by side, one per CTA
+      // of the row block
+      unsigned char* rec = recs + ((size_t)grow * per + n_first) * topk_partial_bytes(K);
       float* rf = reinterpret_cast<float*>(rec);
       int32_t* ri = reinterpret_cast<int32_t*>(rec + 8 + 4 * (size_t)K);
       rf[0] = m_run;
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
       float gs = 0.f;
       for (int w = 0; w < 4; ++w)
         if (red_m[w][j] != -INFINITY) gs += red_s[w][j] * ex2_approx((red_m[w][j] - gm) * LH_LOG2E);
-      unsigned char* rec = recs + ((size_t)blockIdx.x * R + j) * topk_partial_bytes(K);
+      unsigned char* rec = recs + ((size_t)j * gridDim.x + blockIdx.x) * topk_partial_bytes(K);
       float* rf = reinterpret_cast<float*>(rec);
       int32_t* ri = reinterpret_cast<int32_t*>(rec + 8 + 4 * (size_t)K);
       rf[0] = gm;
@@ -557,7 +557,8 @@ lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, i
     const int grid = lm_head_rows_grid(V);
     LL_TRY(launch_k(lm_head_rows_kernel, grid, LH_THREADS, LS_SMEM, st, mw, mh, sh,
                     static_cast<unsigned char*>(recs), status));
-    return launch_topk_merge(recs, grid, rows, K, ids, logp, lse, status, st);
+    return launch_topk_merge(recs, topk_partial_bytes(K), grid * topk_partial_bytes(K), grid, rows,
+                             K, ids, logp, lse, status, st);
   }
   static bool configured[64] = {false};
   LL_TRY(allow_max_dynamic_smem(lm_head_topk_kernel, configured));
@@ -569,7 +570,9 @@ lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, i
   const int grid = lm_head_grid(rows, V);
   LL_TRY(launch_k(lm_head_topk_kernel, grid, LH_THREADS, LH_SMEM, st, ma, mw, sh,
                   static_cast<unsigned char*>(recs), status));
-  return launch_topk_merge(recs, grid / sh.tiles_m, rows, K, ids, logp, lse, status, st);
+  const int per = grid / sh.tiles_m;
+  return launch_topk_merge(recs, topk_partial_bytes(K), per * topk_partial_bytes(K), per, rows, K,
+                           ids, logp, lse, status, st);
 }
 
 }  // namespace lilicorr
