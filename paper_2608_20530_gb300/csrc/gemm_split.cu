@@ -292,28 +292,8 @@ lilicorr_status_t launch_split(const GemmArgs& g, int S, cudaStream_t st) {
   sa.g = g;
   sa.S = S;
   sa.w_const = g.w_const;
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(S, ceil_div(g.N, BN), ceil_div(g.M, 128));
-  cfg.blockDim = SP_THREADS;
-  cfg.dynamicSmemBytes = SpCfg<BN>::SMEM;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = S;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_split_kernel<BN>, ma, mw, sa);
-  count_launch();
-  if (e != cudaSuccess) {
-    (void)cudaGetLastError();
-    return LILICORR_ERR_CUDA;
-  }
-  return LILICORR_OK;
+  return launch_cluster_k(gemm_split_kernel<BN>, dim3(S, ceil_div(g.N, BN), ceil_div(g.M, 128)),
+                          SP_THREADS, SpCfg<BN>::SMEM, S, st, ma, mw, sa);
 }
 
 int split_tiles(const GemmArgs& g, int bn) { return ceil_div(g.M, 128) * ceil_div(g.N, bn); }

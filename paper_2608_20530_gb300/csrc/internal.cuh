@@ -64,6 +64,34 @@ lilicorr_status_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   return LILICORR_OK;
 }
 
+// launch_k as a grid of thread-block clusters of `cluster` CTAs along x.
+template <typename... KArgs, typename... Args>
+lilicorr_status_t launch_cluster_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                   int cluster, cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+  count_launch();
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    return LILICORR_ERR_CUDA;
+  }
+  return LILICORR_OK;
+}
+
 // Wait for the preceding launch on the stream to complete and its writes to be visible
 // (a no-op when the kernel was not launched as a dependent), then let the next launch
 // on the stream start its own setup.
