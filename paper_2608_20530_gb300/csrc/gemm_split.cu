@@ -37,10 +37,6 @@ constexpr uint32_t SP_A_BYTES = 128 * SP_BK * 2;
 constexpr long long SP_WAIT = 4000000000ll;
 constexpr float SP_RMS_EPS = 1e-6f;
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t local, uint32_t rank) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));

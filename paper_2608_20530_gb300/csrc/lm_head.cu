@@ -289,57 +289,6 @@ constexpr uint32_t LP_CHUNK = LH_BM * LH_BK * 2;        // 128 rows x 64, A and 
 constexpr uint32_t LP_HALF = LP_CH * LP_CHUNK;          // one operand's bytes of a stage
 constexpr size_t LP_SMEM = 1024 + (size_t)LP_STAGES * 2 * LP_HALF;
 
-__device__ __forceinline__ void lp_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// this CTA's shared-memory address seen in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t lp_map(const void* p, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-  return r;
-}
-// TMA copy of 128 rows x LP_CH chunks into this CTA whose bytes count on a barrier of either CTA
-// of the pair
-__device__ __forceinline__ void lp_load(void* dst, const CUtensorMap* map, uint32_t bar, int row,
-                                        int chunk) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(chunk), "r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ void lp_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-// arrive on the barrier at this offset in both CTAs once the pair's products so far are done
-__device__ __forceinline__ void lp_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;" ::"r"(smem_u32(bar)),
-      "h"((uint16_t)3)
-      : "memory");
-}
-// bounded wait that also acquires what the peer CTA released
-__device__ __forceinline__ bool lp_wait(uint64_t* bar, uint32_t parity) {
-  const long long t0 = clock64();
-  for (;;) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if (clock64() - t0 > LH_WAIT) return false;
-  }
-}
-
 __global__ void __launch_bounds__(LH_THREADS, 1)
     lm_head_pair_kernel(const __grid_constant__ CUtensorMap mapA,
                         const __grid_constant__ CUtensorMap mapW, LhShape sh,
@@ -374,16 +323,10 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(&tmem_base)),
-                 "r"(LH_TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
+  if (warp == 1) pair_tmem_alloc(&tmem_base, LH_TMEM_COLS);
   tc_fence_before();
   __syncthreads();
-  lp_cluster_sync();                                    // both CTAs' barriers are initialised
+  cluster_sync();                                    // both CTAs' barriers are initialised
   tc_fence_after();
   const uint32_t tmem = tmem_base;
   pdl_wait();
@@ -398,21 +341,21 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
         for (int i = 0; i < nk; ++i, ++g) {
           const int s = (int)(g % LP_STAGES);
           const uint32_t ph = (g / LP_STAGES) & 1u;
-          if (!lp_wait(&empty[s], ph ^ 1u)) {
+          if (!mbar_wait_cluster(&empty[s], ph ^ 1u, LH_WAIT)) {
             abort_flag = 1;
             break;
           }
           // a copy of the second CTA may complete before the first expects it: the phase
           // cannot end without the first CTA's arrival
-          const uint32_t bar = lp_map(&full[s], 0);
+          const uint32_t bar = peer_map(&full[s], 0);
           if (rank == 0) mbar_expect_tx(&full[s], 4 * LP_HALF);
-          lp_load(sA + (size_t)s * LP_HALF, &mapA, bar, m0, i * LP_CH);
-          lp_load(sB + (size_t)s * LP_HALF, &mapW, bar, n0, i * LP_CH);
+          pair_load_3d(sA + (size_t)s * LP_HALF, &mapA, bar, 0, m0, i * LP_CH);
+          pair_load_3d(sB + (size_t)s * LP_HALF, &mapW, bar, 0, n0, i * LP_CH);
         }
       }
       // the last commits arrive here from the first CTA: none may be under way at the exit
       for (uint32_t j = g > LP_STAGES ? g - LP_STAGES : 0; j < g && !abort_flag; ++j)
-        if (!lp_wait(&empty[j % LP_STAGES], (j / LP_STAGES) & 1u)) abort_flag = 1;
+        if (!mbar_wait_cluster(&empty[j % LP_STAGES], (j / LP_STAGES) & 1u, LH_WAIT)) abort_flag = 1;
     }
   } else if (warp == 1) {
     // ---- MMA issuer: the first CTA's lane, for both
@@ -421,7 +364,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
       uint32_t g = 0, lt = 0;
       for (int nt = n_first; nt < sh.tiles_n && !abort_flag; nt += per, ++lt) {
         const uint32_t acc = lt & 1u;
-        if (!lp_wait(&acc_empty[acc], ((lt >> 1) & 1u) ^ 1u)) {
+        if (!mbar_wait_cluster(&acc_empty[acc], ((lt >> 1) & 1u) ^ 1u, LH_WAIT)) {
           abort_flag = 1;
           break;
         }
@@ -430,7 +373,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
         for (int i = 0; i < nk; ++i, ++g) {
           const int s = (int)(g % LP_STAGES);
           const uint32_t ph = (g / LP_STAGES) & 1u;
-          if (!lp_wait(&full[s], ph)) {
+          if (!mbar_wait_cluster(&full[s], ph, LH_WAIT)) {
             abort_flag = 1;
             break;
           }
@@ -441,11 +384,11 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
             const uint64_t bd = smem_desc(sB + (size_t)s * LP_HALF + c * LP_CHUNK);
 #pragma unroll
             for (int k = 0; k < LH_BK / 16; ++k)
-              lp_mma(d, ad + 2ull * k, bd + 2ull * k, idesc, (i > 0 || c > 0 || k > 0) ? 1u : 0u);
+              pair_mma_bf16(d, ad + 2ull * k, bd + 2ull * k, idesc, (i > 0 || c > 0 || k > 0) ? 1u : 0u);
           }
-          lp_commit(&empty[s]);
+          pair_commit(&empty[s]);
         }
-        lp_commit(&acc_full[acc]);
+        pair_commit(&acc_full[acc]);
       }
     }
   } else {
@@ -454,19 +397,16 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
     const int row = q * 32 + lane;
     const int grow = (2 * mt + (int)rank) * LH_BM + row;
     const bool valid = grow < sh.rows;
-    const uint32_t back0 = lp_map(&acc_empty[0], 0), back1 = lp_map(&acc_empty[1], 0);
+    const uint32_t back0 = peer_map(&acc_empty[0], 0), back1 = peer_map(&acc_empty[1], 0);
     LhRow st;
     uint32_t lt = 0;
     for (int nt = n_first; nt < sh.tiles_n; nt += per, ++lt) {
       const uint32_t acc = lt & 1u;
-      if (!abort_flag && !lp_wait(&acc_full[acc], (lt >> 1) & 1u)) abort_flag = 1;
+      if (!abort_flag && !mbar_wait_cluster(&acc_full[acc], (lt >> 1) & 1u, LH_WAIT)) abort_flag = 1;
       tc_fence_after();
       lh_fold_tile(tmem + ((uint32_t)(q * 32) << 16) + acc * LH_BN, nt * LH_BN, sh,
                    valid && !abort_flag, row, s_list, st, [&] {
-                     if (lane == 0)
-                       asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
-                                        acc ? back1 : back0)
-                                    : "memory");
+                     if (lane == 0) mbar_arrive_mapped(acc ? back1 : back0);
                    });
     }
     if (valid && !abort_flag)
@@ -486,12 +426,10 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
     }
     __syncthreads();
   }
-  lp_cluster_sync();
+  cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(LH_TMEM_COLS)
-                 : "memory");
+    pair_tmem_dealloc(tmem, LH_TMEM_COLS);
   }
 }
 

@@ -141,12 +141,6 @@ __device__ __forceinline__ bool mbar_wait_cluster_sleep(uint64_t* bar, uint32_t 
     if (clock64() - t0 > limit) return false;
   return true;
 }
-// all threads of all CTAs of the cluster
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;"
-               ::: "memory");
-}
-
 // q / k / v of one head: [128 rows][32] 16-bit values, 64-byte rows, pieces XOR-swizzled
 // by row pair so that ldmatrix over 8 consecutive rows touches 8 distinct bank groups
 __device__ __forceinline__ uint32_t qkv_off(int row, int piece) {
