@@ -375,6 +375,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (leader && !abort_flag && n0 + c * CH < N && !(FOLD && ep.no_c)) {
           tma_store_2d(&mapC, stg, n0 + c * CH, m0);
           tma_store_wait_read_le1();         // the other buffer is free for the next chunk
+        } else if (leader) {
+          // a chunk past N stores nothing, so the last store may still be reading the buffer
+          // that the next chunk takes
+          tma_store_wait_read_all();
         }
       }
       if (FOLD && !OUT_BF16 && ep.c2 && m < M)
