@@ -68,16 +68,26 @@ struct TcEpilogue {
   const float* ss_in; int ss_slots; float ss_scale;
 };
 
+// KCH: 64-wide chunks of Kd per stage, brought by one copy per operand where Kd is whole stages. bf16 outputs at BN = 256 are bound by the copies and stores of an SM (16 copies of a
+// tile's 384 KB and four stores, about 0.25 us each), so their stages are 128-wide: 65,536 x
+// 1536 x 512 95 -> 90 us cold, x 1024 x 512 with SiLU 76 -> 73, x 512 x 1024 69 -> 59. fp32
+// outputs keep three 64-wide stages beside their residual chunks: two made 65,536 x 512 x 1024
+// 91 -> 107 us, and residual chunks five instead of two ahead changed nothing (85 -> 84).
 template <int BN, bool OUT_BF16>
 struct TcCfg {
-  static constexpr int STAGES = BN >= 256 ? 3 : 4;
-  static constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2;
-  static constexpr uint32_t B_BYTES = BN * TC_BK * 2;
+  static constexpr int KCH = BN >= 256 && OUT_BF16 ? 2 : 1;
+  static constexpr int STAGES = BN >= 256 ? (OUT_BF16 ? 2 : 3) : 4;
+  static constexpr uint32_t A_CHUNK = TC_BM * TC_BK * 2, B_CHUNK = BN * TC_BK * 2;
+  static constexpr uint32_t A_BYTES = KCH * A_CHUNK;
+  static constexpr uint32_t B_BYTES = KCH * B_CHUNK;
   static constexpr int CH = OUT_BF16 ? 64 : 32;        // output columns per 128-byte chunk
   static constexpr int NCH = BN / CH;
   static constexpr uint32_t TMEM_COLS = 2 * BN;         // two accumulators
   static constexpr size_t RING = (size_t)STAGES * (A_BYTES + B_BYTES);
-  static constexpr size_t SMEM = 1024 + RING + 4 * (size_t)CHUNK_BYTES + 3 * BN * sizeof(float);
+  // staging chunks, and for fp32 outputs residual chunks and the folded norm's gains and t row
+  static constexpr size_t SMEM = 1024 + RING + (OUT_BF16 ? 2 : 4) * (size_t)CHUNK_BYTES +
+                                 (OUT_BF16 ? 1 : 3) * BN * sizeof(float);
+  static_assert(SMEM + 256 <= SMEM_PER_BLOCK_MAX, "dynamic beside the static barriers");
 };
 
 // FOLD: the instantiation with the folded-RMSNorm epilogue (c2 / ss_out, ss_in); the
@@ -88,17 +98,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                    const __grid_constant__ CUtensorMap mapW,
                    const __grid_constant__ CUtensorMap mapC,
                    const __grid_constant__ CUtensorMap mapR, TcEpilogue ep, int M, int N, int Kd,
-                   uint32_t* status, long long wait_limit, int starve) {
+                   uint32_t* status, long long wait_limit, int starve, int k3) {
   using Cfg = TcCfg<BN, OUT_BF16>;
-  constexpr int S = Cfg::STAGES, CH = Cfg::CH, NCH = Cfg::NCH;
+  constexpr int S = Cfg::STAGES, CH = Cfg::CH, NCH = Cfg::NCH, KCH = Cfg::KCH;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* sA = smem;
   uint8_t* sB = smem + S * Cfg::A_BYTES;
   uint8_t* s_out = smem + Cfg::RING;                   // 2 staging chunks
-  uint8_t* s_res = s_out + 2 * CHUNK_BYTES;            // 2 residual chunks
-  float* s_bias = reinterpret_cast<float*>(s_res + 2 * CHUNK_BYTES);
+  uint8_t* s_res = s_out + 2 * CHUNK_BYTES;            // 2 residual chunks (fp32 outputs)
+  float* s_bias = reinterpret_cast<float*>(OUT_BF16 ? s_res : s_res + 2 * CHUNK_BYTES);
   float* s_gain = s_bias + BN;                         // c2_gain of the tile's columns
   float* s_t = s_gain + BN;                            // c3_t of the tile's sequence
   __shared__ __align__(8) uint64_t full[S], empty[S], acc_full[2], acc_empty[2], res_full[2];
@@ -108,7 +118,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tiles_n = (N + BN - 1) / BN;
   const int tiles = ((M + TC_BM - 1) / TC_BM) * tiles_n;
-  const int nk = (Kd + TC_BK - 1) / TC_BK;
+  const int chunks = (Kd + TC_BK - 1) / TC_BK, nk = (chunks + KCH - 1) / KCH;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -150,9 +160,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             abort_flag = 1;
             break;
           }
-          mbar_expect_tx(&full[s], Cfg::A_BYTES + Cfg::B_BYTES);
-          tma_load_2d(sA + (size_t)s * Cfg::A_BYTES, &mapA, &full[s], i * TC_BK, m0);
-          tma_load_2d(sB + (size_t)s * Cfg::B_BYTES, &mapW, &full[s], i * TC_BK, n0);
+          const int here = min(KCH, chunks - i * KCH);     // the last stage may be short
+          mbar_expect_tx(&full[s], here * (Cfg::A_CHUNK + Cfg::B_CHUNK));
+          uint8_t* a = sA + (size_t)s * Cfg::A_BYTES;
+          uint8_t* w = sB + (size_t)s * Cfg::B_BYTES;
+          if (KCH > 1 && k3) {
+            tma_load_3d(a, &mapA, &full[s], 0, m0, i * KCH);
+            tma_load_3d(w, &mapW, &full[s], 0, n0, i * KCH);
+          } else {
+#pragma unroll
+            for (int c = 0; c < KCH; ++c) {
+              if (c >= here) break;
+              tma_load_2d(a + c * Cfg::A_CHUNK, &mapA, &full[s], (i * KCH + c) * TC_BK, m0);
+              tma_load_2d(w + c * Cfg::B_CHUNK, &mapW, &full[s], (i * KCH + c) * TC_BK, n0);
+            }
+          }
         }
       }
     }
@@ -177,11 +199,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             break;
           }
           tc_fence_after();
-          const uint64_t ad = smem_desc(sA + (size_t)s * Cfg::A_BYTES);
-          const uint64_t bd = smem_desc(sB + (size_t)s * Cfg::B_BYTES);
 #pragma unroll
-          for (int k = 0; k < TC_BK / 16; ++k)
-            mma_bf16(d, ad + 2ull * k, bd + 2ull * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
+          for (int c = 0; c < KCH; ++c) {
+            if (i * KCH + c >= chunks) break;
+            const uint64_t ad = smem_desc(sA + (size_t)s * Cfg::A_BYTES + c * Cfg::A_CHUNK);
+            const uint64_t bd = smem_desc(sB + (size_t)s * Cfg::B_BYTES + c * Cfg::B_CHUNK);
+#pragma unroll
+            for (int k = 0; k < TC_BK / 16; ++k)
+              mma_bf16(d, ad + 2ull * k, bd + 2ull * k, idesc, (i > 0 || c > 0 || k > 0) ? 1u : 0u);
+          }
           mma_commit(&empty[s]);
         }
         mma_commit(&acc_full[acc]);
@@ -203,7 +229,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       mbar_expect_tx(bar, CHUNK_BYTES);
       tma_load_2d(s_res + (k & 1u) * CHUNK_BYTES, &mapR, bar, n0 + c * CH, m0);
     };
-    if (ep.has_residual && leader && (int)blockIdx.x < tiles) issue_res(blockIdx.x, 0, 0);
+    if (!OUT_BF16 && ep.has_residual && leader && (int)blockIdx.x < tiles) issue_res(blockIdx.x, 0, 0);
     // folded RMSNorm of the input rows: the row's sums of squares, loaded a tile ahead
     float4 ssn[SS_LD / 4];
     auto load_ss = [&](int t) {
@@ -226,8 +252,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       epi_bar();                                  // s_bias free again
       // c3: when the tile's rows all belong to one sequence, its c3_t row goes to shared
       // memory with the gains; otherwise every thread reads its own row's
-      const int tb0 = (FOLD && ep.c3) ? min(m0, M - 1) / ep.c3_rows_per : 0;
-      const bool t_shared = (FOLD && ep.c3) && min(m0 + TC_BM - 1, M - 1) / ep.c3_rows_per == tb0;
+      const int tb0 = (FOLD && !OUT_BF16 && ep.c3) ? min(m0, M - 1) / ep.c3_rows_per : 0;
+      const bool t_shared = (FOLD && !OUT_BF16 && ep.c3) && min(m0 + TC_BM - 1, M - 1) / ep.c3_rows_per == tb0;
       for (int j = threadIdx.x - 64; j < BN; j += EPI_THREADS) {
         s_bias[j] = (ep.bias && n0 + j < N) ? ep.bias[n0 + j] : 0.f;
         if (FOLD && !OUT_BF16 && ep.c2) s_gain[j] = n0 + j < N ? ep.c2_gain[n0 + j] : 0.f;
@@ -253,7 +279,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       for (int c = 0; c < NCH; ++c, ++cc) {
         const uint32_t b = cc & 1u;
         // prefetch the next chunk's residual (its buffer was drained a chunk ago)
-        if (ep.has_residual && leader && !abort_flag) {
+        if (!OUT_BF16 && ep.has_residual && leader && !abort_flag) {
           if (c + 1 < NCH) issue_res(t, c + 1, cc + 1);
           else if (t + (int)gridDim.x < tiles) issue_res(t + gridDim.x, 0, cc + 1);
         }
@@ -279,7 +305,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(&acc_empty[acc]);
         }
-        if (ep.has_residual && !abort_flag &&
+        if (!OUT_BF16 && ep.has_residual && !abort_flag &&
             !mbar_wait(&res_full[b], (cc >> 1) & 1u, wait_limit))
           abort_flag = 1;
 #pragma unroll
@@ -299,7 +325,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
               x.x = silu_f(x.x); x.y = silu_f(x.y); x.z = silu_f(x.z); x.w = silu_f(x.w);
             }
           }
-          if (ep.has_residual) {            // fp32 output only: 4 columns = 16 bytes
+          if (!OUT_BF16 && ep.has_residual) {            // 4 columns = 16 bytes
             const float4 rr = *reinterpret_cast<const float4*>(
                 s_res + b * CHUNK_BYTES + swz(row, (half * HC + j) >> 2));
             x.x += rr.x; x.y += rr.y; x.z += rr.z; x.w += rr.w;
@@ -416,8 +442,15 @@ lilicorr_status_t launch_bn(const GemmArgs& g, cudaStream_t st) {
   CUtensorMap ma, mw, mc, mr;
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   const CUtensorMapDataType f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-  if (!make_map(&ma, g.A, bf, 2, g.M, g.Kd, g.lda, TC_BM, TC_BK)) return LILICORR_ERR_CUDA;
-  if (!make_map(&mw, g.W, bf, 2, g.N, g.Kd, g.ldw, BN, TC_BK)) return LILICORR_ERR_CUDA;
+  const bool k3 = Cfg::KCH > 1 && g.Kd % (Cfg::KCH * TC_BK) == 0;
+  auto map = [&](CUtensorMap* m, const void* base, int rows, int ld, int box) {
+    if (!k3) return make_map(m, base, bf, 2, rows, g.Kd, ld, box, TC_BK);
+    const uint64_t dims[3] = {TC_BK, (uint64_t)rows, (uint64_t)(g.Kd / TC_BK)};
+    const uint64_t strides[3] = {2, (uint64_t)ld * 2, TC_BK * 2};
+    const uint32_t b3[3] = {TC_BK, (uint32_t)box, (uint32_t)Cfg::KCH};
+    return make_map_nd(m, base, bf, 3, dims, strides, b3);
+  };
+  if (!map(&ma, g.A, g.M, g.lda, TC_BM) || !map(&mw, g.W, g.N, g.ldw, BN)) return LILICORR_ERR_CUDA;
   if (g.residual) {
     if (!make_map(&mr, g.residual, f32, 4, g.M, g.N, g.ldr, TC_BM, 32)) return LILICORR_ERR_CUDA;
   }
@@ -449,7 +482,7 @@ lilicorr_status_t launch_bn(const GemmArgs& g, cudaStream_t st) {
   const int grid = tiles < num_sms() ? tiles : num_sms();
   const long long wait = g.wait_limit > 0 ? g.wait_limit : WAIT_LIMIT_CYCLES;
   LL_TRY(launch_k(gemm_tc_kernel<BN, OUT_BF16, FOLD>, grid, TC_THREADS, Cfg::SMEM, st, ma, mw, mc, mr, ep,
-                  g.M, g.N, g.Kd, g.status, wait, g.test_starve));
+                  g.M, g.N, g.Kd, g.status, wait, g.test_starve, (int)k3));
   return LILICORR_OK;
 }
 
