@@ -7,8 +7,8 @@
 // each multiplies its part of Kd into its own tensor memory, parks the 128 x BN partial sums
 // in its shared memory, and after a cluster barrier every CTA adds up the S partials of the
 // rows r, r + S, r + 2S, ... (distributed shared memory, in rank order, so the result is the
-// same on every call) and runs the epilogue on them. S is the largest power of two that keeps
-// at least two chunks per CTA and the grid within the SMs.
+// same on every call) and runs the epilogue on them. gemm_split_ways says how S
+// follows from the sizes.
 //
 // Roles: warp 0 (one lane) streams 128 x 64 tiles of A and BN x 64 tiles of W by TMA (128-byte
 // swizzle, four stages), warp 1 issues tcgen05.mma (M = 128, N = BN), warps 4-7 drain the
@@ -298,14 +298,21 @@ int split_tiles(const GemmArgs& g, int bn) { return ceil_div(g.M, 128) * ceil_di
 
 int gemm_split_ss_slots(int N) { return ceil_div(N, 64); }
 
-// CTAs per tile: as many as leave each at least two chunks of Kd and the grid on the GPU at
-// once; 0 where the tiles alone fill more than half of the SMs (the persistent kernel's case).
+// CTAs per tile (0: too many tiles, the persistent kernel's case). Measured back to back, us for
+// S = 1 / 2 / 4 / 8 and the persistent kernel:
+//   120 x 1024 x 1024   8.6  6.4  4.9  5.6   7.7        64 x 256 x 4096   20.8 11.8  7.2  5.5  20.4
+//   120 x 3072 x 1024   8.7  6.5  6.2 11.8   7.8       360 x 1024 x 2560  15.0  9.6  8.1 13.8  14.3
+//   480 x 1024 x 1024   8.8  6.5  6.6 13.4   7.9       480 x 1024 x 2048  13.0  8.7  7.8 14.3  12.2
+//   960 x 1024 x 1024   8.7  7.6 12.6 25.1   8.0      1024 x 512 x 512     6.7  5.5  6.0 13.0   5.7
+// So S doubles while the CTAs fit one an SM and keep two chunks of Kd each, or two an SM and keep
+// four; eight ways, whose clusters are harder to place, only where Kd is long.
 int gemm_split_ways(const GemmArgs& g) {
-  const int tiles = split_tiles(g, 64), nk = ceil_div(g.Kd, SP_BK);
-  if (2 * tiles > num_sms()) return 0;
+  const int tiles = split_tiles(g, 64), nk = ceil_div(g.Kd, SP_BK), sms = num_sms();
   int S = 1;
-  while (S < 8 && 2 * S * tiles <= num_sms() && nk >= 4 * S) S *= 2;
-  return S;
+  while (S < 4 && ((2 * S * tiles <= sms && nk >= 4 * S) || (S * tiles <= sms && nk >= 8 * S)))
+    S *= 2;
+  if (S == 4 && 8 * tiles <= sms && nk >= 40) S = 8;
+  return S > 1 || 2 * tiles <= sms ? S : 0;
 }
 
 bool gemm_split_supported(const GemmArgs& g) {
