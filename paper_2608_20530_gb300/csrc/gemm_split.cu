@@ -111,16 +111,44 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
     tma_load_2d(sA + (size_t)s * SP_A_BYTES, &mapA, &full[s], (kc0 + i) * SP_BK, m0);
   };
   const bool producer = warp == 0 && lane == 0;
-  if (producer && sa.w_const)
-    for (int i = 0; i < pre; ++i) load_w(i);
+  if (producer) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapA)) : "memory");
+    if (sa.w_const)
+      for (int i = 0; i < pre; ++i) load_w(i);
+  }
+  // this thread's columns in the reduction, and what it adds to them
+  constexpr int TPR = BN / 4;                       // threads per row
+  const int c = (threadIdx.x % TPR) * 4, n = n0 + c;
+  const int rows = min(128, g.M - m0);
+  const bool col_ok = n < g.N;                      // N is a multiple of 8
+  float4 bias = make_float4(0.f, 0.f, 0.f, 0.f), gain = bias;
+  auto load_vectors = [&] {
+    if (g.bias && col_ok)
+      bias = make_float4(g.bias[n], g.bias[n + 1], g.bias[n + 2], g.bias[n + 3]);
+    if (g.c2 && col_ok)
+      gain = make_float4(g.c2_gain[n], g.c2_gain[n + 1], g.c2_gain[n + 2], g.c2_gain[n + 3]);
+  };
+  if (sa.w_const) load_vectors();                   // constant with the weights
   pdl_wait();
+
+  if (producer)
+    for (int i = 0; i < pre; ++i) {
+      if (!sa.w_const) load_w(i);
+      load_a(i);
+    }
+  if (!sa.w_const) load_vectors();
+  // the residual of this thread's first rows, asked for before the products
+  constexpr int RP = 4;                             // rounds of the reduction at S = 2
+  float4 res[RP];
+  auto row_of = [&](int i) { return rank + S * (threadIdx.x / TPR) + i * S * (SP_THREADS / TPR); };
+#pragma unroll
+  for (int i = 0; i < RP; ++i)
+    res[i] = g.residual && col_ok && row_of(i) < rows
+                 ? *reinterpret_cast<const float4*>(g.residual + (size_t)(m0 + row_of(i)) * g.ldr + n)
+                 : make_float4(0.f, 0.f, 0.f, 0.f);
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int i = 0; i < pre; ++i) {
-        if (!sa.w_const) load_w(i);
-        load_a(i);
-      }
       for (int i = pre; i < kcn; ++i) {
         if (!mbar_wait(&empty[i % SP_STAGES], ((i / SP_STAGES) & 1) ^ 1, SP_WAIT)) {
           abort_flag = 1;
@@ -172,37 +200,29 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
   __syncwarp();
   cluster_sync();                      // every CTA's partials are in place
 
-  // ---- reduction and epilogue: BN / 4 threads per row, rows rank, rank + S, ...
-  constexpr int TPR = BN / 4;
-  const int c = (threadIdx.x % TPR) * 4, n = n0 + c;
-  const int rows = min(128, g.M - m0);
-  const bool col_ok = n < g.N;                      // N is a multiple of 8
-  float4 bias = make_float4(0.f, 0.f, 0.f, 0.f), gain = bias;
-  if (g.bias && col_ok)
-    bias = make_float4(g.bias[n], g.bias[n + 1], g.bias[n + 2], g.bias[n + 3]);
-  if (g.c2 && col_ok)
-    gain = make_float4(g.c2_gain[n], g.c2_gain[n + 1], g.c2_gain[n + 2], g.c2_gain[n + 3]);
+  // ---- reduction and epilogue: rows rank, rank + S, ...
   const float ss_scale = 1.0f / (float)(g.ss_dim > 0 ? g.ss_dim : g.Kd);
-  // the threads of a row stay together, so the loop runs the same number of rounds for all
-  for (int base = 0; base < 128; base += S * (SP_THREADS / TPR)) {
-    const int r = base + rank + S * (threadIdx.x / TPR);
+  // the threads of a row stay together: all run the same number of rounds
+  const int rounds = 128 / (S * (SP_THREADS / TPR));
+  auto sum_row = [&](int i) {                       // the S partials of a row, in rank order
+    const int r = row_of(i);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r >= rows) return v;
+    if (S == 1) return *reinterpret_cast<const float4*>(part + r * PLD + c);
+    const uint32_t local = smem_u32(part + r * PLD + c);
+    float4 t[8];                                    // every partial in flight, then the sum
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+      if (p < S) t[p] = ld_cluster_f4(local, p);
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+      if (p < S) { v.x += t[p].x; v.y += t[p].y; v.z += t[p].z; v.w += t[p].w; }
+    return v;
+  };
+  auto finish_row = [&](int i, const float4& v, const float4& rr) {
+    const int r = row_of(i);
     const bool live = r < rows;
     const int m = m0 + r;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (live) {
-      const uint32_t local = smem_u32(part + r * PLD + c);
-      if (S == 1) {
-        v = *reinterpret_cast<const float4*>(part + r * PLD + c);
-      } else {
-        float4 t[8];                                // every partial in flight, then the sum
-#pragma unroll
-        for (int p = 0; p < 8; ++p)
-          if (p < S) t[p] = ld_cluster_f4(local, p);
-#pragma unroll
-        for (int p = 0; p < 8; ++p)
-          if (p < S) { v.x += t[p].x; v.y += t[p].y; v.z += t[p].z; v.w += t[p].w; }
-      }
-    }
     float rs = 1.f;
     if (g.ss_in) {                                  // folded RMSNorm of the input rows
       float s = 0.f;
@@ -227,10 +247,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
         x.x = silu_f(x.x); x.y = silu_f(x.y); x.z = silu_f(x.z); x.w = silu_f(x.w);
       }
     }
-    if (g.residual && out) {
-      const float4 rr = *reinterpret_cast<const float4*>(g.residual + (size_t)m * g.ldr + n);
-      x.x += rr.x; x.y += rr.y; x.z += rr.z; x.w += rr.w;
-    }
+    if (g.residual) { x.x += rr.x; x.y += rr.y; x.z += rr.z; x.w += rr.w; }
     if (out && g.C) {
       if (g.c_dt == LILICORR_BF16)
         *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(g.C) + (size_t)m * g.ldc + n) =
@@ -256,7 +273,22 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
       for (int o = TPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (live && threadIdx.x % TPR == 0) g.ss_out[(size_t)m * SS_LD + blockIdx.y] = s;
     }
-  }
+  };
+  float4 sum[RP];
+#pragma unroll
+  for (int i = 0; i < RP; ++i)
+    if (i < rounds) sum[i] = sum_row(i);
+  // the peers' partials are read: the barrier that lets them leave is met behind the stores
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < RP; ++i)
+    if (i < rounds) finish_row(i, sum[i], res[i]);
+  for (int i = RP; i < rounds; ++i)                 // S = 1: the other rounds read theirs now
+    finish_row(i, sum_row(i),
+               g.residual && col_ok && row_of(i) < rows
+                   ? *reinterpret_cast<const float4*>(g.residual + (size_t)(m0 + row_of(i)) * g.ldr + n)
+                   : make_float4(0.f, 0.f, 0.f, 0.f));
 
   // ---- teardown: no CTA leaves while a peer may still read its partials
   if (abort_flag) {
@@ -269,7 +301,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
     __syncthreads();
   }
   __syncwarp();
-  cluster_sync();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, BN);
