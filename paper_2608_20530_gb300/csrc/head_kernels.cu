@@ -474,13 +474,14 @@ target_norm_kernel(const T* __restrict__ Tin, int n_tgt, int H, const float* __r
 }
 
 // ----------------------------------------------------------------------------- nodes
-// One CTA per slot row r = b*L + s. For candidate k (Sec. 3.2; App. A):
+// CTA (r, part): slot row r = b*L + s, one part of the columns. For candidate k (Sec. 3.2; App. A):
 //   c1 = SiLU(W_c1 f_k + b_c1)   (first layer of the confidence network; the second
 //                                 layer is a linear launch that adds into x)
 //   x  = fold[id_k] + hproj[r] + slot[s] + rank[k]
 // with f_k = [logp_k, exp(logp_k), logp_0 - logp_k, k / (K-1), 1{k = 0}].
 template <typename TC1>
-__global__ void node_build_kernel(int L, int K, int D, int V, const int32_t* __restrict__ ids,
+__global__ void node_build_kernel(int L, int K, int D, int cols, int V,
+                                  const int32_t* __restrict__ ids,
                                   const float* __restrict__ logp, const float* __restrict__ fold,
                                   const float* __restrict__ hproj, const float* __restrict__ slot,
                                   const float* __restrict__ rank, const float* __restrict__ w1,
@@ -489,13 +490,15 @@ __global__ void node_build_kernel(int L, int K, int D, int V, const int32_t* __r
   pdl_wait();
   __shared__ float f[LILICORR_MAX_K][LILICORR_N_CONF];
   __shared__ int sid[LILICORR_MAX_K];
-  extern __shared__ __align__(16) float s_w[];     // [N_CONF][D] = W_c1^T, then b_c1 [D]
+  extern __shared__ __align__(16) float s_w[];     // [N_CONF][cols] = W_c1^T, then b_c1 [cols]
   const int r = blockIdx.x;
   const int s = r % L;
-  for (int i = threadIdx.x; i < D; i += blockDim.x) {
+  const int c0 = blockIdx.y * cols, nc = min(cols, D - c0);    // this CTA's columns
+  for (int i = threadIdx.x; i < nc; i += blockDim.x) {
 #pragma unroll
-    for (int j = 0; j < LILICORR_N_CONF; ++j) s_w[j * D + i] = w1[i * LILICORR_N_CONF + j];
-    s_w[LILICORR_N_CONF * D + i] = b1[i];
+    for (int j = 0; j < LILICORR_N_CONF; ++j)
+      s_w[j * cols + i] = w1[(c0 + i) * LILICORR_N_CONF + j];
+    s_w[LILICORR_N_CONF * cols + i] = b1[c0 + i];
   }
   if (threadIdx.x < K) {
     const int k = threadIdx.x;
@@ -514,10 +517,10 @@ __global__ void node_build_kernel(int L, int K, int D, int V, const int32_t* __r
     sid[k] = id;
   }
   __syncthreads();
-  const int D4 = D / 4;
+  const int nc4 = nc / 4;
 #pragma unroll 2
-  for (int i = threadIdx.x; i < K * D4; i += blockDim.x) {
-    const int k = i / D4, n = (i % D4) * 4;
+  for (int i = threadIdx.x; i < K * nc4; i += blockDim.x) {
+    const int k = i / nc4, nl = (i % nc4) * 4, n = c0 + nl;
     const size_t node = (size_t)r * K + k;
     const float4 fo = *reinterpret_cast<const float4*>(fold + (size_t)sid[k] * D + n);
     const float4 hp = *reinterpret_cast<const float4*>(hproj + (size_t)r * D + n);
@@ -529,10 +532,10 @@ __global__ void node_build_kernel(int L, int K, int D, int V, const int32_t* __r
     o.z = fo.z + hp.z + sl.z + rk.z;
     o.w = fo.w + hp.w + sl.w + rk.w;
     *reinterpret_cast<float4*>(x + node * D + n) = o;
-    float4 z = *reinterpret_cast<const float4*>(s_w + LILICORR_N_CONF * D + n);
+    float4 z = *reinterpret_cast<const float4*>(s_w + LILICORR_N_CONF * cols + nl);
 #pragma unroll
     for (int j = 0; j < LILICORR_N_CONF; ++j) {
-      const float4 w = *reinterpret_cast<const float4*>(s_w + j * D + n);
+      const float4 w = *reinterpret_cast<const float4*>(s_w + j * cols + nl);
       const float fj = f[k][j];
       z.x = fmaf(w.x, fj, z.x);
       z.y = fmaf(w.y, fj, z.y);
@@ -836,15 +839,20 @@ lilicorr_status_t launch_node_build(const lilicorr_head* h, int B, const int32_t
   const lilicorr_head_desc& d = h->desc;
   if (B == 0) return LILICORR_OK;
   const float* fold = static_cast<const float*>(h->fold);
+  // Few slot rows: their columns over several CTAs, at least 128 each, until two an SM (one
+  // request of 15 slots x 8 candidates x 1024: 15 CTAs of eight rounds of gathers, 14.1 us cold,
+  // to 120 of one, 5.8). Many rows keep one CTA each, which stages the confidence weights once.
+  const int parts = max(1, min(ceil_div(2 * num_sms(), B * d.L), d.D / 128));
+  const int cols = ceil_div(ceil_div(d.D, parts), 4) * 4;
+  const dim3 grid(B * d.L, ceil_div(d.D, cols));
+  const size_t smem = sizeof(float) * (LILICORR_N_CONF + 1) * cols;
   if (c1_dt == LILICORR_F32)
-    LL_TRY(launch_k(node_build_kernel<float>, B * d.L, 256, sizeof(float) * (LILICORR_N_CONF + 1) * d.D, st, d.L, d.K, d.D, d.V, ids, logp, fold, hproj,
-                                                      h->slot, h->rank, h->conf1_w, h->conf1_b,
-                                                      static_cast<float*>(c1), x, status));
-  else
-    LL_TRY(launch_k(node_build_kernel<__nv_bfloat16>, B * d.L, 256, sizeof(float) * (LILICORR_N_CONF + 1) * d.D, st, 
-        d.L, d.K, d.D, d.V, ids, logp, fold, hproj, h->slot, h->rank, h->conf1_w, h->conf1_b,
-        static_cast<__nv_bfloat16*>(c1), x, status));
-  return LILICORR_OK;
+    return launch_k(node_build_kernel<float>, grid, 256, smem, st, d.L, d.K, d.D, cols, d.V, ids,
+                    logp, fold, hproj, h->slot, h->rank, h->conf1_w, h->conf1_b,
+                    static_cast<float*>(c1), x, status);
+  return launch_k(node_build_kernel<__nv_bfloat16>, grid, 256, smem, st, d.L, d.K, d.D, cols, d.V,
+                  ids, logp, fold, hproj, h->slot, h->rank, h->conf1_w, h->conf1_b,
+                  static_cast<__nv_bfloat16*>(c1), x, status);
 }
 
 lilicorr_status_t launch_rmsnorm(const float* x, int M, int D, const float* gain, void* y,
