@@ -835,11 +835,8 @@ lilicorr_status_t lilicorr_embed_in_out(const lilicorr_head* head, int B, const 
   const lilicorr_head_desc& d = head->desc;
   LL_TRY(run_head(head, B, ids, logp, drafter_hidden, target_hidden, ws, w, stream));
   const int N = B * d.L * d.K;
-  const float* oi = at<float>(ws, w.oi);
-  LL_TRY(launch_unit_rows(oi, N, d.d, 2 * d.d, out_vec, d.d, stream));
-  LL_TRY(launch_unit_rows(oi + d.d, N, d.d, 2 * d.d, in_vec, d.d, stream));
-  LL_TRY(launch_unit_rows(at<float>(ws, w.anc), B, d.d, d.d, anchor_out, d.d, stream));
-  return LILICORR_OK;
+  return launch_unit_vectors(at<float>(ws, w.oi), at<float>(ws, w.anc), N, B, d.d, out_vec, in_vec,
+                             anchor_out, stream);
 }
 
 lilicorr_status_t lilicorr_pair_scores(int B, int L, int K, int d, const float* out_vec,

@@ -398,8 +398,8 @@ extern int g_attn_umma;
 lilicorr_status_t launch_fusion_input(const float* x, int B, int LK, int D, const float* gain,
                                       const float* t, void* fin, lilicorr_dtype_t dt,
                                       cudaStream_t st);
-lilicorr_status_t launch_unit_rows(const float* src, int rows, int n, int ld_src, float* dst,
-                                   int ld_dst, cudaStream_t st);
+lilicorr_status_t launch_unit_vectors(const float* oi, const float* anc, int N, int B, int d,
+                                      float* out, float* in, float* anchor, cudaStream_t st);
 
 // (3)+(4) pair scores and greedy walk (pair_walk.cu)
 struct PairWalkArgs {
