@@ -68,21 +68,23 @@ struct TcEpilogue {
   const float* ss_in; int ss_slots; float ss_scale;
 };
 
-// KCH: 64-wide chunks of Kd per stage, brought by one copy per operand where Kd is whole stages. bf16 outputs at BN = 256 are bound by the copies and stores of an SM (16 copies of a
+// KCH: 64-wide chunks of Kd per stage, brought by one copy per operand where Kd is whole stages.
+// bf16 outputs at BN = 256 (and 192) are bound by the copies and stores of an SM (16 copies of a
 // tile's 384 KB and four stores, about 0.25 us each), so their stages are 128-wide: 65,536 x
 // 1536 x 512 95 -> 90 us cold, x 1024 x 512 with SiLU 76 -> 73, x 512 x 1024 69 -> 59. fp32
 // outputs keep three 64-wide stages beside their residual chunks: two made 65,536 x 512 x 1024
 // 91 -> 107 us, and residual chunks five instead of two ahead changed nothing (85 -> 84).
 template <int BN, bool OUT_BF16>
 struct TcCfg {
-  static constexpr int KCH = BN >= 256 && OUT_BF16 ? 2 : 1;
-  static constexpr int STAGES = BN >= 256 ? (OUT_BF16 ? 2 : 3) : 4;
+  static constexpr int KCH = BN >= 192 && OUT_BF16 ? 2 : 1;
+  static constexpr int STAGES = BN >= 192 ? (OUT_BF16 ? 2 : 3) : 4;
   static constexpr uint32_t A_CHUNK = TC_BM * TC_BK * 2, B_CHUNK = BN * TC_BK * 2;
   static constexpr uint32_t A_BYTES = KCH * A_CHUNK;
   static constexpr uint32_t B_BYTES = KCH * B_CHUNK;
   static constexpr int CH = OUT_BF16 ? 64 : 32;        // output columns per 128-byte chunk
   static constexpr int NCH = BN / CH;
-  static constexpr uint32_t TMEM_COLS = 2 * BN;         // two accumulators
+  static constexpr uint32_t ACC_COLS = BN > 128 ? 256 : BN;   // an accumulator's place
+  static constexpr uint32_t TMEM_COLS = 2 * ACC_COLS;   // two accumulators, a power of two
   static constexpr size_t RING = (size_t)STAGES * (A_BYTES + B_BYTES);
   // staging chunks, and for fp32 outputs residual chunks and the folded norm's gains and t row
   static constexpr size_t SMEM = 1024 + RING + (OUT_BF16 ? 2 : 4) * (size_t)CHUNK_BYTES +
@@ -190,7 +192,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           break;
         }
         tc_fence_after();
-        const uint32_t d = tmem + acc * BN;
+        const uint32_t d = tmem + acc * Cfg::ACC_COLS;
         for (int i = 0; i < nk; ++i, ++g) {
           const int s = (int)(g % S);
           const uint32_t ph = (g / S) & 1u;
@@ -286,7 +288,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int cl = c * CH + half * HC;         // first column of this thread's part
         float v[HC];
         {
-          const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + acc * BN + cl;
+          const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + acc * Cfg::ACC_COLS + cl;
           if constexpr (HC == 32) {
             uint32_t r[32];
             tmem_ld32(ta, r);
@@ -486,19 +488,28 @@ lilicorr_status_t launch_bn(const GemmArgs& g, cudaStream_t st) {
   return LILICORR_OK;
 }
 
-// Column tile: the widest of 256/128/64 that still gives every SM a tile.
+// Column tile: the width whose rounds over the SMs cost least, a round about its width plus 100
+// columns' worth of fill, drain and epilogue. The line before (256 where that gives every SM a
+// tile, else 128, else 64) left rounds half empty: 2880 rows x N = 1024 are two rounds of 128
+// columns or one of 192. Whole networks of 120 nodes a request, width 1024, before and with
+// this rule: 8 requests 166 -> 161 us, 12 207 -> 195, 16 221 -> 212, 24 296 -> 270, 32 323 -> 316, 40
+// and 64 as before; width 512: 32 requests 166 -> 162, 100 366 -> 343, 128 428 -> 418.
 int tc_column_tile(int M, int N) {
-  const int mt = ceil_div(M, TC_BM);
-  const int sms = num_sms();
-  if (N >= 256 && mt * ceil_div(N, 256) >= sms) return 256;
-  if (N >= 128 && mt * ceil_div(N, 128) >= sms / 2) return 128;
-  return 64;
+  const int mt = ceil_div(M, TC_BM), sms = num_sms();
+  int best = 64, cost = INT32_MAX;
+  for (int bn : {256, 192, 128, 64}) {
+    if (bn > 64 && N < bn) continue;
+    const int c = ceil_div((long long)mt * ceil_div(N, bn), sms) * (bn + 100);
+    if (c < cost) { best = bn; cost = c; }
+  }
+  return best;
 }
 
 template <bool OUT_BF16, bool FOLD>
 lilicorr_status_t launch_out(const GemmArgs& g, cudaStream_t st) {
   const int bn = tc_column_tile(g.M, g.N);
   if (bn == 256) return launch_bn<256, OUT_BF16, FOLD>(g, st);
+  if (bn == 192) return launch_bn<192, OUT_BF16, FOLD>(g, st);
   if (bn == 128) return launch_bn<128, OUT_BF16, FOLD>(g, st);
   return launch_bn<64, OUT_BF16, FOLD>(g, st);
 }
