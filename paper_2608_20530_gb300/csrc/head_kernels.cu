@@ -68,7 +68,7 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p, int r, int rows,
 
 // VEC: rows of both operands in whole aligned groups of four elements
 template <typename TA, typename TW, typename TC, bool VEC>
-__global__ void __launch_bounds__(G_THREADS, 2) gemm_simt_kernel(GemmArgs g) {
+__global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g) {
   pdl_wait();
   constexpr int LDT = GB_M + 4, KG = GB_K / G_GROUPS;
   static_assert(GB_M == GB_N && GB_M * GB_K == 8 * G_THREADS, "two groups of four a thread");
