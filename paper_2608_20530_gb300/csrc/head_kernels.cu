@@ -227,12 +227,14 @@ __device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
 }
 
 template <typename TA, typename TW, typename TC, int MB>
-__global__ void __launch_bounds__(SK_THREADS) gemm_skinny_kernel(GemmArgs g) {
+__global__ void __launch_bounds__(SK_THREADS) gemm_skinny_kernel(const GemmArgs g0, const GemmArgs g1) {
   pdl_wait();
+  const GemmArgs& g = blockIdx.z ? g1 : g0;         // one launch may hold two products
   __shared__ float red[SK_THREADS / 32][MB * SK_NB];
   const TA* A = static_cast<const TA*>(g.A);
   const TW* W = static_cast<const TW*>(g.W);
   const int n0 = blockIdx.x * SK_NB, m0 = blockIdx.y * MB;
+  if (n0 >= g.N) return;
   const int nb = min(SK_NB, g.N - n0), mb = min(MB, g.M - m0);
   float acc[MB][SK_NB];
 #pragma unroll
@@ -311,8 +313,9 @@ struct GrCfg {
   static constexpr int WS = KC + 16 / (int)sizeof(TW);        // so 8 lanes' 16-byte reads differ in bank
 };
 template <typename TW, typename TC>
-__global__ void __launch_bounds__(GR_THREADS) gemm_rows_kernel(GemmArgs g) {
+__global__ void __launch_bounds__(GR_THREADS) gemm_rows_kernel(const GemmArgs g0, const GemmArgs g1) {
   pdl_wait();
+  const GemmArgs& g = blockIdx.z ? g1 : g0;         // one launch may hold two products
   using Cfg = GrCfg<TW>;
   constexpr int KC = Cfg::KC, AS = Cfg::AS, WS = Cfg::WS;
   constexpr int WV = 16 / (int)sizeof(TW);                    // weights per 16-byte piece
@@ -321,6 +324,7 @@ __global__ void __launch_bounds__(GR_THREADS) gemm_rows_kernel(GemmArgs g) {
   const float* A = static_cast<const float*>(g.A);
   const TW* W = static_cast<const TW*>(g.W);
   const int m0 = blockIdx.y * GR_M, n0 = blockIdx.x * GR_N;
+  if (n0 >= g.N) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = n0 + lane, r0 = 2 * warp;
   float acc0 = 0.f, acc1 = 0.f;
@@ -374,24 +378,24 @@ __global__ void __launch_bounds__(GR_THREADS) gemm_rows_kernel(GemmArgs g) {
 }
 
 template <typename TA, typename TW, int MB>
-lilicorr_status_t skinny_dispatch_m(const GemmArgs& g, cudaStream_t st) {
-  dim3 grid(ceil_div(g.N, SK_NB), ceil_div(g.M, MB));
-  if (g.c_dt == LILICORR_F32) LL_TRY(launch_k(gemm_skinny_kernel<TA, TW, float, MB>, grid, SK_THREADS, 0, st, g));
-  else LL_TRY(launch_k(gemm_skinny_kernel<TA, TW, __nv_bfloat16, MB>, grid, SK_THREADS, 0, st, g));
-  return LILICORR_OK;
+lilicorr_status_t skinny_dispatch_m(const GemmArgs& g, const GemmArgs* g1, cudaStream_t st) {
+  const dim3 grid(ceil_div(g1 ? max(g.N, g1->N) : g.N, SK_NB), ceil_div(g.M, MB), g1 ? 2 : 1);
+  const GemmArgs& h = g1 ? *g1 : g;
+  if (g.c_dt == LILICORR_F32)
+    return launch_k(gemm_skinny_kernel<TA, TW, float, MB>, grid, SK_THREADS, 0, st, g, h);
+  return launch_k(gemm_skinny_kernel<TA, TW, __nv_bfloat16, MB>, grid, SK_THREADS, 0, st, g, h);
 }
 // rows per CTA: one per sequence-level row (M = 1), four for a few, else sixteen
 template <typename TA, typename TW>
-lilicorr_status_t skinny_dispatch_c(const GemmArgs& g, dim3 grid, cudaStream_t st) {
-  (void)grid;
-  if (g.M == 1) return skinny_dispatch_m<TA, TW, 1>(g, st);
-  if (g.M <= 4) return skinny_dispatch_m<TA, TW, 4>(g, st);
-  return skinny_dispatch_m<TA, TW, SK_MB>(g, st);
+lilicorr_status_t skinny_dispatch_c(const GemmArgs& g, const GemmArgs* g1, cudaStream_t st) {
+  if (g.M == 1) return skinny_dispatch_m<TA, TW, 1>(g, g1, st);
+  if (g.M <= 4) return skinny_dispatch_m<TA, TW, 4>(g, g1, st);
+  return skinny_dispatch_m<TA, TW, SK_MB>(g, g1, st);
 }
 template <typename TA>
-lilicorr_status_t skinny_dispatch_w(const GemmArgs& g, dim3 grid, cudaStream_t st) {
-  if (g.w_dt == LILICORR_F32) return skinny_dispatch_c<TA, float>(g, grid, st);
-  return skinny_dispatch_c<TA, __nv_bfloat16>(g, grid, st);
+lilicorr_status_t skinny_dispatch_w(const GemmArgs& g, const GemmArgs* g1, cudaStream_t st) {
+  if (g.w_dt == LILICORR_F32) return skinny_dispatch_c<TA, float>(g, g1, st);
+  return skinny_dispatch_c<TA, __nv_bfloat16>(g, g1, st);
 }
 
 // ----------------------------------------------------------------------------- target state
@@ -817,24 +821,28 @@ bool gemm_rows_supported(const GemmArgs& g) {
          (reinterpret_cast<uintptr_t>(g.W) & 15) == 0;
 }
 
-lilicorr_status_t launch_gemm_rows(const GemmArgs& g, cudaStream_t st) {
-  if (!gemm_rows_supported(g)) return LILICORR_ERR_SHAPE;
-  const dim3 grid(ceil_div(g.N, GR_N), ceil_div(g.M, GR_M));
+lilicorr_status_t launch_gemm_rows(const GemmArgs& g, cudaStream_t st, const GemmArgs* g1) {
+  if (!gemm_rows_supported(g) || (g1 && !gemm_rows_supported(*g1))) return LILICORR_ERR_SHAPE;
+  const dim3 grid(ceil_div(g1 ? max(g.N, g1->N) : g.N, GR_N), ceil_div(g.M, GR_M), g1 ? 2 : 1);
+  const GemmArgs& h = g1 ? *g1 : g;
   if (g.w_dt == LILICORR_F32) {
-    if (g.c_dt == LILICORR_F32) return launch_k(gemm_rows_kernel<float, float>, grid, GR_THREADS, 0, st, g);
-    return launch_k(gemm_rows_kernel<float, __nv_bfloat16>, grid, GR_THREADS, 0, st, g);
+    if (g.c_dt == LILICORR_F32)
+      return launch_k(gemm_rows_kernel<float, float>, grid, GR_THREADS, 0, st, g, h);
+    return launch_k(gemm_rows_kernel<float, __nv_bfloat16>, grid, GR_THREADS, 0, st, g, h);
   }
   if (g.c_dt == LILICORR_F32)
-    return launch_k(gemm_rows_kernel<__nv_bfloat16, float>, grid, GR_THREADS, 0, st, g);
-  return launch_k(gemm_rows_kernel<__nv_bfloat16, __nv_bfloat16>, grid, GR_THREADS, 0, st, g);
+    return launch_k(gemm_rows_kernel<__nv_bfloat16, float>, grid, GR_THREADS, 0, st, g, h);
+  return launch_k(gemm_rows_kernel<__nv_bfloat16, __nv_bfloat16>, grid, GR_THREADS, 0, st, g, h);
 }
 
-lilicorr_status_t launch_gemm_skinny(const GemmArgs& g, cudaStream_t st) {
+lilicorr_status_t launch_gemm_skinny(const GemmArgs& g, cudaStream_t st, const GemmArgs* g1) {
   if (g.M == 0 || g.N == 0) return LILICORR_OK;
-  if ((g.Kd % 8) || (g.lda % 8) || (g.ldw % 8)) return launch_gemm_simt(g, st);
-  dim3 grid(ceil_div(g.N, SK_NB), ceil_div(g.M, SK_MB));
-  if (g.a_dt == LILICORR_F32) return skinny_dispatch_w<float>(g, grid, st);
-  return skinny_dispatch_w<__nv_bfloat16>(g, grid, st);
+  if ((g.Kd % 8) || (g.lda % 8) || (g.ldw % 8) || (g1 && g1->ldw % 8)) {
+    LL_TRY(launch_gemm_simt(g, st));
+    return g1 ? launch_gemm_simt(*g1, st) : LILICORR_OK;
+  }
+  if (g.a_dt == LILICORR_F32) return skinny_dispatch_w<float>(g, g1, st);
+  return skinny_dispatch_w<__nv_bfloat16>(g, g1, st);
 }
 
 lilicorr_status_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st) {

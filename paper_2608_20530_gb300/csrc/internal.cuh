@@ -196,8 +196,7 @@ struct lilicorr_head {
   // the projections that do not depend on the top-K pass run on two side streams that
   // fork from and join the caller's stream (fork/join nodes under graph capture)
   cudaStream_t side, side2;
-  cudaEvent_t ev_fork, ev_join, ev_join2, ev_t, ev_hid;  // ev_t: the target state t is ready
-                                                          // ev_hid: the drafter states are
+  cudaEvent_t ev_fork, ev_join, ev_join2;   // ev_join: side, ev_join2: side2
   void* pool;                 // one device allocation holding everything below
   size_t pool_bytes;
   // matrices in head dtype; vectors and tables in fp32
@@ -316,10 +315,13 @@ struct GemmArgs {
 constexpr int SS_LD = 16;  // floats per row of a folded-RMSNorm sums-of-squares buffer
 int gemm_tc_ss_slots(int M, int N);
 lilicorr_status_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
-lilicorr_status_t launch_gemm_skinny(const GemmArgs& g, cudaStream_t st);   // M <= 64
+// `second`: another product of the same rows, types and Kd in the same launch
+lilicorr_status_t launch_gemm_skinny(const GemmArgs& g, cudaStream_t st,
+                                     const GemmArgs* second = nullptr);   // M <= 64
 // fp32 activations, per-sequence row counts (16 x 32 output blocks, no K split)
 bool gemm_rows_supported(const GemmArgs& g);
-lilicorr_status_t launch_gemm_rows(const GemmArgs& g, cudaStream_t st);
+lilicorr_status_t launch_gemm_rows(const GemmArgs& g, cudaStream_t st,
+                                   const GemmArgs* second = nullptr);
 bool gemm_tc_operands_ok(const GemmArgs& g);   // what both TMA-fed kernels below ask
 bool gemm_tc_supported(const GemmArgs& g);
 lilicorr_status_t launch_gemm_tc(const GemmArgs& g, cudaStream_t st);
