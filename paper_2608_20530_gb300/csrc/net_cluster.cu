@@ -935,11 +935,28 @@ __global__ void __launch_bounds__(NC_THREADS, 1)
         if (me != 0) {
           if (tid == 0) mbar_arrive_peer(pe.at(NC_CC - me, sh.prb));   // to rank 0
         } else if (xg_wait(sh.prb, sh.abort)) {
-          for (int i = tid; i < npr; i += NC_RW) {
-            float v = pr[i];
+          // four records' twelve remote words in flight a thread (one record at a time waited
+          // for a remote load three times in a row at 16 slots x 8 candidates)
+          constexpr int RU = 4;
+          for (int i0 = tid; i0 < npr; i0 += RU * NC_RW) {
+            float v[RU][NC_CC];
 #pragma unroll
-            for (int q = 1; q < NC_CC; ++q) v += ld_peer_f32(pe.at(q, pr + i));
-            pr[i] = v;
+            for (int u = 0; u < RU; ++u) {
+              const int i = i0 + u * NC_RW;
+              if (i >= npr) continue;
+              v[u][0] = pr[i];
+#pragma unroll
+              for (int q = 1; q < NC_CC; ++q) v[u][q] = ld_peer_f32(pe.at(q, pr + i));
+            }
+#pragma unroll
+            for (int u = 0; u < RU; ++u) {
+              const int i = i0 + u * NC_RW;
+              if (i >= npr) continue;
+              float sum = v[u][0];
+#pragma unroll
+              for (int q = 1; q < NC_CC; ++q) sum += v[u][q];
+              pr[i] = sum;
+            }
           }
           rw_bar();
           const float an = fmaxf(sqrtf(pr[o_an]), 1e-12f);
@@ -957,9 +974,11 @@ __global__ void __launch_bounds__(NC_THREADS, 1)
             a.tl.A[(size_t)b * K + k] = v;
           }
           rw_bar();
+          uint8_t* best = reinterpret_cast<uint8_t*>(s_ss);      // the norms are in the record
+          walk::best_of_rows(pr + o_ad, pr, L, K, best, tid, NC_RW);
+          rw_bar();
           if (wr == 0) {
-            walk::walk_sequence(pr + o_ad, pr, b, L, K, nullptr, s_slot);
-            __syncwarp();
+            walk::follow(best, L, K, s_slot);
             for (int s = lane; s < L; s += 32) {
               const size_t o = (size_t)b * L + s;
               const int c = s_slot[s];

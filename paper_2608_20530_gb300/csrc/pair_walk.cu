@@ -16,9 +16,9 @@
 // of a sequence to finish (atomic ticket, nobody waits) loads the sequence's
 // scores into shared memory and walks them.
 // walk_kernel: grid B, the walk alone over given scores.
-// The walk is one warp: per step one butterfly over the candidates' lanes carries the best
-// (ties to the lower index) and the second-best score, for the choice and the
-// best-minus-second margin; the tokens are gathered for all slots after the walk. In Viterbi mode (App. E) the same warp computes the exact
+// The walk follows a table of every score row's best candidate (walk.cuh); margins (best minus
+// second-best score of a step) and tokens are formed for all slots after it. In Viterbi mode
+// (App. E) one warp computes the exact
 // maximiser of the path score g(c) = sigma (A[c_1] + sum_s P[s-1, c_{s-1}, c_s]) instead:
 // lane k keeps the best score of a path ending at candidate k, one sweep over the slots
 // records each lane's best predecessor (ties to the lower index) in shared memory, and
@@ -107,19 +107,33 @@ __device__ void viterbi_sequence(const float* A, const float* P, int b, int L, i
   }
 }
 
+// Walk the scores A, P of sequence b (the whole CTA calls): the path, then choices, tokens and
+// margins of all slots at once. back: [L * K] bytes (the Viterbi predecessors, or each score
+// row's best candidate), path: [L] bytes, both in shared memory.
 __device__ __forceinline__ void run_walk(const PairWalkArgs& a, const float* A, const float* P,
                                          int b, uint8_t* back, uint8_t* path) {
-  if (a.walk_mode == LILICORR_WALK_VITERBI)
-    viterbi_sequence(A, P, b, a.L, a.K, a.sigma, a.path_score, back, path);
-  else
-    walk_sequence(A, P, b, a.L, a.K, a.margin, path);
+  const bool greedy = a.walk_mode != LILICORR_WALK_VITERBI;
+  if (greedy) {
+    best_of_rows(A, P, a.L, a.K, back, threadIdx.x, PW_THREADS);
+    __syncthreads();
+  }
+  if ((threadIdx.x >> 5) != 0) return;
+  if (greedy) follow(back, a.L, a.K, path);
+  else viterbi_sequence(A, P, b, a.L, a.K, a.sigma, a.path_score, back, path);
   __syncwarp();
-  const int lane = threadIdx.x & 31;
-  for (int s = lane; s < a.L; s += 32) {        // choices and tokens, all slots at once
+  const int lane = threadIdx.x & 31, K = a.K;
+  for (int s = lane; s < a.L; s += 32) {
     const size_t o = (size_t)b * a.L + s;
     const int c = path[s];
     if (a.choice) a.choice[o] = c;
-    if (a.tokens) a.tokens[o] = a.ids[o * a.K + c];
+    if (a.tokens) a.tokens[o] = a.ids[o * K + c];
+    if (greedy && a.margin) {                   // best minus second-best of the step's row
+      const float* row = s == 0 ? A : P + ((size_t)(s - 1) * K + path[s - 1]) * K;
+      float second = -INFINITY;
+      for (int k = 0; k < K; ++k)
+        if (k != c) second = fmaxf(second, row[k]);
+      a.margin[o] = K > 1 ? row[c] - second : INFINITY;
+    }
   }
 }
 
@@ -145,10 +159,8 @@ __device__ __forceinline__ void walk_after_pairs(const PairWalkArgs& a, float* s
     A = sm;
     P = sm + K;
   }
-  if ((threadIdx.x >> 5) == 0) {
-    run_walk(a, A, P, b, s_back, s_path);
-    if ((threadIdx.x & 31) == 0) a.counters[b] = 0u;   // leave the workspace reusable
-  }
+  run_walk(a, A, P, b, s_back, s_path);
+  if (threadIdx.x == 0) a.counters[b] = 0u;     // leave the workspace reusable
 }
 
 // pair_block_kernel's staging: rows padded to a multiple of 4 per slot, row stride d + 4.
@@ -473,7 +485,7 @@ __global__ void __launch_bounds__(PW_THREADS) walk_kernel(PairWalkArgs a) {
     A = sm;
     P = sm + K;
   }
-  if ((threadIdx.x >> 5) == 0) run_walk(a, A, P, b, s_back, s_path);
+  run_walk(a, A, P, b, s_back, s_path);
 }
 
 }  // namespace
