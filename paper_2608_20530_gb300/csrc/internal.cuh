@@ -153,6 +153,10 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+__device__ __forceinline__ float dot4(const float4& x, const float4& y, float acc) {
+  return fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, acc))));
+}
+
 __device__ __forceinline__ float silu_f(float z) { return z / (1.0f + __expf(-z)); }
 // two floats as a bf16 pair (round to nearest even), lo in the low half
 __device__ __forceinline__ uint32_t bf16_pack2(float lo, float hi) {

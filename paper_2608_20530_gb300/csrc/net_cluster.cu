@@ -901,31 +901,46 @@ __global__ void __launch_bounds__(NC_THREADS, 1)
         float* pr = reinterpret_cast<float*>(sm + OFF_RING);
         const int npair = (L - 1) * K * K, o_ad = npair, o_on = o_ad + K, o_in = o_on + LK,
                   o_an = o_in + LK, npr = o_an + 1;
-        for (int idx = tid; idx < npair; idx += NC_RW) {
-          const int s = idx / (K * K), j = (idx / K) % K, k = idx % K;
-          const int n1 = s * K + j, n2 = (s + 1) * K + k;
-          float dot = 0.f;
+        // pair dots in 2 x 2 blocks, so a piece read from shared memory feeds two products
+        const int K2 = (K + 1) >> 1, nblk = (L - 1) * K2 * K2;
+        for (int idx = tid; idx < nblk; idx += NC_RW) {
+          const int s = idx / (K2 * K2), rem = idx - s * K2 * K2;
+          const int j0 = 2 * (rem / K2), k0 = 2 * (rem % K2);
+          const int j1 = min(j0 + 1, K - 1), k1 = min(k0 + 1, K - 1);   // an odd K repeats its last
+          float d00 = 0.f, d01 = 0.f, d10 = 0.f, d11 = 0.f;
 #pragma unroll 4
           for (int p = 0; p < 16; ++p) {
-            const float4 o = *stg_at(n1, p), i = *stg_at(n2, 16 + p);
-            dot = fmaf(o.x, i.x, fmaf(o.y, i.y, fmaf(o.z, i.z, fmaf(o.w, i.w, dot))));
+            const float4 o0 = *stg_at(s * K + j0, p), o1 = *stg_at(s * K + j1, p);
+            const float4 i0 = *stg_at((s + 1) * K + k0, 16 + p), i1 = *stg_at((s + 1) * K + k1, 16 + p);
+            d00 = dot4(o0, i0, d00);
+            d01 = dot4(o0, i1, d01);
+            d10 = dot4(o1, i0, d10);
+            d11 = dot4(o1, i1, d11);
           }
-          pr[idx] = dot;
+          float* out = pr + s * K * K;
+          out[j0 * K + k0] = d00;
+          out[j0 * K + k1] = d01;               // a repeated row or column writes the same value
+          out[j1 * K + k0] = d10;
+          out[j1 * K + k1] = d11;
         }
-        for (int k = tid; k < K; k += NC_RW) {
-          const float* an = vec + V_ANC;
+        // the last warp, which has few blocks: anchor dots, a candidate's 16 pieces over the
+        // lanes that candidates leave free
+        if (wr == NC_RW / 32 - 1) {
+          int kp = 1;
+          while (kp < K) kp <<= 1;
+          const int k = lane & (kp - 1), parts = 32 / kp;
           float dot = 0.f;
-          for (int p = 0; p < 16; ++p) {
-            const float4 i = *stg_at(k, 16 + p);
-            dot = fmaf(an[4 * p], i.x, fmaf(an[4 * p + 1], i.y, fmaf(an[4 * p + 2], i.z, fmaf(an[4 * p + 3], i.w, dot))));
-          }
-          pr[o_ad + k] = dot;
+          if (k < K)
+            for (int p = lane / kp; p < 16; p += parts)
+              dot = dot4(*reinterpret_cast<const float4*>(vec + V_ANC + 4 * p), *stg_at(k, 16 + p), dot);
+          for (int o = kp; o < 32; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+          if (lane < K) pr[o_ad + lane] = dot;
         }
         if (cg == 0 && r < LK) {
           pr[o_on + r] = s_ss[r] + s_ss[NC_M + r];
           pr[o_in + r] = s_ss[2 * NC_M + r] + s_ss[3 * NC_M + r];
         }
-        if (wr == 0) {
+        if (wr == NC_RW / 32 - 2) {
           float q = 0.f;
           for (int c = lane; c < NC_SL; c += 32) q = fmaf(vec[V_ANC + c], vec[V_ANC + c], q);
           q = warp_sum(q);

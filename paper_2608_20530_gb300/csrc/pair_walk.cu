@@ -169,10 +169,6 @@ __host__ __device__ __forceinline__ size_t pb_smem_bytes(int K, int d) {
   return sizeof(float) * (size_t)2 * pb_rows(K) * (d + 4);
 }
 
-__device__ __forceinline__ float dot4(const float4& x, const float4& y, float acc) {
-  return fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, acc))));
-}
-
 // Dot products of the 4 x 4 block of rows x (xr..xr+3, the earlier slot) and y (yr..yr+3,
 // slot j) over the 16-byte columns f = split, split + step, ... within [f0, f1); the thread's
 // squared norms of those rows alongside when nx / ny are asked for.
