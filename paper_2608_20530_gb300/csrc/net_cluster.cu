@@ -82,8 +82,7 @@ constexpr uint32_t OFF_SSX = OFF_SS + 4 * NC_M * 4;
 constexpr uint32_t OFF_DIST = OFF_SSX + 2 * NC_CC * NC_M * 4;      // [8][127]
 constexpr uint32_t OFF_SAME = OFF_DIST + NC_NH * (2 * NC_MAX_L - 1) * 4;
 constexpr uint32_t OFF_SLOT = OFF_SAME + NC_NH * 4;                // [128]
-constexpr uint32_t OFF_IDS = OFF_SLOT + NC_M;                      // [128]
-constexpr uint32_t OFF_BAR = (OFF_IDS + NC_M * 4 + 63) & ~63u;
+constexpr uint32_t OFF_BAR = (OFF_SLOT + NC_M + 63) & ~63u;
 constexpr int N_DONE = 2 + 4 * NC_MAX_LAYERS + 1, N_READY = N_DONE, N_XG = 3 + 6 * NC_MAX_LAYERS;
 constexpr int X_C1 = N_XG - 1;            // exchange of the confidence MLP's first layer
 constexpr int N_W1F = NC_MAX_LAYERS;
@@ -489,7 +488,6 @@ __global__ void __launch_bounds__(NC_THREADS, 1)
   float* s_dist = reinterpret_cast<float*>(sm + OFF_DIST);
   float* s_same = reinterpret_cast<float*>(sm + OFF_SAME);
   uint8_t* s_slot = sm + OFF_SLOT;
-  int32_t* s_ids = reinterpret_cast<int32_t*>(sm + OFF_IDS);
   float* vec = reinterpret_cast<float*>(sm + OFF_VEC);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -598,14 +596,6 @@ __global__ void __launch_bounds__(NC_THREADS, 1)
       if (ok) {
         const int s = r / K, k = r % K;
         const size_t rk = ((size_t)b * L + s) * K;
-        if (cg == 0) {
-          int id = a.ids[rk + k];
-          if (id < 0 || id >= a.V) {                // an id outside the vocabulary: flag, read row 0
-            set_status(a.status, LILICORR_ERR_ARG);
-            id = 0;
-          }
-          s_ids[r] = id;
-        }
         const float lp = a.logp[rk + k], lp0 = a.logp[rk];
         f[0] = lp;
         f[1] = expf(lp);
@@ -623,21 +613,25 @@ __global__ void __launch_bounds__(NC_THREADS, 1)
         const int row = i / (NC_SL / 4), c = (i % (NC_SL / 4)) * 4;
         cp_async16(tab_at(sm, row, c), a.hproj + ((size_t)b * L + row) * NC_D + c0s + c);
       }
-      rw_bar();                                      // s_ids complete
-      for (int i = tid; i < LK * (NC_SL / 4); i += NC_RW) {
-        const int n = i / (NC_SL / 4), c = (i % (NC_SL / 4)) * 4;
-        cp_async16(fold_at(n, c), a.fold + (size_t)s_ids[n] * NC_D + c0s + c);
+      // every thread reads the ids of the nodes whose pieces it copies, all before the copies
+      constexpr int FT = NC_M * (NC_SL / 4) / NC_RW;         // pieces a thread
+      int32_t id[FT];
+#pragma unroll
+      for (int u = 0; u < FT; ++u) {
+        const int n = (tid + u * NC_RW) / (NC_SL / 4);
+        id[u] = n < LK ? a.ids[(size_t)b * LK + n] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < FT; ++u) {
+        const int i = tid + u * NC_RW, n = i / (NC_SL / 4), c = (i % (NC_SL / 4)) * 4;
+        if (n >= LK) continue;
+        if (id[u] < 0 || id[u] >= a.V) {            // an id outside the vocabulary: flag, read row 0
+          set_status(a.status, LILICORR_ERR_ARG);
+          id[u] = 0;
+        }
+        cp_async16(fold_at(n, c), a.fold + (size_t)id[u] * NC_D + c0s + c);
       }
       cp_async_wait_all();
-      rw_bar();
-      for (int i = tid; i < L * (NC_SL / 4); i += NC_RW) {   // S[s] = hproj + slot + b_c2
-        const int row = i / (NC_SL / 4), c = (i % (NC_SL / 4)) * 4;
-        float4 x = *reinterpret_cast<float4*>(tab_at(sm, row, c));
-        const float4 y = *reinterpret_cast<const float4*>(tab_at(sm, L + row, c));
-        const float4 z = *reinterpret_cast<const float4*>(vec + V_C2B + c);
-        x.x += y.x + z.x; x.y += y.y + z.y; x.z += y.z + z.z; x.w += y.w + z.w;
-        *reinterpret_cast<float4*>(tab_at(sm, row, c)) = x;
-      }
       rw_bar();
       {
         const int srow = ok ? r / K : 0, rrow = 2 * L + (ok ? r % K : 0);
@@ -646,8 +640,11 @@ __global__ void __launch_bounds__(NC_THREADS, 1)
         for (int u = 0; u < 4; ++u) {
           const int c = 16 * cg + 4 * u;
           const float4 x = *reinterpret_cast<const float4*>(fold_at(ok ? r : 0, c));
-          const float4 y = *reinterpret_cast<const float4*>(tab_at(sm, srow, c));
+          float4 y = *reinterpret_cast<const float4*>(tab_at(sm, srow, c));
+          const float4 ys = *reinterpret_cast<const float4*>(tab_at(sm, L + srow, c));
+          const float4 yb = *reinterpret_cast<const float4*>(vec + V_C2B + c);
           const float4 z = *reinterpret_cast<const float4*>(tab_at(sm, rrow, c));
+          y.x += ys.x + yb.x; y.y += ys.y + yb.y; y.z += ys.z + yb.z; y.w += ys.w + yb.w;
           v[4 * u] = ok ? x.x + y.x + z.x : 0.f;
           v[4 * u + 1] = ok ? x.y + y.y + z.y : 0.f;
           v[4 * u + 2] = ok ? x.z + y.z + z.z : 0.f;
@@ -889,7 +886,8 @@ __global__ void __launch_bounds__(NC_THREADS, 1)
       s_ss[cg * NC_M + r] = ss;                    // 32 columns' part of |o|^2 (cg < 2) or |i|^2
       rw_bar();
       const int dh = a.d2 / 2;
-      for (int row = wr; row < LK; row += NC_RW / 32)
+      // (the tail forms the scores itself: nothing reads the vectors then)
+      for (int row = wr; row < LK && !a.tail; row += NC_RW / 32)
         *reinterpret_cast<float4*>(a.oi + ((size_t)b * LK + row) * a.d2 + (lane < 16 ? 0 : dh) + c0s +
                                    4 * (lane & 15)) = *stg_at(row, lane);
       if (a.tail) {
