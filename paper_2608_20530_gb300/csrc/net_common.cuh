@@ -191,6 +191,7 @@ __device__ __forceinline__ uint32_t ex2_h2(uint32_t x) {
 __device__ __forceinline__ float2 h2_to_f2(uint32_t x) {
   return __half22float2(*reinterpret_cast<const __half2*>(&x));
 }
+constexpr uint32_t ONES_H2 = 0x3C003C00u;      // two fp16 ones
 // SiLU(z) = z sigmoid(z) = z (1 + tanh(z / 2)) / 2 for two values with one packed fp16
 // tanh (one MUFU operation per pair; the result feeds a bf16 operand, whose rounding is
 // coarser than the fp16 tanh)
@@ -255,7 +256,8 @@ __device__ __forceinline__ void st32f(uint32_t taddr, const float (&v)[32]) {
 
 // Attention core of one head (App. A: bidirectional attention over the L*K nodes with the
 // signed slot-distance and same-slot biases) for the 16 queries q0..q0+15 of one warp, in
-// blocks of KB (32 or 64) keys with an online softmax in log2 units; probabilities P = 2^(S - max) as
+// blocks of KB (32 or 64) keys with an online softmax in log2 units (its sums are one more product,
+// of P with ones: no unpacking, adding and shuffling of the probabilities); probabilities P = 2^(S - max) as
 // fp16 pairs (one MUFU operation per pair). q, k (bf16) and v (fp16) of the head are at qb,
 // qb + 8192 and qb + 16384 (qkv_off layout). s_slot: slot of each node; sd: the head's
 // distance bias (log2 units) indexed by sj - si; same_l2: its same-slot bias (log2 units).
@@ -276,7 +278,7 @@ __device__ __forceinline__ void head_attention(uint32_t qb, int LK, int K, const
     ldsm_x4(qb + qkv_off(q0 + (lane & 15), ks * 2 + (lane >> 4)), qa[ks]);
   const int i0 = q0 + g8, i1 = i0 + 8;
   const int si0 = s_slot[i0], si1 = s_slot[i1];
-  float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
+  float m0 = -INFINITY, m1 = -INFINITY, ol[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int nb = 0; nb < 4; ++nb) o[nb][0] = o[nb][1] = o[nb][2] = o[nb][3] = 0.f;
 #pragma unroll 1
@@ -338,8 +340,8 @@ __device__ __forceinline__ void head_attention(uint32_t qb, int LK, int K, const
     const float c0 = ex2f(m0 - mn0), c1 = ex2f(m1 - mn1);   // 0 on the first block
     m0 = mn0;
     m1 = mn1;
-    l0 *= c0;
-    l1 *= c1;
+    ol[0] *= c0; ol[1] *= c0;
+    ol[2] *= c1; ol[3] *= c1;
 #pragma unroll
     for (int nb = 0; nb < 4; ++nb) {
       o[nb][0] *= c0; o[nb][1] *= c0;
@@ -350,9 +352,6 @@ __device__ __forceinline__ void head_attention(uint32_t qb, int LK, int K, const
     for (int nb = 0; nb < NB; ++nb) {
       const uint32_t h01 = ex2_h2(pack_h2(s4[nb][0] - mn0, s4[nb][1] - mn0));
       const uint32_t h23 = ex2_h2(pack_h2(s4[nb][2] - mn1, s4[nb][3] - mn1));
-      const float2 f01 = h2_to_f2(h01), f23 = h2_to_f2(h23);
-      l0 += f01.x + f01.y;
-      l1 += f23.x + f23.y;
       const int kk = nb >> 1;
       if ((nb & 1) == 0) {
         pa[kk][0] = h01;
@@ -363,7 +362,8 @@ __device__ __forceinline__ void head_attention(uint32_t qb, int LK, int K, const
       }
     }
 #pragma unroll
-    for (int kk = 0; kk < NB / 2; ++kk)
+    for (int kk = 0; kk < NB / 2; ++kk) {
+      mma_f16_16816(ol, pa[kk], ONES_H2, ONES_H2);
 #pragma unroll
       for (int nb = 0; nb < 4; nb += 2) {
         uint32_t vf[4];
@@ -372,13 +372,10 @@ __device__ __forceinline__ void head_attention(uint32_t qb, int LK, int K, const
         mma_f16_16816(o[nb], pa[kk], vf[0], vf[1]);
         mma_f16_16816(o[nb + 1], pa[kk], vf[2], vf[3]);
       }
+    }
   }
-  l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-  l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-  l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-  l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-  inv0 = 1.0f / l0;
-  inv1 = 1.0f / l1;
+  inv0 = 1.0f / ol[0];
+  inv1 = 1.0f / ol[2];
 }
 
 
@@ -406,8 +403,7 @@ __device__ __forceinline__ void head_attention_part(uint32_t qb, uint32_t kb, ui
   const int si0 = s_slot[qoff + q0 + g8], si1 = s_slot[qoff + q0 + g8 + 8];
   m0 = -INFINITY;
   m1 = -INFINITY;
-  l0 = 0.f;
-  l1 = 0.f;
+  float ol[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int nb = 0; nb < 4; ++nb) o[nb][0] = o[nb][1] = o[nb][2] = o[nb][3] = 0.f;
 #pragma unroll 1
@@ -467,8 +463,8 @@ __device__ __forceinline__ void head_attention_part(uint32_t qb, uint32_t kb, ui
     const float c0 = ex2f(m0 - mn0), c1 = ex2f(m1 - mn1);   // 0 on the first block
     m0 = mn0;
     m1 = mn1;
-    l0 *= c0;
-    l1 *= c1;
+    ol[0] *= c0; ol[1] *= c0;
+    ol[2] *= c1; ol[3] *= c1;
 #pragma unroll
     for (int nb = 0; nb < 4; ++nb) {
       o[nb][0] *= c0; o[nb][1] *= c0;
@@ -479,9 +475,6 @@ __device__ __forceinline__ void head_attention_part(uint32_t qb, uint32_t kb, ui
     for (int nb = 0; nb < NB; ++nb) {
       const uint32_t h01 = ex2_h2(pack_h2(s4[nb][0] - mn0, s4[nb][1] - mn0));
       const uint32_t h23 = ex2_h2(pack_h2(s4[nb][2] - mn1, s4[nb][3] - mn1));
-      const float2 f01 = h2_to_f2(h01), f23 = h2_to_f2(h23);
-      l0 += f01.x + f01.y;
-      l1 += f23.x + f23.y;
       const int kk = nb >> 1;
       if ((nb & 1) == 0) {
         pa[kk][0] = h01;
@@ -492,7 +485,8 @@ __device__ __forceinline__ void head_attention_part(uint32_t qb, uint32_t kb, ui
       }
     }
 #pragma unroll
-    for (int kk = 0; kk < NB / 2; ++kk)
+    for (int kk = 0; kk < NB / 2; ++kk) {
+      mma_f16_16816(ol, pa[kk], ONES_H2, ONES_H2);
 #pragma unroll
       for (int nb = 0; nb < 4; nb += 2) {
         uint32_t vf[4];
@@ -501,11 +495,10 @@ __device__ __forceinline__ void head_attention_part(uint32_t qb, uint32_t kb, ui
         mma_f16_16816(o[nb], pa[kk], vf[0], vf[1]);
         mma_f16_16816(o[nb + 1], pa[kk], vf[2], vf[3]);
       }
+    }
   }
-  l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-  l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-  l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-  l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
+  l0 = ol[0];
+  l1 = ol[2];
 }
 
 // one 16-byte store into a peer's shared memory (peer address), ordinary (weak) semantics;
