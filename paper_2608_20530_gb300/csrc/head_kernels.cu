@@ -5,6 +5,8 @@
 // fp32 linear layer with fused bias / per-sequence bias / SiLU / residual
 // epilogue. The fp32 head runs every matrix product here; the bf16 head runs its
 // large products on the tensor cores (gemm_tc.cu) and the rest here.
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace lilicorr {
@@ -653,7 +655,10 @@ __global__ void unit_vectors_kernel(const float* __restrict__ oi, const float* _
 // keys), the four queries' probabilities of a key one piece (2 reads per 16 products). One
 // query a warp and single words read twice per product: 128 nodes x 128 (sequence, head)
 // pairs of 32, 45 us -> 22 us (cold).
-constexpr int AQ = 4;
+// While all queries fit the GPU's warps at one each (few short sequences), a warp takes AQ = 1:
+// the same sums, a quarter of the chain. Whole networks at D 256: two sequences of 8 nodes
+// 85.1 -> 82.1 us, of 32 nodes 102.9 -> 99.6; one of 32 at D 64 59.4 -> 55.3. At two waves of
+// CTAs AQ = 4 is ahead (one sequence of 256 nodes: 164, AQ = 1 172).
 
 __device__ __forceinline__ void fma4(float& acc, const float4& a, const float4& b) {
   acc = fmaf(a.x, b.x, acc);
@@ -662,7 +667,7 @@ __device__ __forceinline__ void fma4(float& acc, const float4& a, const float4& 
   acc = fmaf(a.w, b.w, acc);
 }
 
-template <typename TO>
+template <typename TO, int AQ>
 __global__ void __launch_bounds__(256)
 attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads, int q_per_cta,
                  const float* __restrict__ dist, const float* __restrict__ same,
@@ -696,7 +701,21 @@ attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads
   const float scale = rsqrtf((float)hd);
   const float sh = same[h];
   float* q = Qw + (size_t)warp * AQ * hd;
-  float4* p = reinterpret_cast<float4*>(Pw + (size_t)warp * LK * AQ);
+  float* p = Pw + (size_t)warp * LK * AQ;
+  auto load_p = [&](int j, float (&e)[AQ]) {
+    if constexpr (AQ == 4) {
+      const float4 v = *reinterpret_cast<const float4*>(p + 4 * j);
+      e[0] = v.x; e[1] = v.y; e[2] = v.z; e[3] = v.w;
+    } else {
+      e[0] = p[j];
+    }
+  };
+  auto store_p = [&](int j, const float (&e)[AQ]) {
+    if constexpr (AQ == 4)
+      *reinterpret_cast<float4*>(p + 4 * j) = make_float4(e[0], e[1], e[2], e[3]);
+    else
+      p[j] = e[0];
+  };
   // P V: lane = columns 4 cg.., keys ks, ks + nks, ...
   const int cg = lane % hv, ks = lane / hv, nks = 32 / hv;
   for (int i0 = q0 + AQ * warp; i0 < q1; i0 += AQ * nw) {
@@ -727,6 +746,7 @@ attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads
         for (int a = 0; a < AQ; ++a) qv[a] = *reinterpret_cast<const float4*>(q + a * hd + c);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
+          if (AQ == 1 && j0 + 32 * t >= LK) break;      // no lane has a key there
           const float4 kv = *reinterpret_cast<const float4*>(kr[t] + c);
 #pragma unroll
           for (int a = 0; a < AQ; ++a) fma4(s[t][a], qv[a], kv);
@@ -742,7 +762,7 @@ attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads
           s[t][a] = s[t][a] * scale + s_dist[sj - si[a] + L - 1] + (si[a] == sj ? sh : 0.f);
           mx[a] = fmaxf(mx[a], s[t][a]);
         }
-        p[j] = make_float4(s[t][0], s[t][1], s[t][2], s[t][3]);
+        store_p(j, s[t]);
       }
     }
     float sum[AQ];
@@ -752,11 +772,14 @@ attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads
       sum[a] = 0.f;
     }
     for (int j = lane; j < LK; j += 32) {      // each lane the keys it scored
-      float4 e = p[j];
-      e.x = __expf(e.x - mx[0]); e.y = __expf(e.y - mx[1]);
-      e.z = __expf(e.z - mx[2]); e.w = __expf(e.w - mx[3]);
-      p[j] = e;
-      sum[0] += e.x; sum[1] += e.y; sum[2] += e.z; sum[3] += e.w;
+      float e[AQ];
+      load_p(j, e);
+#pragma unroll
+      for (int a = 0; a < AQ; ++a) {
+        e[a] = __expf(e[a] - mx[a]);
+        sum[a] += e[a];
+      }
+      store_p(j, e);
     }
     __syncwarp();
     float4 o[AQ];
@@ -769,8 +792,8 @@ attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads
 #pragma unroll 4
       for (int j = ks; j < LK; j += nks) {
         const float4 v = *reinterpret_cast<const float4*>(Vs + j * hd + 4 * cg);
-        const float4 pj = p[j];
-        const float w[AQ] = {pj.x, pj.y, pj.z, pj.w};
+        float w[AQ];
+        load_p(j, w);
 #pragma unroll
         for (int a = 0; a < AQ; ++a) {
           o[a].x = fmaf(w[a], v.x, o[a].x);
@@ -803,7 +826,7 @@ attention_kernel(const float* __restrict__ qkv, int L, int K, int D, int n_heads
 
 // floats of shared memory beside s_dist, for `warps` warps
 size_t attention_floats(int LK, int hd, int warps) {
-  return (size_t)LK * (2 * hd + 4) + (size_t)warps * AQ * (hd + LK);
+  return (size_t)LK * (2 * hd + 4) + (size_t)warps * 4 * (hd + LK);     // AQ <= 4
 }
 
 }  // namespace
@@ -940,23 +963,30 @@ lilicorr_status_t launch_attention(const float* qkv, int B, int L, int K, int D,
   int warps = 8;
   while (warps > 2 && attention_floats(LK, hd, warps) * sizeof(float) > most) warps /= 2;
   const size_t smem = (attention_floats(LK, hd, warps) + 2 * L - 1) * sizeof(float);
-  static bool cfg_f32[64] = {false}, cfg_bf16[64] = {false};
-  LL_TRY(allow_max_dynamic_smem(attention_kernel<float>, cfg_f32));
-  LL_TRY(allow_max_dynamic_smem(attention_kernel<__nv_bfloat16>, cfg_bf16));
+  // one query a warp while that is one wave of CTAs, else four
+  const int aq = (long long)B * n_heads * ceil_div(LK, warps) <= num_sms() ? 1 : 4;
   // split the queries of a (sequence, head) over CTAs until the grid covers the GPU; each warp
   // takes whole groups of AQ
-  int qblocks = ceil_div(4 * num_sms(), B * n_heads);
-  qblocks = max(1, min(qblocks, ceil_div(LK, AQ * warps)));
-  const int q_per_cta = ceil_div(ceil_div(LK, qblocks), AQ) * AQ;
+  int qblocks = aq == 1 ? ceil_div(LK, warps) : ceil_div(4 * num_sms(), B * n_heads);
+  qblocks = max(1, min(qblocks, ceil_div(LK, aq * warps)));
+  const int q_per_cta = ceil_div(ceil_div(LK, qblocks), aq) * aq;
   qblocks = ceil_div(LK, q_per_cta);
-  dim3 grid(B * n_heads, qblocks);
-  if (out_dt == LILICORR_F32)
-    LL_TRY(launch_k(attention_kernel<float>, grid, warps * 32, smem, st, qkv, L, K, D, n_heads, q_per_cta, dist,
-                                                            same, static_cast<float*>(out)));
-  else
-    LL_TRY(launch_k(attention_kernel<__nv_bfloat16>, grid, warps * 32, smem, st, 
-        qkv, L, K, D, n_heads, q_per_cta, dist, same, static_cast<__nv_bfloat16*>(out)));
-  return LILICORR_OK;
+  const dim3 grid(B * n_heads, qblocks);
+  const auto launch = [&](auto q, auto* to) -> lilicorr_status_t {
+    auto* kern = attention_kernel<std::remove_pointer_t<decltype(to)>, decltype(q)::value>;
+    static bool cfg[64] = {false};             // one per kernel: q and to name it
+    LL_TRY(allow_max_dynamic_smem(kern, cfg));
+    return launch_k(kern, grid, warps * 32, smem, st, qkv, L, K, D, n_heads, q_per_cta, dist, same,
+                    to);
+  };
+  const std::integral_constant<int, 1> q1;
+  const std::integral_constant<int, 4> q4;
+  if (out_dt == LILICORR_F32) {
+    float* to = static_cast<float*>(out);
+    return aq == 1 ? launch(q1, to) : launch(q4, to);
+  }
+  __nv_bfloat16* to = static_cast<__nv_bfloat16*>(out);
+  return aq == 1 ? launch(q1, to) : launch(q4, to);
 }
 
 }  // namespace lilicorr

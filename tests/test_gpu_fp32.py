@@ -34,6 +34,18 @@ def test_linear_tiled(M, N, Kd, dt):
 @pytest.mark.parametrize("B,L,K,D", [(1, 1, 1, 32), (2, 5, 7, 64), (9, 16, 8, 256), (1, 32, 16, 320),
                                      (2, 3, 3, 1024), (3, 17, 5, 96)])
 def test_fp32_network_matches_oracle(B, L, K, D):
+    _network_matches_oracle(B, L, K, D)
+
+
+# the attention core's one query a warp (at most a wave of CTAs) and the sizes next to its edge:
+# a last warp without a query, keys that fill no lane group, 8 heads x 19 CTAs of 152
+@pytest.mark.parametrize("B,L,K,D", [(1, 1, 9, 64), (1, 11, 3, 96), (1, 19, 8, 256),
+                                     (1, 17, 9, 256), (2, 9, 8, 64), (3, 7, 7, 32)])
+def test_fp32_attention_one_query(B, L, K, D):
+    _network_matches_oracle(B, L, K, D)
+
+
+def _network_matches_oracle(B, L, K, D):
     ll = _ll()
     wl = workloads.Workload(f"fp32_b{B}_l{L}_k{K}_d{D}", B=B, L=L, V=2000, K=K, d=D, H=128,
                             dtype="f32", logit_kind="normal_planted", logit_param=(3.0, 8.0),
