@@ -423,6 +423,21 @@ bool fold_norms(const HeadCall& c) {
   return true;
 }
 
+// Network kernels: a cluster of four SMs per sequence while every sequence's cluster fits on the
+// GPU at once; beyond that one SM per sequence (fewer waves); two SMs per sequence of 129-256
+// nodes, one 128-node tile each; the chain of kernels, each spread over SMs, for heads that
+// none of them takes.
+enum class NetPath { CLUSTER, FUSED, PAIR, CHAIN };
+NetPath net_path(const HeadCall& c) {
+  const lilicorr_head* h = c.h;
+  if (h->cluster_maps && (g_fused_enabled == 3 ||
+                          (g_fused_enabled == 1 && c.B <= net_cluster_capacity())))
+    return NetPath::CLUSTER;
+  if (h->net_maps && (g_fused_enabled == 2 || (g_fused_enabled == 1 && c.B >= FUSED_MIN_B)))
+    return NetPath::FUSED;
+  return h->pair_maps && g_fused_enabled != 0 ? NetPath::PAIR : NetPath::CHAIN;
+}
+
 // Candidate-dependent part: nodes, the Transformer, fusion and the out/in heads. Writes
 // oi = [W_o u + b_o | W_i u + b_i] (not yet normalised). `pro` holds the candidate-independent
 // part still running on the side streams; the chain waits for each half where it first reads
@@ -437,24 +452,17 @@ lilicorr_status_t run_body(const HeadCall& c, Prologue& pro, const int32_t* ids,
   const lilicorr_head_desc& d = c.d;
   const lilicorr_dtype_t F32 = LILICORR_F32, adt = c.adt;
   const int D = c.D, F = c.F, N = c.N;
-  // Network kernels: a cluster of four SMs per sequence while every sequence's cluster
-  // fits on the GPU at once; beyond that one SM per sequence (fewer waves); the chain of
-  // kernels below, each spread over SMs, for heads neither kernel takes.
-  const bool cluster = h->cluster_maps &&
-                       (g_fused_enabled == 3 ||
-                        (g_fused_enabled == 1 && c.B <= net_cluster_capacity()));
-  const bool fused =
-      h->net_maps && (g_fused_enabled == 2 || (g_fused_enabled == 1 && c.B >= FUSED_MIN_B));
-  // 129-256 nodes per sequence: two CTAs per sequence, one 128-node tile each
-  const bool pair = h->pair_maps && g_fused_enabled != 0;
+  const NetPath path = net_path(c);
   LL_TRY(pro.join_hidden());
-  if (cluster || fused || pair) LL_TRY(pro.join_target());
-  if (cluster) {
+  if (path != NetPath::CHAIN) LL_TRY(pro.join_target());
+  if (path == NetPath::CLUSTER) {
     if (tail_done) *tail_done = tail != nullptr;
     return launch_net_cluster(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st, tail);
   }
-  if (fused) return launch_net_fused(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st);
-  if (pair) return launch_net_pair(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st);
+  if (path == NetPath::FUSED)
+    return launch_net_fused(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st);
+  if (path == NetPath::PAIR)
+    return launch_net_pair(h, c.B, ids, logp, c.hproj, c.t, c.cb, c.oi, c.status, st);
   // nodes: x = fold[id] + hproj + slot + rank, then x += W_c2 c1 + b_c2
   LL_TRY(launch_node_build(h, c.B, ids, logp, c.hproj, c.c1, adt, c.x, c.status, st));
   GemmArgs g = c.G(c.c1, adt, D, h->conf2_w, D, c.x, F32, D, N, D, D), from;
@@ -926,8 +934,14 @@ lilicorr_status_t lilicorr_select_block_walk(const lilicorr_head* head, int B, c
   LL_TRY(launch_topk_lse(logits, d.dtype, R, d.V, d.K, ids, logp, at<float>(ws, w.lse),
                          at<uint32_t>(ws, w.status), at<uint32_t>(ws, w.counters),
                          at<void>(ws, w.partials), stream));
+  // then what is needed soonest: the chain of kernels reads the drafter states first and the
+  // target state near its end (fp32, 16 requests of 32 nodes at D 64: 93 us, target chain first
+  // 137; 16 of 128 at D 256: 309, 316); the network kernels wait for both, and the target chain
+  // is the longer
+  const bool chain = net_path(call) == NetPath::CHAIN;
+  if (chain) LL_TRY(pro.fork_hidden(call, drafter_hidden));
   LL_TRY(pro.fork_target(call, target_hidden));
-  LL_TRY(pro.fork_hidden(call, drafter_hidden));
+  if (!chain) LL_TRY(pro.fork_hidden(call, drafter_hidden));
   ClusterTail tail;
   tail.anchor = at<float>(ws, w.anc);
   tail.A = at<float>(ws, w.A);
