@@ -485,7 +485,7 @@ def test_linear(A: torch.Tensor, W: torch.Tensor, out_dtype=torch.float32, bias=
     """Test hook: one linear layer C = act(A W^T + bias) + residual through kernel `path`
     (0 auto, 1 tiled CUDA cores, 2 few-row CUDA cores, 3 tensor cores, 4 tensor cores for one
     tile of rows, 5 row-block CUDA cores for fp32 A, 6 tensor cores with Kd split over a
-    cluster)."""
+    cluster, 7 tiled CUDA cores with Kd split over a cluster)."""
     M, Kd = A.shape
     N = W.shape[0]
     C = torch.empty((M, N), dtype=out_dtype, device=A.device)

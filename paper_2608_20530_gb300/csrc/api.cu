@@ -202,7 +202,7 @@ GemmArgs gemm(const void* A, lilicorr_dtype_t a_dt, int lda, const void* W, lili
 }
 
 // The kernel that a product of the network takes.
-enum class GemmPath { SKINNY, ROWS, SMALL, SPLIT, TC, SIMT };
+enum class GemmPath { SKINNY, ROWS, SMALL, SPLIT, TC, SIMT, SIMT_SPLIT };
 
 // bf16 operands: tensor cores (one tile of rows and short Kd: whole-K copies; few output
 // tiles: Kd split over a cluster; else the persistent kernel), but for the fewest rows, where
@@ -211,6 +211,18 @@ enum class GemmPath { SKINNY, ROWS, SMALL, SPLIT, TC, SIMT };
 GemmPath gemm_path(const GemmArgs& g) {
   const bool fold = g.c2 || g.ss_in;          // only these two kernels fold an RMSNorm
   if (fold) return gemm_split_supported(g) ? GemmPath::SPLIT : GemmPath::TC;
+  // fp32 throughout and Kd long enough to split (us, 16 x 32 blocks / the kernel taken):
+  // one wave of the split-N kernel's CTAs (32 x 256 x 1024: 16.9 / 4.3), or two at long Kd
+  // (64 x 256 x 4096: 64 / 12); else 64 x 64 tiles, Kd split while tiles are few
+  // (128 x 256 x 256: 5.1 / 4.4, 1024 x 256 x 512: 30.8 / 11.0; unsplit 1024 x 512 x 256:
+  // 18.3 / 9.8). At Kd = 64 the 16 x 32 blocks are ahead (256 x 64: 2.3, tiles 4.1).
+  if (g.a_dt == LILICORR_F32 && g.w_dt == LILICORR_F32 && g.M > 16 && g.Kd >= 256 &&
+      gemm_rows_supported(g)) {
+    const long long ctas = (long long)ceil_div(g.N, 4) * ceil_div(g.M, 16);
+    if (g.lda % 8 == 0 && (ctas <= num_sms() || (ctas <= 2 * num_sms() && g.Kd >= 1024)))
+      return GemmPath::SKINNY;
+    return gemm_simt_ways(g) ? GemmPath::SIMT_SPLIT : GemmPath::SIMT;
+  }
   // fp32 activations (the tensor-core kernels take bf16) at per-sequence row counts above
   // 16: 16 x 32 output blocks with the rows staged (256 x 512 x 512: 54 -> ~5 us); few rows
   // otherwise: the split-N kernel
@@ -240,6 +252,7 @@ lilicorr_status_t run_gemm(const GemmArgs& g, cudaStream_t st) {
     case GemmPath::SMALL: return launch_gemm_small(g, st);
     case GemmPath::SPLIT: return launch_gemm_split(g, st);
     case GemmPath::TC: return gemm_tc_supported(g) ? launch_gemm_tc(g, st) : LILICORR_ERR_SHAPE;
+    case GemmPath::SIMT_SPLIT: return launch_gemm_simt_split(g, st);
     case GemmPath::SIMT: break;
   }
   return launch_gemm_simt(g, st);
@@ -1002,6 +1015,7 @@ lilicorr_status_t lilicorr_test_linear(const void* A, lilicorr_dtype_t a_dt, int
     case 4: return gemm_small_supported(g) ? launch_gemm_small(g, stream) : LILICORR_ERR_SHAPE;
     case 5: return launch_gemm_rows(g, stream);
     case 6: return gemm_split_supported(g) ? launch_gemm_split(g, stream) : LILICORR_ERR_SHAPE;
+    case 7: return launch_gemm_simt_split(g, stream);
   }
   return LILICORR_ERR_ARG;
 }

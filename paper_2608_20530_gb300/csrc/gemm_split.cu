@@ -37,17 +37,6 @@ constexpr uint32_t SP_A_BYTES = 128 * SP_BK * 2;
 constexpr long long SP_WAIT = 4000000000ll;
 constexpr float SP_RMS_EPS = 1e-6f;
 
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t local, uint32_t rank) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(a)
-               : "memory");
-  return v;
-}
-
 struct SplitArgs {
   GemmArgs g;
   int S;             // CTAs per tile (cluster size)

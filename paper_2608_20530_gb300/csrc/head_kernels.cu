@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "internal.cuh"
+#include "tc_ptx.cuh"
 
 namespace lilicorr {
 
@@ -27,6 +28,11 @@ constexpr float UNIT_EPS = 1e-12f;
 // next step's operands are loaded (16 bytes a thread where rows allow) while this one is
 // multiplied.
 // 2048 x 256 x 256: 31 -> 15.5 us; 2048 x 256 x 512: 55 -> 23.6 us (cold).
+// Few tiles leave SMs idle and the chain of steps as long: there a cluster of 2, 4 or 8 CTAs
+// splits Kd (warm, in a graph; the 16 x 32 blocks that had these sizes / split): 128 x 256 x 256
+// 5.1 / 4.4 us, 512 x 256 x 512 13.3 / 7.6, 1024 x 256 x 256 15.8 / 7.3, 512 x 256 x 4096
+// 91 / 33; its error against 64 bits is a third of theirs (9e-8 to 2e-7; 3e-7 to 1e-6).
+// Whole fp32 networks of 4 and 8 sequences of 128 nodes, D 256: 224 -> 145 and 293 -> 195 us.
 constexpr int GB_M = 64, GB_N = 64, GB_K = 32, G_THREADS = 256, G_GROUPS = 4;
 
 __device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
@@ -69,8 +75,10 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p, int r, int rows,
 }
 
 // VEC: rows of both operands in whole aligned groups of four elements
-template <typename TA, typename TW, typename TC, bool VEC>
-__global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g) {
+// SPLIT: the CTAs of a cluster take a part of Kd's steps each (at least one) and then a part of
+// the tile's rows each, whose sums they read from one another
+template <typename TA, typename TW, typename TC, bool VEC, bool SPLIT>
+__global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g, int ways) {
   pdl_wait();
   constexpr int LDT = GB_M + 4, KG = GB_K / G_GROUPS;
   static_assert(GB_M == GB_N && GB_M * GB_K == 8 * G_THREADS, "two groups of four a thread");
@@ -80,7 +88,11 @@ __global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g) {
   const TA* A = static_cast<const TA*>(g.A);
   const TW* W = static_cast<const TW*>(g.W);
   const int tid = threadIdx.x, grp = tid >> 6;
-  const int m0 = blockIdx.y * GB_M, n0 = blockIdx.x * GB_N;
+  const int rank = SPLIT ? blockIdx.x % ways : 0;
+  const int m0 = blockIdx.y * GB_M, n0 = (SPLIT ? blockIdx.x / ways : blockIdx.x) * GB_N;
+  const int steps = (g.Kd + GB_K - 1) / GB_K;
+  const int kbeg = SPLIT ? steps * rank / ways * GB_K : 0;
+  const int kend = SPLIT ? min(g.Kd, steps * (rank + 1) / ways * GB_K) : g.Kd;
   const int tx = tid & 7, ty = (tid >> 3) & 7;
   const int lr = tid >> 3, lk = (tid & 7) * 4;        // rows lr and lr + 32, columns lk..lk + 3
   uint64_t acc[8][4];
@@ -106,12 +118,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g) {
       sm[b][1][lk + 2][r] = rw[h].z; sm[b][1][lk + 3][r] = rw[h].w;
     }
   };
-  fetch(0);
+  fetch(kbeg);
   stash(0);
   __syncthreads();
   int b = 0;
-  for (int k0 = 0; k0 < g.Kd; k0 += GB_K, b ^= 1) {
-    const bool more = k0 + GB_K < g.Kd;
+  for (int k0 = kbeg; k0 < kend; k0 += GB_K, b ^= 1) {
+    const bool more = k0 + GB_K < kend;
     if (more) fetch(k0 + GB_K);
 #pragma unroll
     for (int kk = 0; kk < KG; ++kk) {
@@ -161,17 +173,31 @@ __global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g) {
     // each thread overwrites only what it has just read itself
     put(grp);
   }
-  __syncthreads();
+  if (SPLIT) tc::cluster_sync();             // every CTA's sums are in place
+  else __syncthreads();
   // ---- epilogue: 16 threads a row, four columns each
   TC* C = static_cast<TC*>(g.C);
   const int c = (tid & 15) * 4, n = n0 + c;
+  const int rows = SPLIT ? GB_M / ways : GB_M;
 #pragma unroll
-  for (int r = tid >> 4; r < GB_M; r += G_THREADS / 16) {
-    const int m = m0 + r;
+  for (int r1 = tid >> 4; r1 < rows; r1 += G_THREADS / 16) {
+    const int r = rank * rows + r1, m = m0 + r;
     if (m >= g.M) break;
-    const float4 s0 = *reinterpret_cast<const float4*>(red + r * LDT + c);
-    const float4 s1 = *reinterpret_cast<const float4*>(red + (GB_M + r) * LDT + c);
-    const float s[4] = {s0.x + s1.x, s0.y + s1.y, s0.z + s1.z, s0.w + s1.w};
+    float s[4];
+    if (SPLIT) {                             // in the order of Kd
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[j] = 0.f;
+#pragma unroll 4
+      for (int q = 0; q < ways; ++q) {
+        const float4 s0 = tc::ld_cluster_f4(tc::smem_u32(red + r * LDT + c), q);
+        const float4 s1 = tc::ld_cluster_f4(tc::smem_u32(red + (GB_M + r) * LDT + c), q);
+        s[0] += s0.x + s1.x; s[1] += s0.y + s1.y; s[2] += s0.z + s1.z; s[3] += s0.w + s1.w;
+      }
+    } else {
+      const float4 s0 = *reinterpret_cast<const float4*>(red + r * LDT + c);
+      const float4 s1 = *reinterpret_cast<const float4*>(red + (GB_M + r) * LDT + c);
+      s[0] = s0.x + s1.x; s[1] = s0.y + s1.y; s[2] = s0.z + s1.z; s[3] = s0.w + s1.w;
+    }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       if (n + j >= g.N) break;
@@ -183,22 +209,39 @@ __global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g) {
       st_elem(C, (size_t)m * g.ldc + n + j, v);
     }
   }
+  if (SPLIT) {
+    __syncwarp();
+    tc::cluster_sync();                      // no CTA leaves while a peer reads its sums
+  }
 }
 
 template <typename TA, typename TW, bool VEC>
 lilicorr_status_t gemm_dispatch_c(const GemmArgs& g, dim3 grid, cudaStream_t st) {
   if (g.c_dt == LILICORR_F32)
-    return launch_k(gemm_simt_kernel<TA, TW, float, VEC>, grid, G_THREADS, 0, st, g);
-  return launch_k(gemm_simt_kernel<TA, TW, __nv_bfloat16, VEC>, grid, G_THREADS, 0, st, g);
+    return launch_k(gemm_simt_kernel<TA, TW, float, VEC, false>, grid, G_THREADS, 0, st, g, 1);
+  return launch_k(gemm_simt_kernel<TA, TW, __nv_bfloat16, VEC, false>, grid, G_THREADS, 0, st, g, 1);
 }
+template <typename TW>
+lilicorr_status_t gemm_split_dispatch_c(const GemmArgs& g, dim3 grid, int ways, cudaStream_t st) {
+  grid.x *= ways;
+  if (g.c_dt == LILICORR_F32)
+    return launch_cluster_k(gemm_simt_kernel<float, TW, float, true, true>, grid, G_THREADS, 0,
+                            ways, st, g, ways);
+  return launch_cluster_k(gemm_simt_kernel<float, TW, __nv_bfloat16, true, true>, grid, G_THREADS,
+                          0, ways, st, g, ways);
+}
+
+// groups of four elements: Kd and the row strides multiples of 4, bases on 16 (fp32) or 8
+// (bf16) bytes; other operands are read element by element
+bool gemm_simt_vec(const GemmArgs& g) {
+  const uintptr_t am = g.a_dt == LILICORR_F32 ? 15 : 7, wm = g.w_dt == LILICORR_F32 ? 15 : 7;
+  return g.Kd % 4 == 0 && g.lda % 4 == 0 && g.ldw % 4 == 0 &&
+         !(reinterpret_cast<uintptr_t>(g.A) & am) && !(reinterpret_cast<uintptr_t>(g.W) & wm);
+}
+
 template <typename TA>
 lilicorr_status_t gemm_dispatch_w(const GemmArgs& g, dim3 grid, cudaStream_t st) {
-  // groups of four elements: Kd and the row strides multiples of 4, bases on 16 (fp32) or 8
-  // (bf16) bytes; other operands are read element by element
-  const uintptr_t am = sizeof(TA) * 4 - 1, wm = g.w_dt == LILICORR_F32 ? 15 : 7;
-  const bool vec = g.Kd % 4 == 0 && g.lda % 4 == 0 && g.ldw % 4 == 0 &&
-                   !(reinterpret_cast<uintptr_t>(g.A) & am) &&
-                   !(reinterpret_cast<uintptr_t>(g.W) & wm);
+  const bool vec = gemm_simt_vec(g);
   if (g.w_dt == LILICORR_F32)
     return vec ? gemm_dispatch_c<TA, float, true>(g, grid, st)
                : gemm_dispatch_c<TA, float, false>(g, grid, st);
@@ -866,6 +909,26 @@ lilicorr_status_t launch_gemm_skinny(const GemmArgs& g, cudaStream_t st, const G
   }
   if (g.a_dt == LILICORR_F32) return skinny_dispatch_w<float>(g, g1, st);
   return skinny_dispatch_w<__nv_bfloat16>(g, g1, st);
+}
+
+// CTAs per tile of the split kernel: as many as still are one wave with a step of Kd each; eight
+// only for few tiles, since 16 clusters of eight did not run at once (256 x 256 x 512: 11.5 us,
+// four ways 7.6).
+int gemm_simt_ways(const GemmArgs& g) {
+  if (g.a_dt != LILICORR_F32 || g.M <= 0 || g.N <= 0 || !gemm_simt_vec(g)) return 0;
+  const long long tiles = (long long)ceil_div(g.N, GB_N) * ceil_div(g.M, GB_M);
+  const int steps = ceil_div(g.Kd, GB_K);
+  int ways = tiles <= 8 ? 8 : 4;
+  while (ways > 1 && (tiles * ways > num_sms() || steps < ways)) ways /= 2;
+  return ways > 1 ? ways : 0;
+}
+
+lilicorr_status_t launch_gemm_simt_split(const GemmArgs& g, cudaStream_t st) {
+  const int ways = gemm_simt_ways(g);
+  if (!ways) return LILICORR_ERR_SHAPE;
+  const dim3 grid(ceil_div(g.N, GB_N), ceil_div(g.M, GB_M));
+  return g.w_dt == LILICORR_F32 ? gemm_split_dispatch_c<float>(g, grid, ways, st)
+                                : gemm_split_dispatch_c<__nv_bfloat16>(g, grid, ways, st);
 }
 
 lilicorr_status_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st) {

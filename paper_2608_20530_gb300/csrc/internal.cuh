@@ -319,6 +319,9 @@ struct GemmArgs {
 constexpr int SS_LD = 16;  // floats per row of a folded-RMSNorm sums-of-squares buffer
 int gemm_tc_ss_slots(int M, int N);
 lilicorr_status_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
+// the same with Kd split over a cluster of that many CTAs (0: not taken)
+int gemm_simt_ways(const GemmArgs& g);
+lilicorr_status_t launch_gemm_simt_split(const GemmArgs& g, cudaStream_t st);
 // `second`: another product of the same rows, types and Kd in the same launch
 lilicorr_status_t launch_gemm_skinny(const GemmArgs& g, cudaStream_t st,
                                      const GemmArgs* second = nullptr);   // M <= 64

@@ -31,6 +31,27 @@ def test_linear_tiled(M, N, Kd, dt):
     assert (C.double() - want).abs().max().item() <= tol
 
 
+# clusters of 2, 4 and 8, uneven parts of Kd and a short last step, ragged tiles; path 0 where
+# the rule takes another kernel (one wave of the split-N kernel, Kd below 256, more tiles than SMs)
+@pytest.mark.parametrize("path,M,N,Kd", [(7, 1, 1, 64), (7, 65, 63, 36), (7, 64, 64, 2052),
+                                         (7, 130, 260, 292), (7, 512, 512, 320), (7, 640, 256, 256),
+                                         (0, 32, 256, 1024), (0, 64, 256, 4096), (0, 33, 256, 256),
+                                         (0, 33, 256, 248), (0, 1000, 512, 264), (0, 1100, 96, 1000)])
+@pytest.mark.parametrize("wdt", [torch.float32, torch.bfloat16])
+def test_linear_tiled_split(path, M, N, Kd, wdt):
+    ll = _ll()
+    g = torch.Generator(device="cuda").manual_seed(M * 7 + N + Kd)
+    A = torch.randn((M, Kd), generator=g, device="cuda")
+    W = torch.randn((N, Kd), generator=g, device="cuda").to(wdt)
+    bias = torch.randn(N, generator=g, device="cuda")
+    res = torch.randn((M, N), generator=g, device="cuda")
+    C = ll.test_linear(A, W, torch.float32, bias=bias, residual=res, path=path)
+    want = A.double() @ W.double().T + bias + res
+    # an fp32 sum of Kd + 2 terms, in any order
+    tol = (Kd + 2) * 2.0 ** -24 * (A.double().abs() @ W.double().abs().T + 8).max().item()
+    assert (C.double() - want).abs().max().item() <= tol
+
+
 @pytest.mark.parametrize("B,L,K,D", [(1, 1, 1, 32), (2, 5, 7, 64), (9, 16, 8, 256), (1, 32, 16, 320),
                                      (2, 3, 3, 1024), (3, 17, 5, 96)])
 def test_fp32_network_matches_oracle(B, L, K, D):
