@@ -29,7 +29,9 @@ extern "C" {
  * 5 = row-block CUDA-core kernel for fp32 A (Kd a multiple of 8, lda of 4, ldw of 8, A and
  *     W 16-byte aligned; LILICORR_ERR_SHAPE otherwise),
  * 6 = tensor cores with Kd split over a cluster (bf16 A and W, few output tiles;
- *     LILICORR_ERR_SHAPE otherwise).
+ *     LILICORR_ERR_SHAPE otherwise),
+ * 7 = tiled CUDA cores with Kd split over a cluster (fp32 A, few output tiles, Kd and row
+ *     strides multiples of 4; LILICORR_ERR_SHAPE otherwise).
  * status: a device uint32 word that receives bounded-wait timeouts (may be NULL). */
 lilicorr_status_t lilicorr_test_linear(const void* A, lilicorr_dtype_t a_dt, int lda, const void* W,
                                        lilicorr_dtype_t w_dt, int ldw, void* C,

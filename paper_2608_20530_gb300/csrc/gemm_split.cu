@@ -3,12 +3,12 @@
 //
 // A head of width 1024 with one request multiplies 120 node rows by [1024 .. 3072, 1024 .. 2048]
 // weights: 16 to 48 tiles of 128 x 64, so a kernel with one CTA per tile leaves two thirds of
-// the SMs idle while the others stream Kd / 64 chunks one after the other. Here S = 1, 2, 4 or 8 CTAs, one cluster, share a tile:
-// each multiplies its part of Kd into its own tensor memory, parks the 128 x BN partial sums
-// in its shared memory, and after a cluster barrier every CTA adds up the S partials of the
-// rows r, r + S, r + 2S, ... (distributed shared memory, in rank order, so the result is the
-// same on every call) and runs the epilogue on them. gemm_split_ways says how S
-// follows from the sizes.
+// the SMs idle while the others stream Kd / 64 chunks one after the other. Here S = 1, 2, 4 or 8
+// CTAs, one cluster, share a tile: each multiplies its part of Kd into its own tensor memory,
+// parks the 128 x BN partial sums in its shared memory, and after a cluster barrier every CTA
+// adds up the S partials of the rows r, r + S, r + 2S, ... (distributed shared memory, in rank
+// order, so the result is the same on every call) and runs the epilogue on them.
+// gemm_split_ways says how S follows from the sizes.
 //
 // Roles: warp 0 (one lane) streams 128 x 64 tiles of A and BN x 64 tiles of W by TMA (128-byte
 // swizzle, four stages), warp 1 issues tcgen05.mma (M = 128, N = BN), warps 4-7 drain the
@@ -16,13 +16,13 @@
 // first four chunks are requested before the wait on the preceding launch: only A's copy,
 // the products and the reduction are left on the chain. What bounds it is that latency, not a
 // pipe: with these products, the RMSNorms folded into them and the target chain beside the
-// body, the network of width 1024 takes 115 us for one request (170 before) and 309 us for 24
-// (352: its prologue's 15- and 24-row products); serving_b32's drafter-state product (512
-// rows, 16 tiles, Kd = 4096) beside the top-K pass 136.7 -> 131.7 us a call. The same epilogues as the persistent
-// kernel (gemm_tc.cu): bias, per-sequence bias, SiLU, residual, and the RMSNorm folded into
-// the products around it. Every mbarrier wait is bounded; on timeout the kernel records
-// LILICORR_ERR_TIMEOUT, keeps every thread on its barriers, lets copies in flight land, frees
-// its tensor memory and returns.
+// body, the network of width 1024 went from 170 to 115 us for one request and from 352 to 309
+// for 24 (its prologue's 15- and 24-row products; 100 and 278 with what followed); serving_b32's
+// drafter-state product (512 rows, 16 tiles, Kd = 4096) beside the top-K pass 136.7 -> 131.7 us a
+// call. The same epilogues as the persistent kernel (gemm_tc.cu): bias, per-sequence bias, SiLU,
+// residual, and the RMSNorm folded into the products around it. Every mbarrier wait is bounded;
+// on timeout the kernel records LILICORR_ERR_TIMEOUT, keeps every thread on its barriers, lets
+// copies in flight land, frees its tensor memory and returns.
 #include "tc_ptx.cuh"
 
 namespace lilicorr {
