@@ -370,9 +370,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
               const float4* tr = reinterpret_cast<const float4*>(
                   t_shared ? s_t + cl
                            : ep.c3_t + (size_t)(m < M ? m / ep.c3_rows_per : 0) * N + n0 + cl);
+              // s_t holds zeros past N; a row of c3_t ends there (N is whole groups of HC)
+              const bool t_in = t_shared || n0 + cl < N;
 #pragma unroll
               for (int j = 0; j < HC; j += 4) {
-                const float4 tv = tr[j / 4];
+                const float4 tv = t_in ? tr[j / 4] : make_float4(0.f, 0.f, 0.f, 0.f);
                 wv[j / 2] = pack_bf16x2(g[j] * tv.x, g[j + 1] * tv.y);
                 wv[j / 2 + 1] = pack_bf16x2(g[j + 2] * tv.z, g[j + 3] * tv.w);
               }

@@ -36,7 +36,10 @@ def test_linear_wide_stages(M, N, Kd):
     assert int(status.item()) == 0
 
 
-@pytest.mark.parametrize("B,L,K,D", [(90, 15, 15, 512), (80, 16, 8, 1024)])
+# 256-column tiles; then 192-column ones, whose last is past N in part (1024 = 5 x 192 + 64, 512 =
+# 2 x 192 + 128), with row tiles that span sequences: 2880 rows x 1024 and 12,000 x 512
+@pytest.mark.parametrize("B,L,K,D", [(90, 15, 15, 512), (80, 16, 8, 1024), (24, 15, 8, 1024),
+                                     (100, 15, 8, 512)])
 def test_wide_network_matches_oracle(B, L, K, D):
     ll = _ll()
     wl = workloads.Workload(f"wide_b{B}_d{D}", B=B, L=L, V=1000, K=K, d=D, H=64, dtype="bf16",
