@@ -210,7 +210,7 @@ enum class GemmPath { SKINNY, ROWS, SMALL, SPLIT, TC, SIMT, SIMT_SPLIT };
 // the CUDA cores (the fp32 head keeps fp32 arithmetic throughout).
 GemmPath gemm_path(const GemmArgs& g) {
   const bool fold = g.c2 || g.ss_in;          // only these two kernels fold an RMSNorm
-  if (fold) return gemm_split_supported(g) ? GemmPath::SPLIT : GemmPath::TC;
+  if (fold) return gemm_split_takes(g) ? GemmPath::SPLIT : GemmPath::TC;
   // fp32 throughout and Kd long enough to split (us, 16 x 32 blocks / the kernel taken):
   // one wave of the split-N kernel's CTAs (32 x 256 x 1024: 16.9 / 4.3), or two at long Kd
   // (64 x 256 x 4096: 64 / 12); else 64 x 64 tiles, Kd split while tiles are few
@@ -228,7 +228,7 @@ GemmPath gemm_path(const GemmArgs& g) {
   // otherwise: the split-N kernel
   if (g.a_dt == LILICORR_F32 && g.M > 16 && g.M <= 1024 && gemm_rows_supported(g))
     return GemmPath::ROWS;
-  if (g.M > 4 && gemm_split_supported(g)) return GemmPath::SPLIT;
+  if (g.M > 4 && gemm_split_takes(g)) return GemmPath::SPLIT;
   if (g.M <= 64 || (g.a_dt == LILICORR_F32 && g.M <= 1024)) return GemmPath::SKINNY;
   if (gemm_small_supported(g)) return GemmPath::SMALL;
   if (gemm_tc_supported(g)) return GemmPath::TC;

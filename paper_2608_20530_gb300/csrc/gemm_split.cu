@@ -33,6 +33,7 @@ using namespace tc;
 constexpr int SP_THREADS = 256;
 constexpr int SP_STAGES = 4;
 constexpr int SP_BK = 64;
+constexpr int SP_FEW = 64;               // rows up to which sums leave the tensor core early
 constexpr uint32_t SP_A_BYTES = 128 * SP_BK * 2;
 constexpr long long SP_WAIT = 4000000000ll;
 constexpr float SP_RMS_EPS = 1e-6f;
@@ -43,8 +44,12 @@ struct SplitArgs {
   int w_const;       // W is constant: its copies may start before the preceding launch ends
 };
 
-template <int BN>
+template <int BN, bool FEW>
 struct SpCfg {
+  // two CTAs fit an SM by shared memory: their columns must too, or clusters could hold one
+  // another up at the allocation
+  static constexpr uint32_t TMEM_COLS = FEW ? 4 * BN : BN;
+  static_assert(2 * TMEM_COLS <= 512, "two CTAs an SM");
   static constexpr uint32_t B_BYTES = BN * SP_BK * 2;
   static constexpr size_t RING = (size_t)SP_STAGES * (SP_A_BYTES + B_BYTES);
   static constexpr int PLD = BN + 4;                       // row stride of the partial sums
@@ -52,11 +57,34 @@ struct SpCfg {
   static constexpr size_t SMEM = 1024 + RING;
 };
 
-template <int BN>
-__global__ void __launch_bounds__(SP_THREADS, 1)
+// v += x; with COMP, e gathers the sum's rounding error (Knuth's two-sum).
+template <bool COMP>
+__device__ __forceinline__ void add_part(float& v, float& e, float x) {
+  const float s = __fadd_rn(v, x);
+  if (COMP) {
+    const float b = __fsub_rn(s, v);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(v, __fsub_rn(s, b)), __fsub_rn(x, b)));
+  }
+  v = s;
+}
+
+// FEW (M <= 64): the sums of a product of few rows are held to what the few-row CUDA-core kernel,
+// which had these sizes, gives. The tensor core truncates each time it adds 16 products to an
+// accumulator, always towards zero, so a chain of n adds is about n * 1.2e-8 of the result
+// short (measured: 2.4e-8 after two, 9.5e-8 after eight, 4.0e-7 after 32). Here an accumulator takes
+// two adds, two accumulators a 64-wide chunk, two chunks in flight, and a thread per row adds
+// them up in fp32 registers. Relative error against 64 bits, few-row kernel / one chain / this, at
+// Kd = 512, 1024, 2048 and 4096:
+// 6.2e-8 / 1.2e-7 / 6.1e-8, 6.9e-8 / 2.3e-7 / 6.8e-8, 7.9e-8 / 4.7e-7 / 7.8e-8, 8.4e-8 / 4.7e-7 / 7.8e-8
+// (the ranks' parts are added with their rounding errors carried). It costs a product 0.4 to 1.3 us
+// (64 x 1024 x 1024: 4.5 -> 5.3 us, the few-row kernel 25.7; 16 x 1024 x 4096: 5.5 -> 6.8, 11.9), a
+// whole network of up to 64 nodes about a tenth (width 512, 48 nodes: 70 -> 77 us; 230 with the
+// few-row kernel).
+template <int BN, bool FEW>
+__global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
     gemm_split_kernel(const __grid_constant__ CUtensorMap mapA,
                       const __grid_constant__ CUtensorMap mapW, const SplitArgs sa) {
-  using Cfg = SpCfg<BN>;
+  using Cfg = SpCfg<BN, FEW>;
   constexpr int PLD = Cfg::PLD;
   const GemmArgs& g = sa.g;
   extern __shared__ uint8_t smem_raw[];
@@ -65,7 +93,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
   uint8_t* sA = smem;
   uint8_t* sB = smem + SP_STAGES * SP_A_BYTES;
   float* part = reinterpret_cast<float*>(smem);            // once the products are done
-  __shared__ __align__(8) uint64_t full[SP_STAGES], empty[SP_STAGES], acc_full;
+  __shared__ __align__(8) uint64_t full[SP_STAGES], empty[SP_STAGES], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base;
   __shared__ volatile int abort_flag;
 
@@ -74,17 +102,21 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
   const int n0 = blockIdx.y * BN, m0 = blockIdx.z * 128;
   const int nk = (g.Kd + SP_BK - 1) / SP_BK;
   const int kc0 = nk * rank / S, kcn = nk * (rank + 1) / S - kc0;   // this CTA's chunks (>= 1)
+  const int rows = min(128, g.M - m0);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < SP_STAGES; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(&acc_full, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], (rows + 31) / 32);      // FEW: the warps that drain
+    }
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(&tmem_base, BN);
+  if (warp == 1) tmem_alloc(&tmem_base, Cfg::TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -108,7 +140,6 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
   // this thread's columns in the reduction, and what it adds to them
   constexpr int TPR = BN / 4;                       // threads per row
   const int c = (threadIdx.x % TPR) * 4, n = n0 + c;
-  const int rows = min(128, g.M - m0);
   const bool col_ok = n < g.N;                      // N is a multiple of 8
   float4 bias = make_float4(0.f, 0.f, 0.f, 0.f), gain = bias;
   auto load_vectors = [&] {
@@ -159,29 +190,80 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
         tc_fence_after();
         const uint64_t ad = smem_desc(sA + (size_t)s * SP_A_BYTES);
         const uint64_t bd = smem_desc(sB + (size_t)s * Cfg::B_BYTES);
+        if constexpr (FEW) {
+          const int b = i & 1;
+          if (!mbar_wait(&acc_empty[b], ((i >> 1) & 1) ^ 1, SP_WAIT)) {
+            abort_flag = 1;
+            break;
+          }
+          tc_fence_after();
 #pragma unroll
-        for (int k = 0; k < SP_BK / 16; ++k)
-          mma_bf16(tmem, ad + 2ull * k, bd + 2ull * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
-        mma_commit(&empty[s]);
+          for (int k = 0; k < SP_BK / 16; ++k)
+            mma_bf16(tmem + (2 * b + (k >> 1)) * BN, ad + 2ull * k, bd + 2ull * k, idesc, k & 1);
+          mma_commit(&empty[s]);
+          mma_commit(&acc_full[b]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < SP_BK / 16; ++k)
+            mma_bf16(tmem, ad + 2ull * k, bd + 2ull * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
+          mma_commit(&empty[s]);
+        }
       }
-      mma_commit(&acc_full);
+      if (!FEW) mma_commit(&acc_full[0]);
     }
   } else if (warp >= 4) {
     // ---- partial sums of this CTA's part of Kd: thread = row. Every copy has landed and been
     //      multiplied once the accumulator is complete, so they may overwrite the ring.
     const int q = warp & 3, row = q * 32 + lane;
-    if (!mbar_wait(&acc_full, 0, SP_WAIT)) abort_flag = 1;
-    tc_fence_after();
-    if (!abort_flag) {
+    const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
+    if constexpr (FEW) {
+      if (q * 32 < rows) {
+        float sum[BN];
 #pragma unroll
-      for (int c = 0; c < BN; c += 32) {
-        uint32_t r[32];
-        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + c, r);
+        for (int j = 0; j < BN; ++j) sum[j] = 0.f;
+        bool ok = true;
+        for (int i = 0; i < kcn; ++i) {
+          const int b = i & 1;
+          ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (i >> 1) & 1, SP_WAIT));
+          if (!ok) break;
+          tc_fence_after();
 #pragma unroll
-        for (int j = 0; j < 32; j += 4)
-          *reinterpret_cast<float4*>(part + row * PLD + c + j) =
-              make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                          __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+          for (int c = 0; c < BN; c += 16) {
+            uint32_t r0[16], r1[16];
+            tmem_ld16(lanes + 2 * b * BN + c, r0);
+            tmem_ld16(lanes + (2 * b + 1) * BN + c, r1);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) sum[c + j] += __uint_as_float(r0[j]) + __uint_as_float(r1[j]);
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_empty[b]);
+        }
+        if (!ok) {
+          abort_flag = 1;
+        } else {
+#pragma unroll
+          for (int j = 0; j < BN; j += 4)
+            *reinterpret_cast<float4*>(part + row * PLD + j) =
+                make_float4(sum[j], sum[j + 1], sum[j + 2], sum[j + 3]);
+        }
+      }
+    } else {
+      const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[0], 0, SP_WAIT));
+      tc_fence_after();
+      if (!ok) {
+        abort_flag = 1;
+      } else {
+#pragma unroll
+        for (int c = 0; c < BN; c += 32) {
+          uint32_t r[32];
+          tmem_ld32(lanes + c, r);
+#pragma unroll
+          for (int j = 0; j < 32; j += 4)
+            *reinterpret_cast<float4*>(part + row * PLD + c + j) =
+                make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
+                            __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+        }
       }
     }
     tc_fence_before();
@@ -203,9 +285,16 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
 #pragma unroll
     for (int p = 0; p < 8; ++p)
       if (p < S) t[p] = ld_cluster_f4(local, p);
+    float4 e = make_float4(0.f, 0.f, 0.f, 0.f);     // FEW: what the adds round off
 #pragma unroll
     for (int p = 0; p < 8; ++p)
-      if (p < S) { v.x += t[p].x; v.y += t[p].y; v.z += t[p].z; v.w += t[p].w; }
+      if (p < S) {
+        add_part<FEW>(v.x, e.x, t[p].x);
+        add_part<FEW>(v.y, e.y, t[p].y);
+        add_part<FEW>(v.z, e.z, t[p].z);
+        add_part<FEW>(v.w, e.w, t[p].w);
+      }
+    if (FEW) { v.x += e.x; v.y += e.y; v.z += e.z; v.w += e.w; }
     return v;
   };
   auto finish_row = [&](int i, const float4& v, const float4& rr) {
@@ -230,7 +319,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
       x.x += br.x; x.y += br.y; x.z += br.z; x.w += br.w;
     }
     if (g.act == ACT_SILU) {
-      if (g.c_dt == LILICORR_BF16) {
+      if (!FEW && g.c_dt == LILICORR_BF16) {          // (few rows: exp, as the few-row kernel)
         x.x = silu_tanh(x.x); x.y = silu_tanh(x.y); x.z = silu_tanh(x.z); x.w = silu_tanh(x.w);
       } else {
         x.x = silu_f(x.x); x.y = silu_f(x.y); x.z = silu_f(x.z); x.w = silu_f(x.w);
@@ -293,14 +382,14 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, BN);
+    tmem_dealloc(tmem, Cfg::TMEM_COLS);
   }
 }
 
-template <int BN>
+template <int BN, bool FEW>
 lilicorr_status_t launch_split(const GemmArgs& g, int S, cudaStream_t st) {
   static bool configured[64] = {false};
-  LL_TRY(allow_max_dynamic_smem(gemm_split_kernel<BN>, configured));
+  LL_TRY(allow_max_dynamic_smem(gemm_split_kernel<BN, FEW>, configured));
   CUtensorMap ma, mw;
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   if (!make_map(&ma, g.A, bf, 2, g.M, g.Kd, g.lda, 128, SP_BK)) return LILICORR_ERR_CUDA;
@@ -309,8 +398,9 @@ lilicorr_status_t launch_split(const GemmArgs& g, int S, cudaStream_t st) {
   sa.g = g;
   sa.S = S;
   sa.w_const = g.w_const;
-  return launch_cluster_k(gemm_split_kernel<BN>, dim3(S, ceil_div(g.N, BN), ceil_div(g.M, 128)),
-                          SP_THREADS, SpCfg<BN>::SMEM, S, st, ma, mw, sa);
+  return launch_cluster_k(gemm_split_kernel<BN, FEW>,
+                          dim3(S, ceil_div(g.N, BN), ceil_div(g.M, 128)), SP_THREADS,
+                          SpCfg<BN, FEW>::SMEM, S, st, ma, mw, sa);
 }
 
 int split_tiles(const GemmArgs& g, int bn) { return ceil_div(g.M, 128) * ceil_div(g.N, bn); }
@@ -346,9 +436,19 @@ bool gemm_split_supported(const GemmArgs& g) {
   return gemm_split_ways(g) > 0;
 }
 
+// Whether the network gives a product to this kernel. Up to 64 rows only where its error is no
+// larger than the few-row kernel's: Kd over at least four CTAs (shorter sums are closer there: 2560
+// columns x Kd 328, two CTAs 6.3e-8 against 5.7e-8), 16 chunks each at most.
+bool gemm_split_takes(const GemmArgs& g) {
+  if (!gemm_split_supported(g)) return false;
+  const int S = gemm_split_ways(g);
+  return g.M > SP_FEW || (S >= 4 && ceil_div(g.Kd, SP_BK) <= 16 * S);
+}
+
 lilicorr_status_t launch_gemm_split(const GemmArgs& g, cudaStream_t st) {
   if (g.M == 0 || g.N == 0) return LILICORR_OK;
-  return launch_split<64>(g, gemm_split_ways(g), st);
+  const int S = gemm_split_ways(g);
+  return g.M <= SP_FEW ? launch_split<64, true>(g, S, st) : launch_split<64, false>(g, S, st);
 }
 
 }  // namespace lilicorr

@@ -334,6 +334,7 @@ bool gemm_tc_supported(const GemmArgs& g);
 lilicorr_status_t launch_gemm_tc(const GemmArgs& g, cudaStream_t st);
 // few output tiles: Kd split over a cluster (gemm_split.cu)
 bool gemm_split_supported(const GemmArgs& g);
+bool gemm_split_takes(const GemmArgs& g);      // and is the network's choice
 int gemm_split_ss_slots(int N);
 lilicorr_status_t launch_gemm_split(const GemmArgs& g, cudaStream_t st);
 // one tile of rows (M <= 128, Kd <= 512, a multiple of 64): whole-K TMA copies (gemm_small.cu)

@@ -459,17 +459,6 @@ constexpr uint32_t LS_TMEM_COLS = 32;      // two 16-column accumulators
 // ord_f32(x) > ord_f32(y)
 __device__ __forceinline__ uint32_t ord_f32(float v) { return (uint32_t)(make_key(v, 0u) >> 32); }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32"
-      " {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 __device__ __forceinline__ void ls_bar() {  // the four epilogue warps
   asm volatile("bar.sync 1, %0;" ::"n"(LH_EPI) : "memory");
 }
