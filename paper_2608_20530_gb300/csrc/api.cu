@@ -235,9 +235,11 @@ GemmPath gemm_path(const GemmArgs& g) {
   return GemmPath::SIMT;
 }
 
-// Whether g, with its folded RMSNorm, runs on a kernel that folds it.
+// Whether g, with its folded RMSNorm, runs on a kernel that folds it, and no faster one would take
+// the product without.
 bool folds(const GemmArgs& g) {
-  return gemm_path(g) == GemmPath::SPLIT || (g.M > 64 && gemm_tc_supported(g));
+  return gemm_path(g) == GemmPath::SPLIT ||
+         (g.M > 64 && !gemm_small_supported(g) && gemm_tc_supported(g));
 }
 
 // Sums of squares per row that a folded producer writes.

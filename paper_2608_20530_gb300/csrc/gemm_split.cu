@@ -436,13 +436,38 @@ bool gemm_split_supported(const GemmArgs& g) {
   return gemm_split_ways(g) > 0;
 }
 
-// Whether the network gives a product to this kernel. Up to 64 rows only where its error is no
-// larger than the few-row kernel's: Kd over at least four CTAs (shorter sums are closer there: 2560
-// columns x Kd 328, two CTAs 6.3e-8 against 5.7e-8), 16 chunks each at most.
+// Whether the network gives a product to this kernel. Measured back to back, us, this kernel (S ways)
+// against what else takes the product:
+//   65-128 rows, Kd = 64 or 256: 5.3-6.1 / 4.7-5.4 (S = 1 / 2), whole-K copies (gemm_small.cu)
+//     3.0-3.8 / 3.5-4.3; Kd = 512, fp32 out: 3.9-4.5 (S = 4) against 4.2-5.3, bf16 out 4.1-4.9 against
+//     4.3-4.5, 48 tiles (S = 2) 5.7-6.0 against 4.5-5.3
+//   more rows, fp32 / bf16 out, persistent kernel: Kd = 64 or 256, 6.0 / 5.9 and 5.1-5.4 / 5.2-5.6 against
+//     4.1 / 3.6 and 4.7-5.0 / 4.2-4.5; Kd = 512, S = 4, 4.3-4.6 / 4.3-4.8 against 5.9 / 5.4, S = 2 with a CTA
+//     an SM 5.8-6.1 / 5.9-6.1 against 5.9-6.1 / 5.4, with two 6.6-7.2 / 6.5-7.2 against 6.0 / 5.5; Kd = 1024, S = 4,
+//     4.8-6.9 / 4.8-7.0 against 8.0 / 7.5, S = 2 with two CTAs an SM 7.4-8.3 / 7.6-8.3 against 8.1 / 7.7;
+//     Kd = 2048, S = 2, 9.5-10.5 against 12.1 / 11.7
+//   5-64 rows, few-row kernel: 3.9-5.2 (Kd = 512 or 1024) against 2.9-4.3 while that is one wave of CTAs,
+//     against 5.3-72 beyond.
+// Where every product folds an RMSNorm, the kernels that the fold saves decide up to 128 rows: on heads
+// of width 64 and 128 this kernel's networks took 1.3 to 1.5 times as long as the unfolded ones with
+// whole-K copies (two requests of 64 nodes at width 128: 99.9 against 66.8 us), on width 320 0.83.
+// Up to 64 rows only where its error is no larger than the few-row kernel's: Kd over at
+// least four CTAs (shorter sums are closer there: 2560 columns x Kd 328, two CTAs 6.3e-8 against
+// 5.7e-8), 16 chunks each at most.
 bool gemm_split_takes(const GemmArgs& g) {
   if (!gemm_split_supported(g)) return false;
-  const int S = gemm_split_ways(g);
-  return g.M > SP_FEW || (S >= 4 && ceil_div(g.Kd, SP_BK) <= 16 * S);
+  const int S = gemm_split_ways(g), nk = ceil_div(g.Kd, SP_BK);
+  const bool fold = g.c2 || g.ss_in;
+  if (g.M <= SP_FEW)
+    return S >= 4 && nk <= 16 * S && (fold || ceil_div(g.N, 4) * ceil_div(g.M, 16) > num_sms());
+  if (fold && g.M <= 128) return nk >= 5;
+  const bool bf16 = g.c_dt == LILICORR_BF16;
+  if (gemm_small_supported(g)) return S >= 4 && !bf16;
+  if (S == 2) {
+    const bool one = 2 * split_tiles(g, 64) <= num_sms();
+    return nk >= (bf16 ? (one ? 14 : 24) : (one ? 8 : 16));
+  }
+  return S >= 4;
 }
 
 lilicorr_status_t launch_gemm_split(const GemmArgs& g, cudaStream_t st) {
