@@ -271,15 +271,18 @@ __device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
   }
 }
 
-template <typename TA, typename TW, typename TC, int MB>
+// TWO: the launch holds two products, the second at blockIdx.z = 1. A kernel of its own: the choice and
+// the narrower product's early exit cost one-product launches too (bf16, 173 -> 255 registers: 16 x
+// 256 x 4096 6.3 -> 9.7 us, 4 x 1536 x 256 2.8 -> 4.5).
+template <typename TA, typename TW, typename TC, int MB, bool TWO>
 __global__ void __launch_bounds__(SK_THREADS) gemm_skinny_kernel(const GemmArgs g0, const GemmArgs g1) {
   pdl_wait();
-  const GemmArgs& g = blockIdx.z ? g1 : g0;         // one launch may hold two products
+  const GemmArgs& g = TWO && blockIdx.z ? g1 : g0;
   __shared__ float red[SK_THREADS / 32][MB * SK_NB];
   const TA* A = static_cast<const TA*>(g.A);
   const TW* W = static_cast<const TW*>(g.W);
   const int n0 = blockIdx.x * SK_NB, m0 = blockIdx.y * MB;
-  if (n0 >= g.N) return;
+  if (TWO && n0 >= g.N) return;
   const int nb = min(SK_NB, g.N - n0), mb = min(MB, g.M - m0);
   float acc[MB][SK_NB];
 #pragma unroll
@@ -357,10 +360,10 @@ struct GrCfg {
   static constexpr int AS = KC + 4;                           // row strides (elements), padded
   static constexpr int WS = KC + 16 / (int)sizeof(TW);        // so 8 lanes' 16-byte reads differ in bank
 };
-template <typename TW, typename TC>
+template <typename TW, typename TC, bool TWO>                   // TWO: as the few-row kernel's
 __global__ void __launch_bounds__(GR_THREADS) gemm_rows_kernel(const GemmArgs g0, const GemmArgs g1) {
   pdl_wait();
-  const GemmArgs& g = blockIdx.z ? g1 : g0;         // one launch may hold two products
+  const GemmArgs& g = TWO && blockIdx.z ? g1 : g0;
   using Cfg = GrCfg<TW>;
   constexpr int KC = Cfg::KC, AS = Cfg::AS, WS = Cfg::WS;
   constexpr int WV = 16 / (int)sizeof(TW);                    // weights per 16-byte piece
@@ -369,7 +372,7 @@ __global__ void __launch_bounds__(GR_THREADS) gemm_rows_kernel(const GemmArgs g0
   const float* A = static_cast<const float*>(g.A);
   const TW* W = static_cast<const TW*>(g.W);
   const int m0 = blockIdx.y * GR_M, n0 = blockIdx.x * GR_N;
-  if (n0 >= g.N) return;
+  if (TWO && n0 >= g.N) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = n0 + lane, r0 = 2 * warp;
   float acc0 = 0.f, acc1 = 0.f;
@@ -425,10 +428,12 @@ __global__ void __launch_bounds__(GR_THREADS) gemm_rows_kernel(const GemmArgs g0
 template <typename TA, typename TW, int MB>
 lilicorr_status_t skinny_dispatch_m(const GemmArgs& g, const GemmArgs* g1, cudaStream_t st) {
   const dim3 grid(ceil_div(g1 ? max(g.N, g1->N) : g.N, SK_NB), ceil_div(g.M, MB), g1 ? 2 : 1);
-  const GemmArgs& h = g1 ? *g1 : g;
+  if constexpr (std::is_same<TA, float>::value)
+    if (g1)                                        // fp32 in and out (launch_gemm_skinny)
+      return launch_k(gemm_skinny_kernel<TA, TW, float, MB, true>, grid, SK_THREADS, 0, st, g, *g1);
   if (g.c_dt == LILICORR_F32)
-    return launch_k(gemm_skinny_kernel<TA, TW, float, MB>, grid, SK_THREADS, 0, st, g, h);
-  return launch_k(gemm_skinny_kernel<TA, TW, __nv_bfloat16, MB>, grid, SK_THREADS, 0, st, g, h);
+    return launch_k(gemm_skinny_kernel<TA, TW, float, MB, false>, grid, SK_THREADS, 0, st, g, g);
+  return launch_k(gemm_skinny_kernel<TA, TW, __nv_bfloat16, MB, false>, grid, SK_THREADS, 0, st, g, g);
 }
 // rows per CTA: one per sequence-level row (M = 1), four for a few, else sixteen
 template <typename TA, typename TW>
@@ -889,24 +894,34 @@ bool gemm_rows_supported(const GemmArgs& g) {
 
 lilicorr_status_t launch_gemm_rows(const GemmArgs& g, cudaStream_t st, const GemmArgs* g1) {
   if (!gemm_rows_supported(g) || (g1 && !gemm_rows_supported(*g1))) return LILICORR_ERR_SHAPE;
+  if (g1 && (g.c_dt != LILICORR_F32 || g1->c_dt != LILICORR_F32)) {
+    LL_TRY(launch_gemm_rows(g, st));
+    return launch_gemm_rows(*g1, st);
+  }
   const dim3 grid(ceil_div(g1 ? max(g.N, g1->N) : g.N, GR_N), ceil_div(g.M, GR_M), g1 ? 2 : 1);
-  const GemmArgs& h = g1 ? *g1 : g;
+  if (g1)
+    return g.w_dt == LILICORR_F32
+               ? launch_k(gemm_rows_kernel<float, float, true>, grid, GR_THREADS, 0, st, g, *g1)
+               : launch_k(gemm_rows_kernel<__nv_bfloat16, float, true>, grid, GR_THREADS, 0, st, g, *g1);
   if (g.w_dt == LILICORR_F32) {
     if (g.c_dt == LILICORR_F32)
-      return launch_k(gemm_rows_kernel<float, float>, grid, GR_THREADS, 0, st, g, h);
-    return launch_k(gemm_rows_kernel<float, __nv_bfloat16>, grid, GR_THREADS, 0, st, g, h);
+      return launch_k(gemm_rows_kernel<float, float, false>, grid, GR_THREADS, 0, st, g, g);
+    return launch_k(gemm_rows_kernel<float, __nv_bfloat16, false>, grid, GR_THREADS, 0, st, g, g);
   }
   if (g.c_dt == LILICORR_F32)
-    return launch_k(gemm_rows_kernel<__nv_bfloat16, float>, grid, GR_THREADS, 0, st, g, h);
-  return launch_k(gemm_rows_kernel<__nv_bfloat16, __nv_bfloat16>, grid, GR_THREADS, 0, st, g, h);
+    return launch_k(gemm_rows_kernel<__nv_bfloat16, float, false>, grid, GR_THREADS, 0, st, g, g);
+  return launch_k(gemm_rows_kernel<__nv_bfloat16, __nv_bfloat16, false>, grid, GR_THREADS, 0, st, g, g);
 }
 
 lilicorr_status_t launch_gemm_skinny(const GemmArgs& g, cudaStream_t st, const GemmArgs* g1) {
   if (g.M == 0 || g.N == 0) return LILICORR_OK;
-  if ((g.Kd % 8) || (g.lda % 8) || (g.ldw % 8) || (g1 && g1->ldw % 8)) {
-    LL_TRY(launch_gemm_simt(g, st));
-    return g1 ? launch_gemm_simt(*g1, st) : LILICORR_OK;
+  // two products in one launch: fp32 in and out, rows in whole groups of eight
+  if (g1 && (g.a_dt != LILICORR_F32 || g.c_dt != LILICORR_F32 || g1->c_dt != LILICORR_F32 ||
+             g.Kd % 8 || g.lda % 8 || g.ldw % 8 || g1->ldw % 8)) {
+    LL_TRY(launch_gemm_skinny(g, st));
+    return launch_gemm_skinny(*g1, st);
   }
+  if ((g.Kd % 8) || (g.lda % 8) || (g.ldw % 8)) return launch_gemm_simt(g, st);
   if (g.a_dt == LILICORR_F32) return skinny_dispatch_w<float>(g, g1, st);
   return skinny_dispatch_w<__nv_bfloat16>(g, g1, st);
 }
