@@ -1040,9 +1040,14 @@ lilicorr_status_t launch_attention(const float* qkv, int B, int L, int K, int D,
   const size_t most = SMEM_PER_BLOCK_MAX - 2 * LILICORR_MAX_L * sizeof(float);
   int warps = 8;
   while (warps > 2 && attention_floats(LK, hd, warps) * sizeof(float) > most) warps /= 2;
-  const size_t smem = (attention_floats(LK, hd, warps) + 2 * L - 1) * sizeof(float);
   // one query a warp while that is one wave of CTAs, else four
   const int aq = (long long)B * n_heads * ceil_div(LK, warps) <= num_sms() ? 1 : 4;
+  // More (sequence, head) pairs than SMs: no warps without a query, so that more CTAs fit an SM
+  // (whole networks of width 64 and 1024 sequences of 4, 8, 16, 32 nodes: 256 -> 155, 328 -> 233,
+  // 442 -> 396, 721 -> 725 us; one query a warp as before AQ = 4: 168, 261, 458, 839). In one wave
+  // the idle warps help to bring K and V (16 sequences of 12 nodes, width 256: 115, without 120).
+  if ((long long)B * n_heads > num_sms()) warps = min(warps, ceil_div(LK, aq));
+  const size_t smem = (attention_floats(LK, hd, warps) + 2 * L - 1) * sizeof(float);
   // split the queries of a (sequence, head) over CTAs until the grid covers the GPU; each warp
   // takes whole groups of AQ
   int qblocks = aq == 1 ? ceil_div(LK, warps) : ceil_div(4 * num_sms(), B * n_heads);

@@ -66,6 +66,13 @@ def test_fp32_attention_one_query(B, L, K, D):
     _network_matches_oracle(B, L, K, D)
 
 
+# more (sequence, head) pairs than SMs: a CTA of one warp, of two, of an odd number, of all eight
+@pytest.mark.parametrize("B,L,K,D", [(20, 1, 3, 64), (24, 4, 2, 64), (20, 3, 3, 256), (21, 7, 3, 64),
+                                     (20, 8, 4, 64)])
+def test_fp32_attention_many_short_sequences(B, L, K, D):
+    _network_matches_oracle(B, L, K, D)
+
+
 def _network_matches_oracle(B, L, K, D):
     ll = _ll()
     wl = workloads.Workload(f"fp32_b{B}_l{L}_k{K}_d{D}", B=B, L=L, V=2000, K=K, d=D, H=128,
