@@ -77,8 +77,14 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p, int r, int rows,
 // VEC: rows of both operands in whole aligned groups of four elements
 // SPLIT: the CTAs of a cluster take a part of Kd's steps each (at least one) and then a part of
 // the tile's rows each, whose sums they read from one another
-template <typename TA, typename TW, typename TC, bool VEC, bool SPLIT>
-__global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g, int ways) {
+// PER_SM: CTAs an SM holds. Two (128 registers) from two tiles an SM on, so that one's first loads and
+// last sums run beside the other's products: with one such products of short Kd took longer than 4 x 4
+// outputs a thread at four CTAs an SM had (65,536 x 256 x 64: 100 us, one 170, two 106;
+// 32,768 x 512 x 32: 70, 143, 89), and long ones gain too (8192 x 512 x 512: 121, two 111). In one wave
+// one is ahead (2048 x 256 x 256: 11.0, two 11.9); in less than two the first SMs to come free would
+// take two each (network of width 512, four sequences of 100 nodes, 168 tiles: 267 us, with two 283).
+template <typename TA, typename TW, typename TC, bool VEC, bool SPLIT, int PER_SM = 1>
+__global__ void __launch_bounds__(G_THREADS, PER_SM) gemm_simt_kernel(GemmArgs g, int ways) {
   pdl_wait();
   constexpr int LDT = GB_M + 4, KG = GB_K / G_GROUPS;
   static_assert(GB_M == GB_N && GB_M * GB_K == 8 * G_THREADS, "two groups of four a thread");
@@ -217,6 +223,11 @@ __global__ void __launch_bounds__(G_THREADS, 1) gemm_simt_kernel(GemmArgs g, int
 
 template <typename TA, typename TW, bool VEC>
 lilicorr_status_t gemm_dispatch_c(const GemmArgs& g, dim3 grid, cudaStream_t st) {
+  if (VEC && (long long)grid.x * grid.y > 2 * num_sms()) {
+    if (g.c_dt == LILICORR_F32)
+      return launch_k(gemm_simt_kernel<TA, TW, float, VEC, false, 2>, grid, G_THREADS, 0, st, g, 1);
+    return launch_k(gemm_simt_kernel<TA, TW, __nv_bfloat16, VEC, false, 2>, grid, G_THREADS, 0, st, g, 1);
+  }
   if (g.c_dt == LILICORR_F32)
     return launch_k(gemm_simt_kernel<TA, TW, float, VEC, false>, grid, G_THREADS, 0, st, g, 1);
   return launch_k(gemm_simt_kernel<TA, TW, __nv_bfloat16, VEC, false>, grid, G_THREADS, 0, st, g, 1);
