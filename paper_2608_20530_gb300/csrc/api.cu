@@ -957,6 +957,14 @@ lilicorr_status_t lilicorr_select_block_walk(const lilicorr_head* head, int B, c
   if (chain) LL_TRY(pro.fork_hidden(call, drafter_hidden));
   LL_TRY(pro.fork_target(call, target_hidden));
   if (!chain) LL_TRY(pro.fork_hidden(call, drafter_hidden));
+  // One or two requests: the target chain ends about with the top-K pass, and a second join inside
+  // the chain of kernels costs more than waiting here (fp32, one request of 8 nodes at D 64: 73.7 ->
+  // 71.7 us, at D 256 80.0 -> 78.0; bf16, 15 x 8 at D 1024: 114.6 -> 112.5; four of 8 x 4, fp32, D 64,
+  // H 4096 would lose, 73.8 -> 76.7)
+  if (chain && B <= 2) {
+    LL_TRY(pro.join_hidden());
+    LL_TRY(pro.join_target());
+  }
   ClusterTail tail;
   tail.anchor = at<float>(ws, w.anc);
   tail.A = at<float>(ws, w.A);
