@@ -51,6 +51,14 @@ lilicorr_status_t lilicorr_test_linear_timeout(const void* A, const void* W, flo
                                                int Kd, long long wait_cycles, uint32_t* status,
                                                cudaStream_t stream);
 
+/* The same of the layer with Kd split over a cluster (path 6; LILICORR_ERR_SHAPE for shapes that it
+ * does not take): no CTA issues its copies, or with first_only the first CTA of every cluster does
+ * not, so that its peers read partial sums that it never wrote. */
+lilicorr_status_t lilicorr_test_linear_split_timeout(const void* A, const void* W, float* C, int M,
+                                                     int N, int Kd, long long wait_cycles,
+                                                     int first_only, uint32_t* status,
+                                                     cudaStream_t stream);
+
 /* Switch for the fused scoring-network kernels (bf16 heads with D = 256, 8 heads,
  * FFN 2D, L*K <= 128): mode 1 (the default) takes the cluster kernel (four CTAs per
  * sequence) while every sequence's cluster fits on the GPU and the one-CTA kernel for

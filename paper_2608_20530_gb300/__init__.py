@@ -81,6 +81,8 @@ _SIGS = {
     "lilicorr_test_linear": (_I, [_P, _I, _I, _P, _I, _I, _P, _I, _I, _I, _I, _I, _P, _P, _I, _I,
                                   _P, _P]),
     "lilicorr_test_linear_timeout": (_I, [_P, _P, _P, _I, _I, _I, ctypes.c_longlong, _P, _P]),
+    "lilicorr_test_linear_split_timeout": (_I, [_P, _P, _P, _I, _I, _I, ctypes.c_longlong, _I, _P,
+                                                _P]),
 }
 
 
@@ -507,6 +509,20 @@ def test_linear_timeout(A: torch.Tensor, W: torch.Tensor, wait_cycles: int,
     _check(lib().lilicorr_test_linear_timeout(A.data_ptr(), W.data_ptr(), C.data_ptr(), M, N, Kd,
                                               int(wait_cycles), status.data_ptr(), _stream()),
            "test_linear_timeout")
+    return C
+
+
+def test_linear_split_timeout(A: torch.Tensor, W: torch.Tensor, wait_cycles: int,
+                              status: torch.Tensor, first_only: bool = False) -> torch.Tensor:
+    """Test hook: test_linear_timeout of the layer with Kd split over a cluster; ``first_only``
+    withholds the copies of every cluster's first CTA only."""
+    M, Kd = A.shape
+    N = W.shape[0]
+    C = torch.empty((M, N), dtype=torch.float32, device=A.device)
+    _check(lib().lilicorr_test_linear_split_timeout(A.data_ptr(), W.data_ptr(), C.data_ptr(), M, N,
+                                                    Kd, int(wait_cycles), int(first_only),
+                                                    status.data_ptr(), _stream()),
+           "test_linear_split_timeout")
     return C
 
 

@@ -35,7 +35,7 @@ constexpr int SP_STAGES = 4;
 constexpr int SP_BK = 64;
 constexpr int SP_FEW = 64;               // rows up to which sums leave the tensor core early
 constexpr uint32_t SP_A_BYTES = 128 * SP_BK * 2;
-constexpr long long SP_WAIT = 4000000000ll;
+constexpr long long SP_WAIT = 4000000000ll;   // SM cycles, where the arguments give no limit
 constexpr float SP_RMS_EPS = 1e-6f;
 
 struct SplitArgs {
@@ -89,7 +89,6 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
   uint8_t* sA = smem;
   uint8_t* sB = smem + SP_STAGES * SP_A_BYTES;
   float* part = reinterpret_cast<float*>(smem);            // once the products are done
-  // (as many as are used: with FEW's four in both, partial row tiles took 0.3 to 0.6 us longer)
   constexpr int NACC = FEW ? 2 : 1;
   __shared__ __align__(8) uint64_t full[SP_STAGES], empty[SP_STAGES], acc_full[NACC], acc_empty[NACC];
   __shared__ uint32_t tmem_base;
@@ -99,6 +98,7 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
   const int S = sa.S, rank = blockIdx.x;                   // gridDim.x = cluster size = S
   const int n0 = blockIdx.y * BN, m0 = blockIdx.z * 128;
   const int nk = (g.Kd + SP_BK - 1) / SP_BK;
+  const long long wait = g.wait_limit > 0 ? g.wait_limit : SP_WAIT;
   const int kc0 = nk * rank / S, kcn = nk * (rank + 1) / S - kc0;   // this CTA's chunks (>= 1)
 
   if (threadIdx.x == 0) {
@@ -128,7 +128,9 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
     const int s = i % SP_STAGES;
     tma_load_2d(sA + (size_t)s * SP_A_BYTES, &mapA, &full[s], (kc0 + i) * SP_BK, m0);
   };
-  const bool producer = warp == 0 && lane == 0;
+  // (a test's starved producer issues no copies: 1 in every CTA, 2 in the cluster's first)
+  const bool starved = g.test_starve == 1 || (g.test_starve == 2 && rank == 0);
+  const bool producer = warp == 0 && lane == 0 && !starved;
   if (producer) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapA)) : "memory");
     if (sa.w_const)
@@ -166,9 +168,9 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
                  : make_float4(0.f, 0.f, 0.f, 0.f);
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (producer) {
       for (int i = pre; i < kcn; ++i) {
-        if (!mbar_wait(&empty[i % SP_STAGES], ((i / SP_STAGES) & 1) ^ 1, SP_WAIT)) {
+        if (!mbar_wait(&empty[i % SP_STAGES], ((i / SP_STAGES) & 1) ^ 1, wait)) {
           abort_flag = 1;
           break;
         }
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
       constexpr uint32_t idesc = instr_desc(128, BN);
       for (int i = 0; i < kcn; ++i) {
         const int s = i % SP_STAGES;
-        if (!mbar_wait(&full[s], (i / SP_STAGES) & 1, SP_WAIT)) {
+        if (!mbar_wait(&full[s], (i / SP_STAGES) & 1, wait)) {
           abort_flag = 1;
           break;
         }
@@ -190,7 +192,7 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
         const uint64_t bd = smem_desc(sB + (size_t)s * Cfg::B_BYTES);
         if constexpr (FEW) {
           const int b = i & 1;
-          if (!mbar_wait(&acc_empty[b], ((i >> 1) & 1) ^ 1, SP_WAIT)) {
+          if (!mbar_wait(&acc_empty[b], ((i >> 1) & 1) ^ 1, wait)) {
             abort_flag = 1;
             break;
           }
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
         bool ok = true;
         for (int i = 0; i < kcn; ++i) {
           const int b = i & 1;
-          ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (i >> 1) & 1, SP_WAIT));
+          ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (i >> 1) & 1, wait));
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
@@ -247,7 +249,7 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
         }
       }
     } else {
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[0], 0, SP_WAIT));
+      const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[0], 0, wait));
       tc_fence_after();
       if (!ok) {
         abort_flag = 1;
@@ -272,11 +274,12 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
   // ---- reduction and epilogue: rows rank, rank + S, ...
   const float ss_scale = 1.0f / (float)(g.ss_dim > 0 ? g.ss_dim : g.Kd);
   // the threads of a row stay together: all run the same number of rounds
-  const int rounds = 128 / (S * (SP_THREADS / TPR));
+  const int rounds = max(1, (FEW ? SP_FEW : 128) / (S * (SP_THREADS / TPR)));
   auto sum_row = [&](int i) {                       // the S partials of a row, in rank order
-    const int r = row_of(i);
+    // threads past the last row sum it too: left out by a branch, a partial row tile took up to 0.7 us
+    // longer (96 x 512 x 512: 4.1 to 4.8 us by how it was compiled, so 4.2)
+    const int r = min(row_of(i), rows - 1);
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r >= rows) return v;
     if (S == 1) return *reinterpret_cast<const float4*>(part + r * PLD + c);
     const uint32_t local = smem_u32(part + r * PLD + c);
     float4 t[8];                                    // every partial in flight, then the sum
@@ -377,7 +380,7 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
     if (threadIdx.x == 0) {
       set_status(g.status, LILICORR_ERR_TIMEOUT);
       const long long t0 = clock64();               // let copies in flight land
-      while (clock64() - t0 < SP_WAIT / 10) {
+      while (clock64() - t0 < wait / 10) {
       }
     }
     __syncthreads();

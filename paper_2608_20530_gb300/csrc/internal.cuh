@@ -302,9 +302,10 @@ struct GemmArgs {
   int w_const;             // W does not change while calls run (a head's weights): its copies
                            // may start before the preceding launch ends
   uint32_t* status;        // device status word (bounded-wait timeouts), may be null
-  long long wait_limit;    // SM cycles per bounded wait of the tensor-core kernel; 0: ~2 s
-  int test_starve;         // test hook only: the tensor-core kernel's producer issues no
-                           // copies, so its consumers' waits run out (see the testing header)
+  long long wait_limit;    // SM cycles per bounded wait of the persistent and the split
+                           // tensor-core kernel; 0: ~2 s
+  int test_starve;         // test hook only: those kernels' producers issue no copies (2: only the
+                           // first CTA's of a cluster), so that their consumers' waits run out
   // RMSNorm folded into the products around it (tensor-core kernel only). Producer (fp32 C):
   // c2 [M, ldc2] (bf16) receives C times c2_gain per column, ss_out [M, SS_LD] partial sums of
   // squares of C's rows (gemm_ss_slots slots per row). Consumer: the product is
