@@ -81,6 +81,8 @@ _SIGS = {
     "lilicorr_test_linear": (_I, [_P, _I, _I, _P, _I, _I, _P, _I, _I, _I, _I, _I, _P, _P, _I, _I,
                                   _P, _P]),
     "lilicorr_test_linear_timeout": (_I, [_P, _P, _P, _I, _I, _I, ctypes.c_longlong, _P, _P]),
+    "lilicorr_test_lm_head_timeout": (_I, [_P, _P, _I, _I, _I, _I, _P, _P, _P, _P, _S,
+                                           ctypes.c_longlong, _I, _P]),
     "lilicorr_test_linear_split_timeout": (_I, [_P, _P, _P, _I, _I, _I, ctypes.c_longlong, _I, _P,
                                                 _P]),
 }
@@ -524,6 +526,23 @@ def test_linear_split_timeout(A: torch.Tensor, W: torch.Tensor, wait_cycles: int
                                                     status.data_ptr(), _stream()),
            "test_linear_split_timeout")
     return C
+
+
+def test_lm_head_timeout(hidden: torch.Tensor, w_vocab: torch.Tensor, K: int, ws: Workspace,
+                         wait_cycles: int, second_only: bool = False) -> None:
+    """Test hook: lm_head_topk on pairs of CTAs with their copies withheld (``second_only``: those of
+    every pair's second CTA), so that its bounded waits run out and ``ws`` holds the timeout
+    status."""
+    rows, H = hidden.shape
+    V = w_vocab.shape[0]
+    ids = torch.empty((rows, K), dtype=torch.int32, device=hidden.device)
+    logp = torch.empty((rows, K), dtype=torch.float32, device=hidden.device)
+    lse = torch.empty((rows,), dtype=torch.float32, device=hidden.device)
+    _check(lib().lilicorr_test_lm_head_timeout(hidden.data_ptr(), w_vocab.data_ptr(), rows, H, V, K,
+                                               ids.data_ptr(), logp.data_ptr(), lse.data_ptr(),
+                                               ws.ptr, ws.nbytes, int(wait_cycles),
+                                               int(second_only), _stream()),
+           "test_lm_head_timeout")
 
 
 def test_attention_path(mode: int) -> int:

@@ -830,6 +830,24 @@ lilicorr_status_t lilicorr_lm_head_topk(const void* hidden, const void* w_vocab,
                              reinterpret_cast<uint32_t*>(w), stream);
 }
 
+lilicorr_status_t lilicorr_test_lm_head_timeout(const void* hidden, const void* w_vocab, int rows,
+                                                int H, int V, int K, int32_t* ids, float* logp,
+                                                float* lse, void* ws, size_t ws_bytes,
+                                                long long wait_cycles, int second_only,
+                                                cudaStream_t stream) {
+  if (rows <= 0 || H <= 0 || V <= 0 || K <= 0 || K > LILICORR_MAX_K || K > V)
+    return LILICORR_ERR_SHAPE;
+  if (wait_cycles < 100000 || wait_cycles > 4000000000ll) return LILICORR_ERR_ARG;
+  if (!lm_head_supported(rows, H, V, K)) return LILICORR_ERR_SHAPE;
+  if (!hidden || !w_vocab || !ids || !logp || !lse || !ws) return LILICORR_ERR_ARG;
+  if (!aligned16(hidden) || !aligned16(w_vocab) || !aligned16(ws)) return LILICORR_ERR_ARG;
+  if (ws_bytes < lilicorr_lm_head_topk_workspace_bytes(rows, H, V, K)) return LILICORR_ERR_WORKSPACE;
+  unsigned char* w = static_cast<unsigned char*>(ws);
+  return launch_lm_head_topk(hidden, w_vocab, rows, H, V, K, w + 256, ids, logp, lse,
+                             reinterpret_cast<uint32_t*>(w), stream, wait_cycles,
+                             second_only ? 2 : 1);
+}
+
 size_t lilicorr_workspace_bytes(const lilicorr_head* head, int B) {
   if (!head || B < 0) return 0;
   return ws_layout(head->desc, B).total;

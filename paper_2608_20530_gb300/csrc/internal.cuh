@@ -282,7 +282,9 @@ bool lm_head_supported(int rows, int H, int V, int K);
 size_t lm_head_records_bytes(int rows, int V, int K);
 lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, int rows, int H,
                                       int V, int K, void* recs, int32_t* ids, float* logp,
-                                      float* lse, uint32_t* status, cudaStream_t st);
+                                      float* lse, uint32_t* status, cudaStream_t st,
+                                      // of the paired kernel, as in GemmArgs (2: the second CTAs)
+                                      long long wait_limit = 0, int test_starve = 0);
 // merge P partial records per row, record p of row r at partials + p * ld_p + r * ld_row
 lilicorr_status_t launch_topk_merge(const void* partials, size_t ld_p, size_t ld_row, int P,
                                     int rows, int K, int32_t* ids, float* logp, float* lse,

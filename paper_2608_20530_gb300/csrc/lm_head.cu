@@ -292,7 +292,7 @@ constexpr size_t LP_SMEM = 1024 + (size_t)LP_STAGES * 2 * LP_HALF;
 __global__ void __launch_bounds__(LH_THREADS, 1)
     lm_head_pair_kernel(const __grid_constant__ CUtensorMap mapA,
                         const __grid_constant__ CUtensorMap mapW, LhShape sh,
-                        unsigned char* __restrict__ recs, uint32_t* status) {
+                        unsigned char* __restrict__ recs, uint32_t* status, long long wait, int starve) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -333,7 +333,8 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
 
   if (warp == 0) {
     // ---- producer of this CTA's halves
-    if (lane == 0) {
+    // (a test's starved producer issues no copies: 1 in both CTAs, 2 in the second)
+    if (lane == 0 && starve != 1 && !(starve == 2 && rank == 1)) {
       const int m0 = (2 * mt + (int)rank) * LH_BM;
       uint32_t g = 0;
       for (int nt = n_first; nt < sh.tiles_n && !abort_flag; nt += per) {
@@ -341,7 +342,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
         for (int i = 0; i < nk; ++i, ++g) {
           const int s = (int)(g % LP_STAGES);
           const uint32_t ph = (g / LP_STAGES) & 1u;
-          if (!mbar_wait_cluster(&empty[s], ph ^ 1u, LH_WAIT)) {
+          if (!mbar_wait_cluster(&empty[s], ph ^ 1u, wait)) {
             abort_flag = 1;
             break;
           }
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
       }
       // the last commits arrive here from the first CTA: none may be under way at the exit
       for (uint32_t j = g > LP_STAGES ? g - LP_STAGES : 0; j < g && !abort_flag; ++j)
-        if (!mbar_wait_cluster(&empty[j % LP_STAGES], (j / LP_STAGES) & 1u, LH_WAIT)) abort_flag = 1;
+        if (!mbar_wait_cluster(&empty[j % LP_STAGES], (j / LP_STAGES) & 1u, wait)) abort_flag = 1;
     }
   } else if (warp == 1) {
     // ---- MMA issuer: the first CTA's lane, for both
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
       uint32_t g = 0, lt = 0;
       for (int nt = n_first; nt < sh.tiles_n && !abort_flag; nt += per, ++lt) {
         const uint32_t acc = lt & 1u;
-        if (!mbar_wait_cluster(&acc_empty[acc], ((lt >> 1) & 1u) ^ 1u, LH_WAIT)) {
+        if (!mbar_wait_cluster(&acc_empty[acc], ((lt >> 1) & 1u) ^ 1u, wait)) {
           abort_flag = 1;
           break;
         }
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
         for (int i = 0; i < nk; ++i, ++g) {
           const int s = (int)(g % LP_STAGES);
           const uint32_t ph = (g / LP_STAGES) & 1u;
-          if (!mbar_wait_cluster(&full[s], ph, LH_WAIT)) {
+          if (!mbar_wait_cluster(&full[s], ph, wait)) {
             abort_flag = 1;
             break;
           }
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
     uint32_t lt = 0;
     for (int nt = n_first; nt < sh.tiles_n; nt += per, ++lt) {
       const uint32_t acc = lt & 1u;
-      if (!abort_flag && !mbar_wait_cluster(&acc_full[acc], (lt >> 1) & 1u, LH_WAIT)) abort_flag = 1;
+      if (!abort_flag && !mbar_wait_cluster(&acc_full[acc], (lt >> 1) & 1u, wait)) abort_flag = 1;
       tc_fence_after();
       lh_fold_tile(tmem + ((uint32_t)(q * 32) << 16) + acc * LH_BN, nt * LH_BN, sh,
                    valid && !abort_flag, row, s_list, st, [&] {
@@ -421,7 +422,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
     if (threadIdx.x == 0) {
       set_status(status, LILICORR_ERR_TIMEOUT);
       const long long t0 = clock64();          // let copies in flight land
-      while (clock64() - t0 < LH_WAIT / 10) {
+      while (clock64() - t0 < wait / 10) {
       }
     }
     __syncthreads();
@@ -740,10 +741,12 @@ size_t lm_head_records_bytes(int rows, int V, int K) {
 
 lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, int rows, int H,
                                       int V, int K, void* recs, int32_t* ids, float* logp,
-                                      float* lse, uint32_t* status, cudaStream_t st) {
+                                      float* lse, uint32_t* status, cudaStream_t st,
+                                      long long wait_limit, int test_starve) {
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   LhShape sh;
   sh.rows = rows; sh.H = H; sh.V = V; sh.K = K;
+  if (test_starve && (rows <= LS_BN || !lm_head_plan(rows, V).pair)) return LILICORR_ERR_SHAPE;
   if (rows <= LS_BN) {
     // few rows: vocabulary tiles as the A operand, the hidden rows as B (N = 16)
     static bool configured_rows[64] = {false};
@@ -769,7 +772,8 @@ lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, i
     static bool configured_pair[64] = {false};
     LL_TRY(allow_max_dynamic_smem(lm_head_pair_kernel, configured_pair));
     LL_TRY(launch_cluster_k(lm_head_pair_kernel, p.grid, LH_THREADS, LP_SMEM, 2, st, ma, mw, sh,
-                            static_cast<unsigned char*>(recs), status));
+                            static_cast<unsigned char*>(recs), status,
+                            wait_limit > 0 ? wait_limit : LH_WAIT, test_starve));
   } else {
     if (!make_map(&ma, hidden, bf, 2, rows, H, H, LH_BM, LH_BK)) return LILICORR_ERR_CUDA;
     if (!make_map(&mw, w_vocab, bf, 2, V, H, H, LH_BN, LH_BK)) return LILICORR_ERR_CUDA;

@@ -51,3 +51,36 @@ def test_split_hook_rejects_unbounded_limits():
     for bad in (0, 10, 10**12):
         with pytest.raises(ll.LilicorrError):
             ll.test_linear_split_timeout(A, A, bad, status)
+
+
+# a tile a pair and several, fewer steps of H than stages and more, a pair whose second CTA has no rows
+@pytest.mark.parametrize("rows,H,V,K", [(129, 64, 257, 4), (256, 512, 39000, 8), (257, 192, 9000, 8),
+                                        (400, 1024, 40000, 16)])
+@pytest.mark.parametrize("second_only", [False, True])
+def test_lm_head_pair_times_out(rows, H, V, K, second_only):
+    ll = _ll()
+    g = torch.Generator(device="cuda").manual_seed(rows + V)
+    hid = torch.randn((rows, H), generator=g, device="cuda").to(torch.bfloat16)
+    w = (H ** -0.5 * 4 * torch.randn((V, H), generator=g, device="cuda")).to(torch.bfloat16)
+    ws = ll.Workspace(int(ll.lib().lilicorr_lm_head_topk_workspace_bytes(rows, H, V, K)))
+    want = ll.lm_head_topk(hid, w, K, ws=ws)
+    assert ws.status() == 0
+    for _ in range(2):
+        t0 = time.perf_counter()
+        ll.test_lm_head_timeout(hid, w, K, ws, LIMIT, second_only)
+        assert ws.status() == TIMEOUT                  # reads and clears it
+        dt = time.perf_counter() - t0
+        assert dt < 5.0, f"the timed-out call took {dt:.2f} s"
+        got = ll.lm_head_topk(hid, w, K, ws=ws)
+        assert ws.status() == 0
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+def test_lm_head_hook_rejects_other_kernels_and_limits():
+    ll = _ll()
+    h = torch.zeros((384, 64), device="cuda", dtype=torch.bfloat16)
+    w = torch.zeros((39000, 64), device="cuda", dtype=torch.bfloat16)
+    ws = ll.Workspace(1 << 24)
+    for rows, limit in ((16, LIMIT), (100, LIMIT), (256, 10), (256, 10 ** 12)):
+        with pytest.raises(ll.LilicorrError):
+            ll.test_lm_head_timeout(h[:rows], w, 4, ws, limit)
