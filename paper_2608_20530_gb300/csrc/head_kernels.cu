@@ -544,6 +544,10 @@ target_norm_kernel(const T* __restrict__ Tin, int n_tgt, int H, const float* __r
 //                                 layer is a linear launch that adds into x)
 //   x  = fold[id_k] + hproj[r] + slot[s] + rank[k]
 // with f_k = [logp_k, exp(logp_k), logp_0 - logp_k, k / (K-1), 1{k = 0}].
+constexpr int NODE_COLS_MAX = 1984;
+static_assert(NODE_COLS_MAX * (LILICORR_N_CONF + 1) * sizeof(float) +
+              LILICORR_MAX_K * (LILICORR_N_CONF + 1) * sizeof(float) <= 48 * 1024,
+              "staged weights and the static arrays");
 template <typename TC1>
 __global__ void node_build_kernel(int L, int K, int D, int cols, int V,
                                   const int32_t* __restrict__ ids,
@@ -992,7 +996,10 @@ lilicorr_status_t launch_node_build(const lilicorr_head* h, int B, const int32_t
   // Few slot rows: their columns over several CTAs, at least 128 each, until two an SM (one
   // request of 15 slots x 8 candidates x 1024: 15 CTAs of eight rounds of gathers, 14.1 us cold,
   // to 120 of one, 5.8). Many rows keep one CTA each, which stages the confidence weights once.
-  const int parts = max(1, min(ceil_div(2 * num_sms(), B * d.L), d.D / 128));
+  // Wide heads are split for any number of rows: a CTA stages 24 bytes a column in the 48 KB that a
+  // launch may have unasked.
+  const int parts = max(ceil_div(d.D, NODE_COLS_MAX),
+                        min(ceil_div(2 * num_sms(), B * d.L), d.D / 128));
   const int cols = ceil_div(ceil_div(d.D, parts), 4) * 4;
   const dim3 grid(B * d.L, ceil_div(d.D, cols));
   const size_t smem = sizeof(float) * (LILICORR_N_CONF + 1) * cols;
