@@ -62,7 +62,7 @@ lilicorr_status_t lilicorr_test_linear_split_timeout(const void* A, const void* 
 /* lilicorr_lm_head_topk with the copies of its paired kernel withheld, in both CTAs of a pair or with
  * second_only in the second one, and a limit as above: the workspace's status word receives
  * LILICORR_ERR_TIMEOUT, the outputs unspecified values. LILICORR_ERR_SHAPE where another kernel takes
- * the call (128 rows or fewer, and row counts that single CTAs take in fewer rounds). */
+ * the call (128 rows or fewer, H below 2048, and row counts that single CTAs take in fewer rounds). */
 lilicorr_status_t lilicorr_test_lm_head_timeout(const void* hidden, const void* w_vocab, int rows,
                                                 int H, int V, int K, int32_t* ids, float* logp,
                                                 float* lse, void* ws, size_t ws_bytes,

@@ -812,7 +812,7 @@ lilicorr_status_t lilicorr_topk_lse_merge(const void* partials, int P, int rows,
 
 size_t lilicorr_lm_head_topk_workspace_bytes(int rows, int H, int V, int K) {
   if (!lm_head_supported(rows, H, V, K)) return 0;
-  return 256 + align_up(lm_head_records_bytes(rows, V, K), 256);
+  return 256 + align_up(lm_head_records_bytes(rows, H, V, K), 256);
 }
 
 lilicorr_status_t lilicorr_lm_head_topk(const void* hidden, const void* w_vocab, int rows, int H,

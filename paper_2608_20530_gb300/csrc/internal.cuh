@@ -279,7 +279,7 @@ __device__ __forceinline__ int32_t key_id(uint64_t k) {
 }
 // LM-head projection fused with step (1) (lm_head.cu): records [rows][P] in ws, then merged
 bool lm_head_supported(int rows, int H, int V, int K);
-size_t lm_head_records_bytes(int rows, int V, int K);
+size_t lm_head_records_bytes(int rows, int H, int V, int K);
 lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, int rows, int H,
                                       int V, int K, void* recs, int32_t* ids, float* logp,
                                       float* lse, uint32_t* status, cudaStream_t st,

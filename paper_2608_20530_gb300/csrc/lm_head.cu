@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(LH_THREADS, 1)
 }
 
 // ----------------------------------------------------------------------------- many rows
-// More than 128 rows: two CTAs of a cluster (one tensor-core pair, cta_group::2) share a tile of
+// More than 128 rows at long H: two CTAs of a cluster (one tensor-core pair, cta_group::2) share a tile of
 // 256 rows x 256 vocabulary entries. Each keeps 128 of the rows and brings 128 of the W_vocab
 // rows, so a step of H costs it two thirds of the copies and shared memory of a CTA on its own
 // for the same products. The first CTA's MMA lane issues for both; its `full` barriers count
@@ -710,10 +710,14 @@ LhPlan lm_head_plan_of(int rows, int V, bool pair) {
 // A tile of a pair takes about 0.87 of the time of a tile of one CTA (151,936 x 4096: 25.4
 // against 29.2 us at 500 rows, 23.3 against 27.1 at 1024), so pairs win unless an odd number of
 // 128-row blocks makes them walk more tiles (384 rows: 16 a pair, 12 a CTA, 425 against 362 us;
-// 640 rows: 24 and 20, 583 against 563).
-LhPlan lm_head_plan(int rows, int V) {
+// 640 rows: 24 and 20, 583 against 563). That is the copies' time: at short H a tile is bound by its
+// epilogue, which pairs do not shorten. Pairs against single CTAs with as many tiles each, 129 to 1024
+// rows, V = 32,000 and 151,936: 1.00 to 1.03 at H = 512 and 1024, 0.97 to 1.00 and 0.82 to 0.99 at 2048,
+// 0.92 to 0.98 and 0.70 to 0.95 at 4096.
+constexpr int LP_MIN_H = 2048;
+LhPlan lm_head_plan(int rows, int H, int V) {
   const LhPlan one = lm_head_plan_of(rows, V, false);
-  if (rows <= LH_BM) return one;
+  if (rows <= LH_BM || H < LP_MIN_H) return one;
   const LhPlan two = lm_head_plan_of(rows, V, true);
   return 87 * ceil_div(two.tiles_n, two.per) <= 100 * ceil_div(one.tiles_n, one.per) ? two : one;
 }
@@ -734,9 +738,9 @@ bool lm_head_supported(int rows, int H, int V, int K) {
          encode_fn() != nullptr;
 }
 
-size_t lm_head_records_bytes(int rows, int V, int K) {
+size_t lm_head_records_bytes(int rows, int H, int V, int K) {
   if (rows <= LS_BN) return (size_t)lm_head_rows_grid(V) * rows * topk_partial_bytes(K);
-  return (size_t)lm_head_plan(rows, V).per * rows * topk_partial_bytes(K);
+  return (size_t)lm_head_plan(rows, H, V).per * rows * topk_partial_bytes(K);
 }
 
 lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, int rows, int H,
@@ -746,7 +750,7 @@ lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, i
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   LhShape sh;
   sh.rows = rows; sh.H = H; sh.V = V; sh.K = K;
-  if (test_starve && (rows <= LS_BN || !lm_head_plan(rows, V).pair)) return LILICORR_ERR_SHAPE;
+  if (test_starve && (rows <= LS_BN || !lm_head_plan(rows, H, V).pair)) return LILICORR_ERR_SHAPE;
   if (rows <= LS_BN) {
     // few rows: vocabulary tiles as the A operand, the hidden rows as B (N = 16)
     static bool configured_rows[64] = {false};
@@ -762,7 +766,7 @@ lilicorr_status_t launch_lm_head_topk(const void* hidden, const void* w_vocab, i
     return launch_topk_merge(recs, topk_partial_bytes(K), grid * topk_partial_bytes(K), grid, rows,
                              K, ids, logp, lse, status, st);
   }
-  const LhPlan p = lm_head_plan(rows, V);
+  const LhPlan p = lm_head_plan(rows, H, V);
   sh.tiles_m = p.tiles_m;
   sh.tiles_n = p.tiles_n;
   const int per = p.per;

@@ -53,9 +53,9 @@ def test_split_hook_rejects_unbounded_limits():
             ll.test_linear_split_timeout(A, A, bad, status)
 
 
-# a tile a pair and several, fewer steps of H than stages and more, a pair whose second CTA has no rows
-@pytest.mark.parametrize("rows,H,V,K", [(129, 64, 257, 4), (256, 512, 39000, 8), (257, 192, 9000, 8),
-                                        (400, 1024, 40000, 16)])
+# a tile a pair and several, whole steps of H and a last one of half, a pair whose second CTA has no rows
+@pytest.mark.parametrize("rows,H,V,K", [(129, 2048, 257, 4), (256, 2112, 39000, 8),
+                                        (257, 2048, 9000, 8), (400, 4096, 40000, 16)])
 @pytest.mark.parametrize("second_only", [False, True])
 def test_lm_head_pair_times_out(rows, H, V, K, second_only):
     ll = _ll()
@@ -78,9 +78,9 @@ def test_lm_head_pair_times_out(rows, H, V, K, second_only):
 
 def test_lm_head_hook_rejects_other_kernels_and_limits():
     ll = _ll()
-    h = torch.zeros((384, 64), device="cuda", dtype=torch.bfloat16)
-    w = torch.zeros((39000, 64), device="cuda", dtype=torch.bfloat16)
+    h = torch.zeros((384, 2048), device="cuda", dtype=torch.bfloat16)
+    w = torch.zeros((39000, 2048), device="cuda", dtype=torch.bfloat16)
     ws = ll.Workspace(1 << 24)
-    for rows, limit in ((16, LIMIT), (100, LIMIT), (256, 10), (256, 10 ** 12)):
+    for rows, limit in ((16, LIMIT), (100, LIMIT), (384, LIMIT), (256, 10), (256, 10 ** 12)):
         with pytest.raises(ll.LilicorrError):
             ll.test_lm_head_timeout(h[:rows], w, 4, ws, limit)
