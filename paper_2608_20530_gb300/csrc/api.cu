@@ -204,12 +204,12 @@ GemmArgs gemm(const void* A, lilicorr_dtype_t a_dt, int lda, const void* W, lili
 // The kernel that a product of the network takes.
 enum class GemmPath { SKINNY, ROWS, SMALL, SPLIT, TC, SIMT, SIMT_SPLIT };
 
-// bf16 operands: tensor cores (one tile of rows and short Kd: whole-K copies; few output
-// tiles: Kd split over a cluster; else the persistent kernel), but for the fewest rows, where
-// the split-N CUDA-core kernel spreads the weights over many CTAs. fp32 operands stay on
-// the CUDA cores (the fp32 head keeps fp32 arithmetic throughout).
+// bf16 operands: tensor cores (few output tiles and Kd long enough: Kd split over a cluster, by
+// gemm_split_takes; one tile of rows and short Kd: whole-K copies; else the persistent kernel),
+// but for few rows, where the split-N CUDA-core kernel spreads the weights over many CTAs.
+// fp32 operands stay on the CUDA cores (the fp32 head keeps fp32 arithmetic throughout).
 GemmPath gemm_path(const GemmArgs& g) {
-  const bool fold = g.c2 || g.ss_in;          // only these two kernels fold an RMSNorm
+  const bool fold = g.c2 || g.ss_in;          // these two kernels fold an RMSNorm
   if (fold) return gemm_split_takes(g) ? GemmPath::SPLIT : GemmPath::TC;
   // fp32 throughout and Kd long enough to split (us, 16 x 32 blocks / the kernel taken):
   // one wave of the split-N kernel's CTAs (32 x 256 x 1024: 16.9 / 4.3), or two at long Kd
@@ -410,8 +410,9 @@ struct Prologue {
   }
 };
 
-// Whether every product around the chain's RMSNorms takes the persistent tensor-core
-// kernel (the only one that folds a norm): bf16 heads with more node rows than one tile.
+// Whether every product around the chain's RMSNorms runs on the persistent or the split tensor-core
+// kernel (the two that fold a norm), with no faster kernel for it unfolded: bf16 heads of width 512 and
+// more at any number of nodes, of 320 above 64 node rows, narrower ones above 128.
 bool fold_norms(const HeadCall& c) {
   const lilicorr_head* h = c.h;
   const int D = c.D, F = c.F, N = c.N;

@@ -10,6 +10,8 @@
 // epilogue warps drain it with tcgen05.ld, add bias / per-sequence bias / SiLU / the
 // residual, stage 128-byte-swizzled chunks in the A buffer (free once the products are
 // done) and store them with TMA. Every mbarrier wait is bounded (about 2 s).
+// The network takes it where Kd is too short to split over a cluster (gemm_split_takes has both
+// sides' times): the products of narrow heads, and bf16 outputs at Kd = 512.
 #include "tc_ptx.cuh"
 
 namespace lilicorr {

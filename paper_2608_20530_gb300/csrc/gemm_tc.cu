@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                               ? ep.bias_rows + (size_t)(m / ep.rows_per_bias) * N : nullptr;
       float rs = 1.f;                             // folded RMSNorm of the input rows
       if (FOLD && ep.ss_in) {
-        float sum = 0.f;                          // slots past ss_slots hold zeros
+        float sum = 0.f;                          // load_ss left zeros past ss_slots
 #pragma unroll
         for (int i = 0; i < SS_LD / 4; ++i) sum += (ssn[i].x + ssn[i].y) + (ssn[i].z + ssn[i].w);
         rs = rsqrtf(sum * ep.ss_scale + TC_RMS_EPS);

@@ -232,6 +232,8 @@ lilicorr_status_t gemm_dispatch_c(const GemmArgs& g, dim3 grid, cudaStream_t st)
     return launch_k(gemm_simt_kernel<TA, TW, float, VEC, false>, grid, G_THREADS, 0, st, g, 1);
   return launch_k(gemm_simt_kernel<TA, TW, __nv_bfloat16, VEC, false>, grid, G_THREADS, 0, st, g, 1);
 }
+// (bf16 weights: through the testing header's path 7 only; the network gives fp32 activations and bf16
+// weights to the 16 x 32 blocks, which are as fast there)
 template <typename TW>
 lilicorr_status_t gemm_split_dispatch_c(const GemmArgs& g, dim3 grid, int ways, cudaStream_t st) {
   grid.x *= ways;
@@ -261,7 +263,7 @@ lilicorr_status_t gemm_dispatch_w(const GemmArgs& g, dim3 grid, cudaStream_t st)
 }
 
 // ----------------------------------------------------------------------------- skinny linear
-// Few rows (M <= 64: one row per slot or per sequence) against long rows (Kd up to H).
+// Few rows (one per slot or per sequence) against long rows (Kd up to H).
 // CTA (column block of SK_NB, row block of SK_MB): its 256 threads split Kd in
 // 8-element vectors, each accumulating SK_MB x SK_NB partial dot products, reduced by
 // warp shuffles and shared memory. Many CTAs stream disjoint weight rows.

@@ -18,7 +18,8 @@ namespace walk {
 // best[row] = the best candidate of a row of scores, ties to the lower index; a NaN never wins
 // over an earlier candidate, so the result is always a candidate. Row 0 is the anchor's (A [K]),
 // row 1 + s*K + k that of predecessor k at slot pair s (P [(L-1)][K][K]); A and P in any memory,
-// best [1 + (L-1)*K] in shared memory. Called by `threads` threads numbered `tid`; they sync.
+// best [1 + (L-1)*K] in shared memory. Called by `threads` threads numbered `tid`, which
+// meet at a barrier of the caller's before the table is read.
 __device__ __forceinline__ void best_of_rows(const float* A, const float* P, int L, int K,
                                              uint8_t* best, int tid, int threads) {
   for (int row = tid; row < 1 + (L - 1) * K; row += threads) {
