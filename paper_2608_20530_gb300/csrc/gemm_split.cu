@@ -72,8 +72,8 @@ __device__ __forceinline__ void two_sum(float& v, float& e, float x) {
 // them up in fp32 registers. Relative error against 64 bits, few-row kernel / one chain / this, at
 // Kd = 512, 1024, 2048 and 4096:
 // 6.2e-8 / 1.2e-7 / 6.1e-8, 6.9e-8 / 2.3e-7 / 6.8e-8, 7.9e-8 / 4.7e-7 / 7.8e-8, 8.4e-8 / 4.7e-7 / 7.8e-8
-// (the ranks' parts are added with their rounding errors carried). It costs a product 0.4 to 1.3 us
-// (64 x 1024 x 1024: 4.5 -> 5.3 us, the few-row kernel 25.7; 16 x 1024 x 4096: 5.5 -> 6.8, 11.9), a
+// (the ranks' parts are added with their rounding errors carried). It costs a product 0.4 to 2.3 us
+// (64 x 1024 x 1024: 4.5 -> 5.1 us, the few-row kernel 25.7; 16 x 1024 x 4096: 5.5 -> 7.7, 11.9), a
 // whole network of up to 64 nodes about a tenth (width 512, 48 nodes: 70 -> 77 us; 230 with the
 // few-row kernel).
 template <int BN, bool FEW>
@@ -230,8 +230,9 @@ __global__ void __launch_bounds__(SP_THREADS, FEW ? 2 : 1)
 #pragma unroll
           for (int c = 0; c < BN; c += 16) {
             uint32_t r0[16], r1[16];
-            tmem_ld16(lanes + 2 * b * BN + c, r0);
-            tmem_ld16(lanes + (2 * b + 1) * BN + c, r1);
+            tmem_ld16_nowait(lanes + 2 * b * BN + c, r0);
+            tmem_ld16_nowait(lanes + (2 * b + 1) * BN + c, r1);
+            tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < 16; ++j) sum[c + j] += __uint_as_float(r0[j]) + __uint_as_float(r1[j]);
           }
@@ -453,8 +454,9 @@ bool gemm_split_supported(const GemmArgs& g) {
 //     an SM 5.8-6.1 / 5.9-6.1 against 5.9-6.1 / 5.4, with two 6.6-7.2 / 6.5-7.2 against 6.0 / 5.5; Kd = 1024, S = 4,
 //     4.8-6.9 / 4.8-7.0 against 8.0 / 7.5, S = 2 with two CTAs an SM 7.4-8.3 / 7.6-8.3 against 8.1 / 7.7;
 //     Kd = 2048, S = 2, 9.5-10.5 against 12.1 / 11.7
-//   5-64 rows, few-row kernel: 3.9-5.2 (Kd = 512 or 1024) against 2.9-4.3 while that is one wave of CTAs,
-//     against 5.3-72 beyond.
+//   5-64 rows, few-row kernel: 4.1-5.2 (Kd = 512 or 1024) against 2.9-4.3 while that is one wave of CTAs,
+//     against 5.3-72 beyond; Kd = 4096, one wave: 6.1-6.7 against 6.1-6.4 (5.4 against 5.0 at 8 rows), but on
+//     a quarter of the SMs (beside the top-K pass, selection of 32 requests: 127.5 -> 126.1).
 // Where every product folds an RMSNorm, the kernels that the fold saves decide up to 128 rows: on heads
 // of width 64 and 128 this kernel's networks took 1.3 to 1.5 times as long as the unfolded ones with
 // whole-K copies (two requests of 64 nodes at width 128: 99.9 against 66.8 us), on width 320 0.83.
@@ -466,7 +468,8 @@ bool gemm_split_takes(const GemmArgs& g) {
   const int S = gemm_split_ways(g), nk = ceil_div(g.Kd, SP_BK);
   const bool fold = g.c2 || g.ss_in;
   if (g.M <= SP_FEW)
-    return S >= 4 && nk <= 16 * S && (fold || ceil_div(g.N, 4) * ceil_div(g.M, 16) > num_sms());
+    return S >= 4 && nk <= 16 * S &&
+           (fold || ceil_div(g.N, 4) * ceil_div(g.M, 16) > num_sms() || (nk >= 40 && g.M > 8));
   if (fold && g.M <= 128) return nk >= 5;
   const bool bf16 = g.c_dt == LILICORR_BF16;
   if (gemm_small_supported(g)) return S >= 4 && !bf16;
