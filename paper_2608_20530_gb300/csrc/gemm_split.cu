@@ -17,7 +17,7 @@
 // the products and the reduction are left on the chain. What bounds it is that latency, not a
 // pipe: with these products, the RMSNorms folded into them and the target chain beside the
 // body, the network of width 1024 went from 170 to 115 us for one request and from 352 to 309
-// for 24 (its prologue's 15- and 24-row products; 100 and 278 with what followed); serving_b32's
+// for 24 (its prologue's 15- and 24-row products; 103 and 280 with what followed); serving_b32's
 // drafter-state product (512 rows, 16 tiles, Kd = 4096) beside the top-K pass 136.7 -> 131.7 us a
 // call. The same epilogues as the persistent kernel (gemm_tc.cu): bias, per-sequence bias, SiLU,
 // residual, and the RMSNorm folded into the products around it. Every mbarrier wait is bounded;
