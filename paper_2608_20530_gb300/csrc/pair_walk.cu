@@ -228,6 +228,7 @@ __device__ __forceinline__ float sum16(float (&v)[N], int split) {
 // bytes of a row (no bank conflicts) and each loaded piece feeds four products; the 16
 // partial sums meet by shuffles. The row norms
 // come out of the same pass (blocks of the first row / column group).
+template <bool WALK>
 __global__ void __launch_bounds__(PW_THREADS) pair_block_kernel(PairWalkArgs a) {
   pdl_wait();
   extern __shared__ float sm[];
@@ -350,10 +351,11 @@ __global__ void __launch_bounds__(PW_THREADS) pair_block_kernel(PairWalkArgs a) 
       if (active && r < nrows && k2 < K) outp[(size_t)r * K + k2] = v / (s_nx[r] * s_ny[k2]);
     }
   }
-  if (!a.do_walk) return;
+  if (!WALK) return;
   walk_after_pairs(a, sm, &s_last, s_back, s_path);
 }
 
+template <bool WALK>
 __global__ void __launch_bounds__(PW_THREADS) pair_rows_kernel(PairWalkArgs a) {
   pdl_wait();
   extern __shared__ float sm[];
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(PW_THREADS) pair_rows_kernel(PairWalkArgs a) {
       }
     }
   }
-  if (!a.do_walk) return;
+  if (!WALK) return;
   walk_after_pairs(a, sm, &s_last, s_back, s_path);
 }
 
@@ -496,8 +498,11 @@ lilicorr_status_t launch_pair_walk(const PairWalkArgs& in, cudaStream_t st) {
   PairWalkArgs a = in;
   const size_t score_bytes = sizeof(float) * ((size_t)a.K + (size_t)(a.L - 1) * a.K * a.K);
   a.scores_in_smem = score_bytes <= PW_SMEM_MAX;
-  static bool cfg_pair[64] = {false}, cfg_walk[64] = {false};
+  static bool cfg_pair[2][64] = {{false}}, cfg_walk[64] = {false};
   if (a.do_pairs) {
+    // the scores alone by instances without the walk, whose code costs them registers (77 for 60 of
+    // pair_rows_kernel: 500 sequences of 4 slots x 8, d = 130, 18.7 -> 16.2 us, 32 of 4 x 32, d =
+    // 1024, 48.0 -> 47.1)
     if (a.do_walk && !a.counters) return LILICORR_ERR_ARG;
     // both slots' vectors staged, 16-byte pieces: when the rows are 16-byte aligned and the
     // staging stays within 100 KB (two CTAs per SM at least)
@@ -505,19 +510,21 @@ lilicorr_status_t launch_pair_walk(const PairWalkArgs& in, cudaStream_t st) {
     const bool v4 = ((a.d | a.ld_vec) & 3) == 0 && aligned16(a.in) && aligned16(a.out) &&
                     aligned16(a.anchor);
     if (v4 && block_smem <= 100 * 1024) {
-      static bool cfg_block[64] = {false};
+      static bool cfg_block[2][64] = {{false}};
       size_t smem = block_smem;
       if (a.do_walk && a.scores_in_smem && score_bytes > smem) smem = score_bytes;
-      LL_TRY(allow_max_dynamic_smem(pair_block_kernel, cfg_block));
-      LL_TRY(launch_k(pair_block_kernel, dim3(a.B, a.L), PW_THREADS, smem, st, a));
+      auto* kernel = a.do_walk ? pair_block_kernel<true> : pair_block_kernel<false>;
+      LL_TRY(allow_max_dynamic_smem(kernel, cfg_block[a.do_walk]));
+      LL_TRY(launch_k(kernel, dim3(a.B, a.L), PW_THREADS, smem, st, a));
       return LILICORR_OK;
     }
     size_t smem = pair_walk_smem_bytes(a.L, a.K, a.d);
     if (smem > PW_SMEM_MAX) return LILICORR_ERR_SHAPE;
     if (a.do_walk && a.scores_in_smem && score_bytes > smem) smem = score_bytes;
-    LL_TRY(allow_max_dynamic_smem(pair_rows_kernel, cfg_pair));
+    auto* kernel = a.do_walk ? pair_rows_kernel<true> : pair_rows_kernel<false>;
+    LL_TRY(allow_max_dynamic_smem(kernel, cfg_pair[a.do_walk]));
     dim3 grid(a.B, a.L);
-    LL_TRY(launch_k(pair_rows_kernel, grid, PW_THREADS, smem, st, a));
+    LL_TRY(launch_k(kernel, grid, PW_THREADS, smem, st, a));
     return LILICORR_OK;
   }
   LL_TRY(allow_max_dynamic_smem(walk_kernel, cfg_walk));
