@@ -65,26 +65,31 @@ __device__ __forceinline__ void warp_argmax(float& v, int& idx) {
 }
 
 // Exact best path of one sequence (one full warp). back: [L * K] bytes of shared memory;
-// the path goes to path[L] in shared memory.
-__device__ void viterbi_sequence(const float* A, const float* P, int b, int L, int K, float sigma,
-                                 float* score, uint8_t* back, uint8_t* path) {
+// the path goes to path[L] in shared memory. U predecessors' scores in flight: eight (200 sequences
+// of 15 slots x 8, 9.8 -> 8.3 us cold against one at a time), but fewer where most of the last eight
+// would be none (2048 of 64 slots, K = 1, 2, 4: 43, 44, 45 us by eight, 22, 22, 32 by two, two and
+// four; of 32 x 12 41 by eight, 38 by four).
+template <int U>
+__device__ __forceinline__ void viterbi_sequence(const float* A, const float* P, int b, int L, int K,
+                                                 float sigma, float* score, uint8_t* back,
+                                                 uint8_t* path) {
   const int lane = threadIdx.x & 31;
   float best = lane < K ? sigma * A[lane] : -INFINITY;
   for (int s = 1; s < L; ++s) {
     const float* Ps = P + (size_t)(s - 1) * K * K;
     float bv = -INFINITY;
     int bk = 0;
-    for (int k0 = 0; k0 < K; k0 += 8) {           // eight predecessors' scores in flight:
-      // 200 x 15 slots x 8, 9.8 -> 8.3 us cold against one at a time
-      float c[8];
+#pragma unroll(U < 8 ? 1 : 4)
+    for (int k0 = 0; k0 < K; k0 += U) {
+      float c[U];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
+      for (int u = 0; u < U; ++u) {
         const int k = k0 + u;
         const float pk = __shfl_sync(0xffffffffu, best, k & 31);
         c[u] = pk + sigma * (lane < K && k < K ? Ps[k * K + lane] : 0.f);
       }
 #pragma unroll
-      for (int u = 0; u < 8; ++u)                 // strict: the lower predecessor on ties
+      for (int u = 0; u < U; ++u)                 // strict: the lower predecessor on ties
         if (k0 + u < K && c[u] > bv) { bv = c[u]; bk = k0 + u; }
     }
     if (lane < K) back[s * K + lane] = (uint8_t)bk;
@@ -107,19 +112,24 @@ __device__ void viterbi_sequence(const float* A, const float* P, int b, int L, i
   }
 }
 
+// as the arguments say (greedy, or the best path), the best path two or four predecessors at a time
+enum { WALK_ANY, WALK_BEST_2, WALK_BEST_4 };
+
 // Walk the scores A, P of sequence b (the whole CTA calls): the path, then choices, tokens and
 // margins of all slots at once. back: [L * K] bytes (the Viterbi predecessors, or each score
 // row's best candidate), path: [L] bytes, both in shared memory.
+template <int MODE>
 __device__ __forceinline__ void run_walk(const PairWalkArgs& a, const float* A, const float* P,
                                          int b, uint8_t* back, uint8_t* path) {
-  const bool greedy = a.walk_mode != LILICORR_WALK_VITERBI;
+  const bool greedy = MODE == WALK_ANY && a.walk_mode != LILICORR_WALK_VITERBI;
   if (greedy) {
     best_of_rows(A, P, a.L, a.K, back, threadIdx.x, PW_THREADS);
     __syncthreads();
   }
   if ((threadIdx.x >> 5) != 0) return;
   if (greedy) follow(back, a.L, a.K, path);
-  else viterbi_sequence(A, P, b, a.L, a.K, a.sigma, a.path_score, back, path);
+  else viterbi_sequence<MODE == WALK_BEST_2 ? 2 : MODE == WALK_BEST_4 ? 4 : 8>(
+      A, P, b, a.L, a.K, a.sigma, a.path_score, back, path);
   __syncwarp();
   const int lane = threadIdx.x & 31, K = a.K;
   for (int s = lane; s < a.L; s += 32) {
@@ -159,7 +169,7 @@ __device__ __forceinline__ void walk_after_pairs(const PairWalkArgs& a, float* s
     A = sm;
     P = sm + K;
   }
-  run_walk(a, A, P, b, s_back, s_path);
+  run_walk<WALK_ANY>(a, A, P, b, s_back, s_path);
   if (threadIdx.x == 0) a.counters[b] = 0u;     // leave the workspace reusable
 }
 
@@ -467,6 +477,7 @@ __global__ void __launch_bounds__(PW_THREADS) pair_rows_kernel(PairWalkArgs a) {
   walk_after_pairs(a, sm, &s_last, s_back, s_path);
 }
 
+template <int MODE>
 __global__ void __launch_bounds__(PW_THREADS) walk_kernel(PairWalkArgs a) {
   pdl_wait();
   extern __shared__ float sm[];
@@ -482,7 +493,7 @@ __global__ void __launch_bounds__(PW_THREADS) walk_kernel(PairWalkArgs a) {
     A = sm;
     P = sm + K;
   }
-  run_walk(a, A, P, b, s_back, s_path);
+  run_walk<MODE>(a, A, P, b, s_back, s_path);
 }
 
 }  // namespace
@@ -498,7 +509,7 @@ lilicorr_status_t launch_pair_walk(const PairWalkArgs& in, cudaStream_t st) {
   PairWalkArgs a = in;
   const size_t score_bytes = sizeof(float) * ((size_t)a.K + (size_t)(a.L - 1) * a.K * a.K);
   a.scores_in_smem = score_bytes <= PW_SMEM_MAX;
-  static bool cfg_pair[2][64] = {{false}}, cfg_walk[64] = {false};
+  static bool cfg_pair[2][64] = {{false}}, cfg_walk[3][64] = {{false}};
   if (a.do_pairs) {
     // the scores alone by instances without the walk, whose code costs them registers (77 for 60 of
     // pair_rows_kernel: 500 sequences of 4 slots x 8, d = 130, 18.7 -> 16.2 us, 32 of 4 x 32, d =
@@ -527,8 +538,12 @@ lilicorr_status_t launch_pair_walk(const PairWalkArgs& in, cudaStream_t st) {
     LL_TRY(launch_k(kernel, grid, PW_THREADS, smem, st, a));
     return LILICORR_OK;
   }
-  LL_TRY(allow_max_dynamic_smem(walk_kernel, cfg_walk));
-  LL_TRY(launch_k(walk_kernel, a.B, PW_THREADS, a.scores_in_smem ? score_bytes : 0, st, a));
+  const int mode = a.walk_mode != LILICORR_WALK_VITERBI ? WALK_ANY
+                   : a.K <= 2 ? WALK_BEST_2 : (a.K - 1) % 8 < 4 ? WALK_BEST_4 : WALK_ANY;
+  auto* kernel = mode == WALK_BEST_4 ? walk_kernel<WALK_BEST_4>
+                 : mode == WALK_BEST_2 ? walk_kernel<WALK_BEST_2> : walk_kernel<WALK_ANY>;
+  LL_TRY(allow_max_dynamic_smem(kernel, cfg_walk[mode]));
+  LL_TRY(launch_k(kernel, a.B, PW_THREADS, a.scores_in_smem ? score_bytes : 0, st, a));
   return LILICORR_OK;
 }
 
