@@ -112,8 +112,9 @@ __device__ __forceinline__ void viterbi_sequence(const float* A, const float* P,
   }
 }
 
-// as the arguments say (greedy, or the best path), the best path two or four predecessors at a time
-enum { WALK_ANY, WALK_BEST_2, WALK_BEST_4 };
+// as the arguments say (greedy along the table, or the best path), greedy along the table, greedy
+// step by step, the best path two or four predecessors at a time
+enum { WALK_ANY, WALK_TABLE, WALK_STEPS, WALK_BEST_2, WALK_BEST_4 };
 
 // Walk the scores A, P of sequence b (the whole CTA calls): the path, then choices, tokens and
 // margins of all slots at once. back: [L * K] bytes (the Viterbi predecessors, or each score
@@ -121,13 +122,14 @@ enum { WALK_ANY, WALK_BEST_2, WALK_BEST_4 };
 template <int MODE>
 __device__ __forceinline__ void run_walk(const PairWalkArgs& a, const float* A, const float* P,
                                          int b, uint8_t* back, uint8_t* path) {
-  const bool greedy = MODE == WALK_ANY && a.walk_mode != LILICORR_WALK_VITERBI;
-  if (greedy) {
+  const bool greedy = MODE == WALK_ANY ? a.walk_mode != LILICORR_WALK_VITERBI : MODE <= WALK_STEPS;
+  if (MODE != WALK_STEPS && greedy) {
     best_of_rows(A, P, a.L, a.K, back, threadIdx.x, PW_THREADS);
     __syncthreads();
   }
   if ((threadIdx.x >> 5) != 0) return;
-  if (greedy) follow(back, a.L, a.K, path);
+  if (MODE == WALK_STEPS) walk_steps(A, P, a.L, a.K, path);
+  else if (greedy) follow(back, a.L, a.K, path);
   else viterbi_sequence<MODE == WALK_BEST_2 ? 2 : MODE == WALK_BEST_4 ? 4 : 8>(
       A, P, b, a.L, a.K, a.sigma, a.path_score, back, path);
   __syncwarp();
@@ -509,7 +511,7 @@ lilicorr_status_t launch_pair_walk(const PairWalkArgs& in, cudaStream_t st) {
   PairWalkArgs a = in;
   const size_t score_bytes = sizeof(float) * ((size_t)a.K + (size_t)(a.L - 1) * a.K * a.K);
   a.scores_in_smem = score_bytes <= PW_SMEM_MAX;
-  static bool cfg_pair[2][64] = {{false}}, cfg_walk[3][64] = {{false}};
+  static bool cfg_pair[2][64] = {{false}}, cfg_walk[5][64] = {{false}};
   if (a.do_pairs) {
     // the scores alone by instances without the walk, whose code costs them registers (77 for 60 of
     // pair_rows_kernel: 500 sequences of 4 slots x 8, d = 130, 18.7 -> 16.2 us, 32 of 4 x 32, d =
@@ -538,9 +540,18 @@ lilicorr_status_t launch_pair_walk(const PairWalkArgs& in, cudaStream_t st) {
     LL_TRY(launch_k(kernel, grid, PW_THREADS, smem, st, a));
     return LILICORR_OK;
   }
-  const int mode = a.walk_mode != LILICORR_WALK_VITERBI ? WALK_ANY
+  // Greedy: step by step where that is a short chain, or where the table's rows are more than the
+  // CTA's threads and share banks (walks alone, us, table / steps: 16,384 of 2 slots x 12 21.6 / 19.1,
+  // of 2 x 8 20.1 / 19.0; 4096 of 3 x 24 11.9 / 9.2, of 8 x 24 23.4 / 19.5, of 8 x 31 26.3 / 33.0;
+  // 2048 of 8 x 32 16.7 / 14.0, of 4 x 20 6.0 / 7.2; one of 8 x 32 4.0 / 4.7). Each walk its own
+  // instance: 32 registers, eight CTAs an SM.
+  const bool steps =
+      a.L <= 2 || (a.K > 8 && a.K % 8 == 0 && 3 * a.L <= a.K && a.B >= 4 * num_sms());
+  const int mode = a.walk_mode != LILICORR_WALK_VITERBI ? steps ? WALK_STEPS : WALK_TABLE
                    : a.K <= 2 ? WALK_BEST_2 : (a.K - 1) % 8 < 4 ? WALK_BEST_4 : WALK_ANY;
-  auto* kernel = mode == WALK_BEST_4 ? walk_kernel<WALK_BEST_4>
+  auto* kernel = mode == WALK_TABLE    ? walk_kernel<WALK_TABLE>
+                 : mode == WALK_STEPS  ? walk_kernel<WALK_STEPS>
+                 : mode == WALK_BEST_4 ? walk_kernel<WALK_BEST_4>
                  : mode == WALK_BEST_2 ? walk_kernel<WALK_BEST_2> : walk_kernel<WALK_ANY>;
   LL_TRY(allow_max_dynamic_smem(kernel, cfg_walk[mode]));
   LL_TRY(launch_k(kernel, a.B, PW_THREADS, a.scores_in_smem ? score_bytes : 0, st, a));

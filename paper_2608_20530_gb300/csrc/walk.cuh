@@ -19,19 +19,59 @@ namespace walk {
 // over an earlier candidate, so the result is always a candidate. Row 0 is the anchor's (A [K]),
 // row 1 + s*K + k that of predecessor k at slot pair s (P [(L-1)][K][K]); A and P in any memory,
 // best [1 + (L-1)*K] in shared memory. Called by `threads` threads numbered `tid`, which
-// meet at a barrier of the caller's before the table is read.
+// meet at a barrier of the caller's before the table is read. Rows of 16 or 32 scores in shared
+// memory share banks 16 or 32 at a time, so there the threads of a warp start at different
+// candidates (walks of 2048 sequences of 8 slots x 32: 58 us from candidate 0 in every row, 17 so;
+// of 8 x 8, where they share eight at a time, 6.0 from candidate 0 and 7.9 so).
 __device__ __forceinline__ void best_of_rows(const float* A, const float* P, int L, int K,
                                              uint8_t* best, int tid, int threads) {
+  const bool turned = (K & 15) == 0;
   for (int row = tid; row < 1 + (L - 1) * K; row += threads) {
     const float* r = row == 0 ? A : P + (size_t)(row - 1) * K;
     float v = r[0];
     int c = 0;
+    if (turned && v == v) {                      // (a NaN in front stays the choice)
+      const int k0 = row * K / 32;
+      v = -INFINITY;
+      c = K;
 #pragma unroll 4
-    for (int k = 1; k < K; ++k) {
-      const float x = r[k];
-      if (x > v) { v = x; c = k; }
+      for (int j = 0; j < K; ++j) {
+        const int k = (k0 + j) & (K - 1);
+        const float x = r[k];
+        if (x > v || (x == v && k < c)) { v = x; c = k; }
+      }
+    } else {
+#pragma unroll 4
+      for (int k = 1; k < K; ++k) {
+        const float x = r[k];
+        if (x > v) { v = x; c = k; }
+      }
     }
     best[row] = (uint8_t)c;
+  }
+}
+
+// The walk without a table, by one full warp: a butterfly over the candidates' lanes per step, the
+// same choices. Bounded by the chain of L steps, where the table is by its 1 + (L-1)*K rows.
+__device__ __forceinline__ void walk_steps(const float* A, const float* P, int L, int K,
+                                           uint8_t* path) {
+  const int lane = threadIdx.x & 31;
+  int width = 1;                                 // lanes that hold candidates, rounded up
+  while (width < K) width <<= 1;
+  int c = 0;
+  for (int s = 0; s < L; ++s) {
+    const float* r = s == 0 ? A : P + ((size_t)(s - 1) * K + c) * K;
+    float v = lane < K ? r[lane] : -INFINITY;
+    const bool front_nan = __shfl_sync(0xffffffffu, v != v, 0);
+    c = v == v && lane < K ? lane : 32;          // a NaN never wins
+    if (v != v) v = -INFINITY;
+    for (int o = width >> 1; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+      const int oc = __shfl_xor_sync(0xffffffffu, c, o);
+      if (ov > v || (ov == v && oc < c)) { v = ov; c = oc; }
+    }
+    c = front_nan ? 0 : __shfl_sync(0xffffffffu, c, 0);    // but in front it stays the choice
+    if (lane == 0) path[s] = (uint8_t)c;
   }
 }
 
