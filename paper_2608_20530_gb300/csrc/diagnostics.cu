@@ -8,11 +8,11 @@
 // local_softmax_kernel: a power-of-two group of lanes per score row (the anchor row of a
 //   sequence, or the row of one predecessor at one slot pair); lane k holds sigma * score[k],
 //   group max and sum.
-// path_probs_kernel: a CTA per sequence, a warp per step: the path is given, so every step
-//   knows its predecessor; the same softmax over the row of the predecessor, the chosen
-//   candidate's probability and its gap to the best other candidate; the logarithms are summed
-//   in step order at the end. 200 sequences of 15 steps: 19 us (a warp walking the steps) -> 5.9
-//   us cold.
+// path_probs_kernel: a CTA per sequence, a warp per step: the path is given, so every step knows
+//   its predecessor; the same softmax over the row of the predecessor, the chosen candidate's
+//   probability and its gap to the best other candidate; the logarithms are summed in step order
+//   at the end. 200 sequences of 15 steps: 19 us (a warp walking the steps) -> 5.9 us cold. Many
+//   sequences of few steps are a warp's each.
 // acceptance_kernel: a warp per sequence, a lane per slot; runs end at the first zero of a
 //   ballot. 14 us (a thread per sequence) -> 3.9 us cold.
 #include "internal.cuh"
@@ -56,16 +56,23 @@ local_softmax_kernel(int B, int L, int K, const float* __restrict__ A, const flo
   if (live && lane < K) (r == 0 ? pa + (size_t)b * K : pp + o)[lane] = p;
 }
 
+// W (1 or 8) warps per sequence
+template <int W>
 __global__ void __launch_bounds__(DG_THREADS)
-path_probs_kernel(int B, int L, int K, const float* __restrict__ A, const float* __restrict__ P,
-                  const int32_t* __restrict__ choice, float sigma, float* __restrict__ prob,
-                  float* __restrict__ gap, float* __restrict__ log_prob) {
+path_probs_kernel(int B, int L, int K, const float* __restrict__ A,
+                  const float* __restrict__ P, const int32_t* __restrict__ choice, float sigma,
+                  float* __restrict__ prob, float* __restrict__ gap, float* __restrict__ log_prob) {
   pdl_wait();
-  __shared__ float s_log[LILICORR_MAX_L];
-  const int b = blockIdx.x, lane = threadIdx.x & 31;
-  for (int s = threadIdx.x >> 5; s < L; s += DG_THREADS / 32) {
+  static_assert(W == 1 || W == DG_THREADS / 32, "a warp or a CTA per sequence");
+  __shared__ float s_log[LILICORR_MAX_L];          // (W = 1 sums as it goes)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = W == 1 ? blockIdx.x * (DG_THREADS / 32) + warp : blockIdx.x;
+  if (b >= B) return;
+  float lp = 0.f;
+  int prev = 0;
+  for (int s = W == 1 ? 0 : warp; s < L; s += W) {
     const int c = choice[(size_t)b * L + s];
-    const int prev = s > 0 ? choice[(size_t)b * L + s - 1] : 0;
+    if (W > 1) prev = s > 0 ? choice[(size_t)b * L + s - 1] : 0;
     const bool valid = c >= 0 && c < K && prev >= 0 && prev < K;
     const float* row = s == 0 ? A + (size_t)b * K
                               : P + (((size_t)b * (L - 1) + (s - 1)) * K + (valid ? prev : 0)) * K;
@@ -80,16 +87,18 @@ path_probs_kernel(int B, int L, int K, const float* __restrict__ A, const float*
       const float ps = valid ? pc : NAN;               // a choice outside [0, K) has no probability
       if (prob) prob[o] = ps;
       if (gap) gap[o] = valid ? (K > 1 ? zc - other : INFINITY) : NAN;
-      s_log[s] = logf(ps);
+      if (W == 1) lp += logf(ps);
+      else s_log[s] = logf(ps);
     }
+    prev = c;
   }
   if (!log_prob) return;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float lp = 0.f;
-    for (int s = 0; s < L; ++s) lp += s_log[s];
-    log_prob[b] = lp;
+  if (W > 1) {
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int s = 0; s < L; ++s) lp += s_log[s];
   }
+  if (W == 1 ? lane == 0 : threadIdx.x == 0) log_prob[b] = lp;
 }
 
 // length of the run of ones that starts at bit 0 of a warp's lanes
@@ -165,9 +174,13 @@ extern "C" lilicorr_status_t lilicorr_path_probs(int B, int L, int K, const floa
   if (!(sigma > 0.f) || !isfinite(sigma)) return LILICORR_ERR_ARG;
   if (B == 0) return LILICORR_OK;
   if (!anchor_scores || (L > 1 && !pair_scores) || !choice) return LILICORR_ERR_ARG;
-  LL_TRY(launch_k(path_probs_kernel, B, DG_THREADS, 0, stream, B, L, K,
-                  anchor_scores, pair_scores, choice, sigma, prob, gap, log_prob));
-  return LILICORR_OK;
+  // a CTA per sequence, or a warp each where sequences are many for their steps (K = 8, us, CTA /
+  // warp: 2048 of 1 slot 4.3 / 2.6, of 4 4.3 / 4.6, of 16 9.2 / 13.9; 4096 of 4 7.2 / 5.4, of 8
+  // 9.4 / 8.9; 16,384 of 1 20.8 / 5.1, of 16 55 / 49, of 64 192 / 183)
+  const bool warps = L == 1 || (B >= 8 * num_sms() && B >= 3LL * num_sms() * L);
+  return launch_k(warps ? path_probs_kernel<1> : path_probs_kernel<DG_THREADS / 32>,
+                  warps ? ceil_div(B, DG_THREADS / 32) : B, DG_THREADS, 0, stream, B, L, K,
+                  anchor_scores, pair_scores, choice, sigma, prob, gap, log_prob);
 }
 
 extern "C" lilicorr_status_t lilicorr_block_acceptance(int B, int L, int K, const int32_t* ids,
