@@ -13,8 +13,8 @@
 //   probability and its gap to the best other candidate; the logarithms are summed in step order
 //   at the end. 200 sequences of 15 steps: 19 us (a warp walking the steps) -> 5.9 us cold. Many
 //   sequences of few steps are a warp's each.
-// acceptance_kernel: a warp per sequence, a lane per slot; runs end at the first zero of a
-//   ballot. 14 us (a thread per sequence) -> 3.9 us cold.
+// acceptance_kernel: a warp per sequence (four lanes where many are short), a lane per slot; runs
+//   end at the first zero of the group's ballot. 14 us (a thread per sequence) -> 3.9 us cold.
 #include "internal.cuh"
 
 namespace lilicorr {
@@ -101,26 +101,28 @@ path_probs_kernel(int B, int L, int K, const float* __restrict__ A,
   if (W == 1 ? lane == 0 : threadIdx.x == 0) log_prob[b] = lp;
 }
 
-// length of the run of ones that starts at bit 0 of a warp's lanes
+// length of the run of ones that starts at the first lane of this lane's group of G
+template <int G>
 __device__ __forceinline__ int run_length(bool one) {
-  const uint32_t zeros = ~__ballot_sync(0xffffffffu, one);
-  return zeros ? __ffs(zeros) - 1 : 32;
+  const uint32_t zeros = ~__ballot_sync(0xffffffffu, one) >> (threadIdx.x & 31 & ~(G - 1));
+  return min(zeros ? __ffs(zeros) - 1 : 32, G);
 }
 
+// G (4 or 32) lanes per sequence, which take its slots G at a time
+template <int G>
 __global__ void __launch_bounds__(DG_THREADS)
 acceptance_kernel(int B, int L, int K, const int32_t* __restrict__ ids,
                   const int32_t* __restrict__ tokens, const int32_t* __restrict__ truth,
                   int32_t* __restrict__ covered, int32_t* __restrict__ oracle_prefix,
                   int32_t* __restrict__ accepted) {
   pdl_wait();
-  const int b = blockIdx.x * (DG_THREADS / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (b >= B) return;
+  const int b = blockIdx.x * (DG_THREADS / G) + threadIdx.x / G;
+  const int lane = threadIdx.x & (G - 1);
   int prefix = 0, acc = 0;
-  for (int s0 = 0; s0 < L; s0 += 32) {
+  for (int s0 = 0; s0 < L; s0 += G) {              // (the same rounds in every lane of a warp)
     const int s = s0 + lane;
     bool cov = false, same = false;
-    if (s < L) {
+    if (b < B && s < L) {
       const size_t o = (size_t)b * L + s;
       const int32_t g = truth[o];
 #pragma unroll 8
@@ -128,11 +130,12 @@ acceptance_kernel(int B, int L, int K, const int32_t* __restrict__ ids,
       same = tokens[o] == g;
       if (covered) covered[o] = cov ? 1 : 0;
     }
-    // a run goes on into the next 32 slots only if it filled the ones before
-    if (prefix == s0) prefix += run_length(cov);
-    if (acc == s0) acc += run_length(same);
+    // a run goes on into the next slots only if it filled the ones before
+    const int more = run_length<G>(cov), more_acc = run_length<G>(same);
+    if (prefix == s0) prefix += more;
+    if (acc == s0) acc += more_acc;
   }
-  if (lane != 0) return;
+  if (lane != 0 || b >= B) return;
   if (oracle_prefix) oracle_prefix[b] = prefix;
   if (accepted) accepted[b] = acc;
 }
@@ -190,7 +193,11 @@ extern "C" lilicorr_status_t lilicorr_block_acceptance(int B, int L, int K, cons
   if (!shape_ok(B, L, K)) return LILICORR_ERR_SHAPE;
   if (B == 0) return LILICORR_OK;
   if (!ids || !tokens || !truth) return LILICORR_ERR_ARG;
-  LL_TRY(launch_k(acceptance_kernel, ceil_div(B, DG_THREADS / 32), DG_THREADS, 0, stream, B, L, K, ids,
-                  tokens, truth, covered, oracle_prefix, accepted));
-  return LILICORR_OK;
+  // a warp per sequence, but four lanes where many short ones would leave most of its lanes idle
+  // (us, warp / four lanes: 16,384 of one slot x 4 3.8 / 2.0, of 8 x 8 4.1 / 3.0, of 16 x 2 3.7 /
+  // 3.4; 4096 of 8 x 32 5.8 / 9.7)
+  const bool few = L <= 8 && B >= 32 * num_sms();
+  return launch_k(few ? acceptance_kernel<4> : acceptance_kernel<32>,
+                  ceil_div((long long)B * (few ? 4 : 32), DG_THREADS), DG_THREADS, 0, stream, B, L, K,
+                  ids, tokens, truth, covered, oracle_prefix, accepted);
 }

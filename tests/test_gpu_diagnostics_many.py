@@ -1,5 +1,5 @@
 """GPU checks of the diagnostics of many sequences: paths by a warp each beside paths by a CTA each
-(numbers that leave a last CTA part empty)."""
+(numbers that leave a last CTA part empty), and runs by four lanes each beside runs by a warp."""
 import pytest
 import torch
 
@@ -32,3 +32,19 @@ def test_paths(B, L, K):
     want = (zc - lse).sum(1)[:-1]
     # relative error of a probability 1e-6, so of a sum of L logarithms L times that
     assert ((lp[:-1].double() - want).abs() < 2e-6 * L + 1e-6 * want.abs()).all()
+
+
+@pytest.mark.parametrize("B,L,K", [(4869, 1, 4), (4869, 3, 1), (4869, 4, 32), (4869, 5, 2),
+                                   (4869, 8, 3), (4869, 9, 3), (4863, 4, 2)])
+def test_runs(B, L, K):
+    ll = _ll()
+    g = torch.Generator(device="cuda").manual_seed(L)
+    ids = torch.randint(0, 2 * K + 1, (B, L, K), generator=g, device="cuda", dtype=torch.int32)
+    truth = torch.randint(0, 2 * K + 1, (B, L), generator=g, device="cuda", dtype=torch.int32)
+    truth[::5] = ids[::5, :, -1]                   # every fifth covered throughout
+    tokens = torch.where(torch.rand(B, L, generator=g, device="cuda") < 0.8, truth, truth + 1)
+    covered, prefix, accepted = ll.block_acceptance(ids, tokens, truth)
+    cov, same = (ids == truth[..., None]).any(-1), tokens == truth
+    assert torch.equal(covered, cov.int())
+    assert torch.equal(prefix, cov.int().cumprod(1).sum(1).int())
+    assert torch.equal(accepted, same.int().cumprod(1).sum(1).int())
