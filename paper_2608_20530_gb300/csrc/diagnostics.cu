@@ -46,7 +46,10 @@ local_softmax_kernel(int B, int L, int K, const float* __restrict__ A, const flo
   const int rows_per_seq = 1 + (L - 1) * K;
   const long long row = (long long)blockIdx.x * (DG_THREADS / G) + threadIdx.x / G;
   const int lane = threadIdx.x % G;
-  const bool live = row < (long long)B * rows_per_seq;   // every lane takes part in the shuffles
+  // every lane takes part in the shuffles, but a whole warp may leave: the rows of 32 lanes then
+  // need no guards (1024 sequences of 8 slots x 32, 33.6 -> 30.6 us)
+  const bool live = row < (long long)B * rows_per_seq;
+  if (G == 32 && !live) return;
   const int b = live ? (int)(row / rows_per_seq) : 0, r = live ? (int)(row % rows_per_seq) : 0;
   const size_t o = ((size_t)b * (L - 1) * K + (r - 1)) * K;
   const float* src = r == 0 ? A + (size_t)b * K : P + o;
