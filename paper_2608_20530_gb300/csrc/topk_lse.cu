@@ -745,8 +745,10 @@ topk_merge_kernel(const unsigned char* __restrict__ recs, size_t ld_p, size_t ld
   // (152 lists of 8 from a 151,936-wide vocabulary: about ten survivors, against some
   // hundreds above the largest K-th key, whose ranks took most of the merge: the merge of 64
   // such rows 20.7 -> 7.8 us cold.) One key a thread; with more lists than threads the counting
-  // would cost what it saves.
-  if (P >= K && P <= TK_THREADS) {
+  // would cost what it saves, and so it does with few survivors (512 rows, us, without / with: 152
+  // lists of 1, 2, 4: 4.7 / 8.0, 5.5 / 8.3, 11.6 / 8.6; 16 lists of 2, 4, 8: 3.8 / 3.9, 3.9 / 4.0,
+  // 5.0 / 4.2).
+  if (K >= 4 && P * K >= 128 && P >= K && P <= TK_THREADS) {
     const uint64_t c = tid < P ? s_keys[tid * K] : 0ull;
     int rank = 0;
     if (c != 0ull)

@@ -28,3 +28,9 @@ def test_merge_matches_the_whole_row(rows, V, K, P):
         # P fp32 sums added up, each term within an ex2.approx (2^-22)
         assert abs(lse[r].item() - wlse) < 1e-5
         assert np.abs(logp[r].cpu().numpy() - wlogp).max() < 1e-5
+
+
+@pytest.mark.parametrize("rows,V,K,P", [(3, 4000, 4, 31), (3, 4000, 4, 32), (3, 4000, 3, 152),
+                                        (2, 3000, 2, 16), (3, 4000, 8, 15), (3, 4000, 8, 16)])
+def test_merge_around_its_bounds_limits(rows, V, K, P):
+    test_merge_matches_the_whole_row(rows, V, K, P)
