@@ -228,7 +228,7 @@ GemmPath gemm_path(const GemmArgs& g) {
   // otherwise: the split-N kernel
   if (g.a_dt == LILICORR_F32 && g.M > 16 && g.M <= 1024 && gemm_rows_supported(g))
     return GemmPath::ROWS;
-  if (g.M > 4 && gemm_split_takes(g)) return GemmPath::SPLIT;
+  if (gemm_split_takes(g)) return GemmPath::SPLIT;
   if (g.M <= 64 || (g.a_dt == LILICORR_F32 && g.M <= 1024)) return GemmPath::SKINNY;
   if (gemm_small_supported(g)) return GemmPath::SMALL;
   if (gemm_tc_supported(g)) return GemmPath::TC;

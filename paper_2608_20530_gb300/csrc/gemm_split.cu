@@ -425,10 +425,13 @@ int gemm_split_ss_slots(int N) { return ceil_div(N, 64); }
 //   960 x 1024 x 1024   8.7  7.6 12.6 25.1   8.0      1024 x 512 x 512     6.7  5.5  6.0 13.0   5.7
 // So S doubles while the CTAs fit one an SM and keep two chunks of Kd each, or two an SM and keep
 // four; eight ways, whose clusters are harder to place, only where Kd is long.
+// Of few rows one chunk each will do: the shorter a CTA's sum, the closer (64 x 1024 x 256: S = 4 4.0 us
+// and an error of 5.4e-8, S = 1 4.8 and 6.1e-8; the few-row kernel 24.4 and 5.5e-8).
 int gemm_split_ways(const GemmArgs& g) {
   const int tiles = split_tiles(g, 64), nk = ceil_div(g.Kd, SP_BK), sms = num_sms();
+  const int least = g.M <= SP_FEW ? 2 : 4;
   int S = 1;
-  while (S < 4 && ((2 * S * tiles <= sms && nk >= 4 * S) || (S * tiles <= sms && nk >= 8 * S)))
+  while (S < 4 && ((2 * S * tiles <= sms && nk >= least * S) || (S * tiles <= sms && nk >= 8 * S)))
     S *= 2;
   if (S == 4 && 8 * tiles <= sms && nk >= 40) S = 8;
   return S > 1 || 2 * tiles <= sms ? S : 0;
@@ -454,21 +457,23 @@ bool gemm_split_supported(const GemmArgs& g) {
 //     an SM 5.8-6.1 / 5.9-6.1 against 5.9-6.1 / 5.4, with two 6.6-7.2 / 6.5-7.2 against 6.0 / 5.5; Kd = 1024, S = 4,
 //     4.8-6.9 / 4.8-7.0 against 8.0 / 7.5, S = 2 with two CTAs an SM 7.4-8.3 / 7.6-8.3 against 8.1 / 7.7;
 //     Kd = 2048, S = 2, 9.5-10.5 against 12.1 / 11.7
-//   5-64 rows, few-row kernel: 4.1-5.2 (Kd = 512 or 1024) against 2.9-4.3 while that is one wave of CTAs,
-//     against 5.3-72 beyond; Kd = 4096, one wave: 6.1-6.7 against 6.1-6.4 (5.4 against 5.0 at 8 rows), but on
+//   5-64 rows, few-row kernel: 3.6-4.4 (Kd = 256 or 384) and 4.1-5.2 (512 or 1024) against 2.7-4.3 while
+//     that is one wave of CTAs, against 4.9-72 beyond; Kd = 4096, one wave: 6.1-6.7 against 6.1-6.4 (5.4 against 5.0 at 8 rows), but on
 //     a quarter of the SMs (beside the top-K pass, selection of 32 requests: 127.5 -> 126.1).
 // Where every product folds an RMSNorm, the kernels that the fold saves decide up to 128 rows: on heads
 // of width 64 and 128 this kernel's networks took 1.3 to 1.5 times as long as the unfolded ones with
 // whole-K copies (two requests of 64 nodes at width 128: 99.9 against 66.8 us), on width 320 0.83.
 // Up to 64 rows only where its error is no larger than the few-row kernel's: Kd over at
-// least four CTAs (shorter sums are closer there: 2560 columns x Kd 328, two CTAs 6.3e-8 against
-// 5.7e-8), 16 chunks each at most.
+// least four CTAs (2560 columns x Kd 328, two CTAs 6.3e-8 against 5.7e-8), 16 chunks each at most. On
+// networks of width 320 or 384 it takes 64 to 73 us where the few-row kernel takes 77 to 203. Up to
+// four rows the few-row kernel has no second wave, and its unfolded networks are ahead (one sequence
+// of four nodes, width 512: 55.1 against 64.3 us, 1024: 73.1 against 81.7).
 bool gemm_split_takes(const GemmArgs& g) {
   if (!gemm_split_supported(g)) return false;
   const int S = gemm_split_ways(g), nk = ceil_div(g.Kd, SP_BK);
   const bool fold = g.c2 || g.ss_in;
   if (g.M <= SP_FEW)
-    return S >= 4 && nk <= 16 * S &&
+    return g.M > 4 && S >= 4 && nk <= 16 * S &&
            (fold || ceil_div(g.N, 4) * ceil_div(g.M, 16) > num_sms() || (nk >= 40 && g.M > 8));
   if (fold && g.M <= 128) return nk >= 5;
   const bool bf16 = g.c_dt == LILICORR_BF16;

@@ -30,6 +30,13 @@ def test_few_rows_sums(M, N, Kd):
     assert err[0] <= 1.03 * err[1], err
 
 
+# one or two chunks a CTA, the last of them short, up to the most tiles that four CTAs each take
+@pytest.mark.parametrize("M,N,Kd", [(5, 768, 256), (16, 256, 256), (64, 1024, 256), (64, 2432, 256),
+                                    (33, 960, 320), (48, 696, 296), (64, 1152, 384), (17, 1344, 448)])
+def test_few_rows_sums_of_short_rows(M, N, Kd):
+    test_few_rows_sums(M, N, Kd)
+
+
 @pytest.mark.parametrize("M,N,Kd", [(5, 512, 512), (33, 1536, 512), (64, 2048, 1024)])
 @pytest.mark.parametrize("path", [0, 6])
 def test_few_rows_silu(M, N, Kd, path):

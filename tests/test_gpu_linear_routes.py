@@ -52,3 +52,10 @@ def test_narrow_network_matches_oracle(B, L, K, D):
         _oracle_check(wl, W, inp, ids, logp, *res, range(B))
     finally:
         head.close()
+
+
+# up to 64 nodes: few-row products, folded from five nodes on where Kd splits over four CTAs
+@pytest.mark.parametrize("B,L,K,D", [(1, 64, 1, 256), (1, 4, 1, 512), (1, 2, 2, 1024), (1, 5, 1, 512),
+                                     (3, 4, 4, 384), (2, 5, 3, 320), (1, 64, 1, 320)])
+def test_network_of_few_nodes_matches_oracle(B, L, K, D):
+    test_narrow_network_matches_oracle(B, L, K, D)
